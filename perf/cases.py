@@ -226,7 +226,8 @@ def _tensors(case, seed):
     if op == "heatbath":
         return {"U": _links(dims, 0.35, gen)}
     if op == "hmc":
-        return {"U": _links(dims, 0.35, gen), "P": _momenta(dims, gen), "eta": _gaussian(shape, gen)}
+        # as rough as an equilibrium configuration at beta = 5.6 (plaquette about 0.53)
+        return {"U": _links(dims, 0.41, gen), "P": _momenta(dims, gen), "eta": _gaussian(shape, gen)}
     return {"props": _propagator_like(dims, gen)}
 
 
