@@ -5,19 +5,15 @@
 // C_Gamma(t) = sum of C_Gamma(x) over the spatial sites of time slice t.
 //
 // In the chiral basis every Gamma used here, and so A = g5 Gamma and
-// B = Gamma g5, has one non-zero per row and column: A[al][pi(al)] = a_al,
-// B[rho(be)][be] = b_be. Then
-//   C(x) = - sum_{al, a, be, b} conj(S[al a][be b]) a_al b_be S[pi(al) a][rho(be) b],
-// a sum of 144 products per Gamma. The requested Gammas fall into a few classes
-// of equal permutations (pi, rho) (three for the sixteen of the chiral basis: the
-// identity for 1 and g5, and two pairings for g_x, g_y / g_z, g_t and their g5
-// partners), so per class and site the "spin Gram" entries
-//   G[al][be] = sum_{a, b} conj(S[al a][be b]) S[pi(al) a][rho(be) b]
-// are formed once and each Gamma is C(x) = - sum a_al b_be G[al][be]. A CTA stages
-// the 12 solutions of its 32 sites in shared memory; four threads per site (one
-// per source spin be) form G[.][be] for every class. Each CTA covers sites of one
-// time slice and writes one partial per Gamma; a second kernel sums the partials
-// of each slice in a fixed order.
+// B = Gamma g5, has one non-zero per row and column, in the columns al ^ x for one
+// x of {0, 2, 3} (0 for 1 and g5, 3 for g_x, g_y, 2 for g_z, g_t and their g5
+// partners): A[al][al ^ x] = a_al, B[be ^ x][be] = b_be. Then
+//   C(x) = - sum_{al, be} a_al b_be G_x[al][be],
+//   G_x[al][be] = sum_{a, b} conj(S[al a][be b]) S[al^x a][be^x b],
+// and since G_x[al^x][be^x] = conj(G_x[al][be]), the sixteen G_0 are real and eight
+// complex entries (be = 0, 1) hold the others. C is linear in them, so the 48 real
+// numbers are summed over the sites of a time slice first and every Gamma is formed
+// once per slice.
 #include <array>
 #include <complex>
 #include <cstring>
@@ -30,21 +26,23 @@ namespace lqcd {
 
 namespace {
 
-constexpr int CSITES = 32;  // sites per CTA (one warp)
+constexpr int CTHREADS = 128;
 constexpr int MAXG = 16;
+constexpr int NGRAM = 48;  // 16 G_0, then 8 complex G_3, then 8 complex G_2
 
 struct Monomial {  // one non-zero per row: M[r][col[r]] = (re[r], im[r])
   int col[4];
   double re[4], im[4];
 };
-struct GammaTab {
-  Monomial A[MAXG], Bt[MAXG];  // A = g5 Gamma (by rows), B^T = (Gamma g5)^T (by columns of B)
-  int cls[MAXG];               // permutation class of each Gamma
-  int pi[MAXG][4], rho[MAXG][4];  // permutations of each class
-  int nclass;
+struct GammaTab {      // a kernel argument
+  double2 a[MAXG][4];  // A = g5 Gamma by rows
+  double2 b[MAXG][4];  // Gamma g5 by columns
+  int x[MAXG];         // the Gamma's x
+  int use;             // bit x set: some Gamma has this x
 };
-
-__constant__ GammaTab c_gamma;
+struct Props {
+  const double2* half[2][12];  // [parity][source]
+};
 
 using cd = std::complex<double>;
 using M4 = std::array<std::array<cd, 4>, 4>;
@@ -102,102 +100,120 @@ bool monomial_rows(const M4& m, Monomial& out) {
   return true;
 }
 
-constexpr int CTHREADS = 4 * CSITES;  // four threads (source spins) per site
-
-// S[j][src][comp]: comp = device real pair index (colour-major: (a * 4 + al))
-__global__ void __launch_bounds__(CTHREADS) k_meson(const double2* const* props, Geom g, int ngam,
-                                                    int tiles_per_slice, double* partials) {
-  extern __shared__ double2 sm[];  // [CSITES][12 sources][12 components]
-  __shared__ double red[CTHREADS / 32][2 * MAXG];
-  const int S3 = g.L[0] * g.L[1] * g.L[2];
-  const int t = blockIdx.x / tiles_per_slice;
-  const int k = blockIdx.x % tiles_per_slice;
-  // staging: thread i loads components of site i % CSITES
-  for (int i = threadIdx.x; i < CSITES * 12; i += CTHREADS) {
-    const int j = i % CSITES, src = i / CSITES;
-    const int s3 = k * CSITES + j;
-    if (s3 >= S3) continue;
-    const long long s = (long long)t * S3 + s3;
-    const int x = (int)(s % g.L[0]);
-    const long long r = s / g.L[0];
-    const int y = (int)(r % g.L[1]), z = (int)((r / g.L[1]) % g.L[2]);
-    const int par = (x + y + z + t) & 1;
-    const int h = (int)(s >> 1);
-    const double2* base = props[2 * src + par];
-    double2* my = sm + (size_t)j * 144 + src * 12;
+// Sums of the 48 numbers over the sites of one CTA, a contiguous range of one parity's
+// sites of one time slice (in the half-lattice index a slice is one range per parity).
+//
+// Bound by the FP64 pipe: 864 FMAs per site (288 for each x), 0.93 ms at 24^3x48 against
+// 0.23 ms of HBM. For one colour pair (a, b) everything above involves only the 4 x 4
+// spin matrix S[.. a][.. b], so a thread takes whole sites, one colour pair at a time:
+// 16 coalesced 16-byte loads, each used in 6 FMAs, no shared memory, and the 48 sums stay
+// in registers over the thread's sites. (The form before it staged each site's 144 numbers
+// in shared memory at a 2304-byte stride, an eight-way bank conflict, formed all 48 complex
+// Gram entries and combined the Gammas at every site: ten Gammas at 24^3x48 took 5.87 ms a
+// call, this form 1.09 ms.)
+__global__ void __launch_bounds__(CTHREADS, 2) k_meson(const Props p, int Vh, int slice, int nb, int use,
+                                                       double* partials) {
+  __shared__ double sm[16][CTHREADS + 1];
+  const int blk = blockIdx.x % (2 * nb);
+  const int t = blockIdx.x / (2 * nb);
+  const int par = blk / nb, k = blk % nb;
+  const int chunk = (slice + nb - 1) / nb;
+  const int lo = t * slice + k * chunk, hi = min((t + 1) * slice, lo + chunk);
+  double g0[16], g3[16], g2[16];
 #pragma unroll
-    for (int c = 0; c < 12; ++c) my[c] = base[(size_t)c * g.Vh + h];
-  }
-  __syncthreads();
-  const int j = threadIdx.x % CSITES, be = threadIdx.x / CSITES;
-  const bool active = k * CSITES + j < S3;
-  const double2* my = sm + (size_t)j * 144;
-  double acc[2 * MAXG];
+  for (int q = 0; q < 16; ++q) g0[q] = g3[q] = g2[q] = 0.0;
+  for (int h = lo + (int)threadIdx.x; h < hi; h += CTHREADS) {
+    for (int a = 0; a < 3; ++a) {
+#pragma unroll 1
+      for (int b = 0; b < 3; ++b) {
+        double2 s[4][4];  // S[al a][be b]; component a * 4 + al of source 3 be + b
 #pragma unroll
-  for (int q = 0; q < 2 * MAXG; ++q) acc[q] = 0.0;
-  if (active) {
-    for (int cl = 0; cl < c_gamma.nclass; ++cl) {
-      const int rb = c_gamma.rho[cl][be];
-      double gr[4], gi[4];
+        for (int be = 0; be < 4; ++be) {
+          const double2* base = p.half[par][3 * be + b] + h;
 #pragma unroll
-      for (int al = 0; al < 4; ++al) {
-        const int pa = c_gamma.pi[cl][al];
-        double sr = 0.0, si = 0.0;
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-          const double2* c1 = my + (3 * be + b) * 12;
-          const double2* c2 = my + (3 * rb + b) * 12;
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            const double2 u = c1[a * 4 + al];  // S[al a][be b]
-            const double2 v = c2[a * 4 + pa];  // S[pi(al) a][rho(be) b]
-            sr += u.x * v.x + u.y * v.y;       // conj(u) v
-            si += u.x * v.y - u.y * v.x;
-          }
+          for (int al = 0; al < 4; ++al) s[al][be] = __ldcs(base + (size_t)(a * 4 + al) * Vh);
         }
-        gr[al] = sr;
-        gi[al] = si;
-      }
-      for (int gm = 0; gm < ngam; ++gm) {
-        if (c_gamma.cls[gm] != cl) continue;
-        const Monomial& A = c_gamma.A[gm];
-        const double br = c_gamma.Bt[gm].re[be], bi = c_gamma.Bt[gm].im[be];
-        double cr = 0.0, ci = 0.0;
+        if (use & 1) {
 #pragma unroll
-        for (int al = 0; al < 4; ++al) {  // a_al G[al][be]
-          cr += A.re[al] * gr[al] - A.im[al] * gi[al];
-          ci += A.re[al] * gi[al] + A.im[al] * gr[al];
+          for (int al = 0; al < 4; ++al)
+#pragma unroll
+            for (int be = 0; be < 4; ++be)
+              g0[al * 4 + be] = fma(s[al][be].x, s[al][be].x, fma(s[al][be].y, s[al][be].y, g0[al * 4 + be]));
         }
-        acc[2 * gm] += br * cr - bi * ci;  // times b_be
-        acc[2 * gm + 1] += br * ci + bi * cr;
+        // conj(u) v for be = 0, 1
+        auto cross = [&](double (&g)[16], int x) {
+#pragma unroll
+          for (int al = 0; al < 4; ++al)
+#pragma unroll
+            for (int be = 0; be < 2; ++be) {
+              const double2 u = s[al][be], v = s[al ^ x][be ^ x];
+              double& re = g[(al * 2 + be) * 2];
+              double& im = g[(al * 2 + be) * 2 + 1];
+              re = fma(u.x, v.x, fma(u.y, v.y, re));
+              im = fma(u.x, v.y, fma(-u.y, v.x, im));
+            }
+        };
+        if (use & 8) cross(g3, 3);
+        if (use & 4) cross(g2, 2);
       }
     }
   }
-  // fixed-order reduction: warp shuffles, then the warps in order
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int q = 0; q < 2 * ngam; ++q) {
-    double v = acc[q];
+  // fixed-order sum over the CTA: eight threads add sixteen values each of one number
+  auto reduce = [&](const double (&g)[16], int first) {
+    __syncthreads();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) red[wid][q] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < 2 * ngam) {
+    for (int q = 0; q < 16; ++q) sm[q][threadIdx.x] = g[q];
+    __syncthreads();
+    const int q = threadIdx.x >> 3, l = threadIdx.x & 7;
     double v = 0.0;
-    for (int w = 0; w < CTHREADS / 32; ++w) v += red[w][threadIdx.x];
-    partials[(size_t)blockIdx.x * 2 * ngam + threadIdx.x] = -v;
-  }
+#pragma unroll
+    for (int i = 0; i < CTHREADS / 8; ++i) v += sm[q][i * 8 + l];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, 8);
+    if (l == 0) partials[(size_t)blockIdx.x * NGRAM + first + q] = v;
+  };
+  if (use & 1) reduce(g0, 0);
+  if (use & 8) reduce(g3, 16);
+  if (use & 4) reduce(g2, 32);
 }
 
-// corr[gm][t] = sum over the tiles of slice t of the partials, in tile order
-__global__ void k_meson_slices(const double* partials, int ngam, int tiles_per_slice, int lt, double* corr) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;  // (gm, t, re/im)
-  if (i >= 2 * ngam * lt) return;
-  const int q = i % (2 * ngam), t = i / (2 * ngam);
+// One CTA per time slice: the slice's 48 numbers (its nblk partials added in a fixed order,
+// four interleaved sums each), then C(t) for every Gamma.
+__global__ void __launch_bounds__(4 * NGRAM) k_meson_slices(const double* partials, int ngam, int nblk, int lt,
+                                                            const GammaTab tab, double* corr) {
+  __shared__ double part[4][NGRAM], g[NGRAM];
+  const int t = blockIdx.x, q = threadIdx.x % NGRAM, w = threadIdx.x / NGRAM;
+  const int x = q < 16 ? 0 : (q < 32 ? 3 : 2);
   double v = 0.0;
-  for (int k = 0; k < tiles_per_slice; ++k) v += partials[((size_t)t * tiles_per_slice + k) * 2 * ngam + q];
-  const int gm = q / 2, ri = q % 2;
-  corr[((size_t)gm * lt + t) * 2 + ri] = v;
+  if ((tab.use >> x) & 1)
+    for (int k = w; k < nblk; k += 4) v += partials[((size_t)t * nblk + k) * NGRAM + q];
+  part[w][q] = v;
+  __syncthreads();
+  if (w == 0) g[q] = (part[0][q] + part[1][q]) + (part[2][q] + part[3][q]);
+  __syncthreads();
+  const int gm = threadIdx.x;
+  if (gm >= ngam) return;
+  double cr = 0.0, ci = 0.0;
+  const int xg = tab.x[gm];
+  auto add = [&](double2 a, double2 b, double re, double im) {  // a b (re + i im)
+    const double pr = a.x * b.x - a.y * b.y, pi = a.x * b.y + a.y * b.x;
+    cr += pr * re - pi * im;
+    ci += pr * im + pi * re;
+  };
+  for (int al = 0; al < 4; ++al) {
+    if (xg == 0) {
+      for (int be = 0; be < 4; ++be) add(tab.a[gm][al], tab.b[gm][be], g[al * 4 + be], 0.0);
+    } else {
+      const double* gx = g + (xg == 3 ? 16 : 32);
+      for (int be = 0; be < 2; ++be) {
+        const double re = gx[(al * 2 + be) * 2], im = gx[(al * 2 + be) * 2 + 1];
+        add(tab.a[gm][al], tab.b[gm][be], re, im);
+        add(tab.a[gm][al ^ xg], tab.b[gm][be ^ xg], re, -im);
+      }
+    }
+  }
+  corr[((size_t)gm * lt + t) * 2] = -cr;
+  corr[((size_t)gm * lt + t) * 2 + 1] = -ci;
 }
 
 }  // namespace
@@ -229,44 +245,39 @@ extern "C" int lqcd_meson_correlator(const lqcd_field* const* props, int ngamma,
     M4 Bt{};
     for (int r = 0; r < 4; ++r)
       for (int c = 0; c < 4; ++c) Bt[c][r] = B[r][c];
-    if (!monomial_rows(A, tab.A[i]) || !monomial_rows(Bt, tab.Bt[i]))
+    Monomial ma, mb;
+    if (!monomial_rows(A, ma) || !monomial_rows(Bt, mb))
       return set_error(LQCD_EINVAL, "gamma code %d is not monomial", gammas[i]);
-    // permutation class: pi from the rows of A, rho from the columns of B
-    int cl = 0;
-    for (; cl < tab.nclass; ++cl)
-      if (!memcmp(tab.pi[cl], tab.A[i].col, sizeof tab.pi[cl]) && !memcmp(tab.rho[cl], tab.Bt[i].col, sizeof tab.rho[cl]))
-        break;
-    if (cl == tab.nclass) {
-      memcpy(tab.pi[cl], tab.A[i].col, sizeof tab.pi[cl]);
-      memcpy(tab.rho[cl], tab.Bt[i].col, sizeof tab.rho[cl]);
-      ++tab.nclass;
+    const int x = ma.col[0];
+    for (int r = 0; r < 4; ++r) {
+      if ((x != 0 && x != 2 && x != 3) || ma.col[r] != (r ^ x) || mb.col[r] != (r ^ x))
+        return set_error(LQCD_EINVAL, "gamma code %d: unexpected spin structure", gammas[i]);
+      tab.a[i][r] = make_double2(ma.re[r], ma.im[r]);
+      tab.b[i][r] = make_double2(mb.re[r], mb.im[r]);
     }
-    tab.cls[i] = cl;
+    tab.x[i] = x;
+    tab.use |= 1 << x;
   }
   lqcd_ctx* c = f0->ctx;
   LQCD_CK(cudaSetDevice(c->device));
   const Geom& g = f0->g;
-  const int S3 = g.L[0] * g.L[1] * g.L[2];
-  const int tps = (S3 + CSITES - 1) / CSITES;
-  const int nblk = tps * g.L[3];
-  const size_t npart = (size_t)nblk * ngamma * 2;
-  std::vector<const double2*> hp(24);
+  Props props_arg;
   for (int i = 0; i < 12; ++i)
-    for (int p = 0; p < 2; ++p) hp[2 * i + p] = static_cast<const double2*>(props[i]->half[p]);
-  LQCD_CK(cudaMemcpyToSymbolAsync(c_gamma, &tab, sizeof tab, 0, cudaMemcpyHostToDevice, c->stream));
-  const size_t ncorr = (size_t)2 * ngamma * g.L[3];
-  const size_t nd = ((npart + ncorr + 31) / 32) * 32;
-  int rc = ctx_staging(c, nd * sizeof(double) + 24 * sizeof(void*) + 256);
-  if (rc != LQCD_OK) return rc;
+    for (int p = 0; p < 2; ++p) props_arg.half[p][i] = static_cast<const double2*>(props[i]->half[p]);
+  // Two sites per thread: the 48 sums' reduction costs about 3% of the site work, and CTAs
+  // stay small enough for even waves; one site per thread while that fills no more than the
+  // resident CTAs.
+  const int lt = g.L[3], slice = g.Vh / lt;
+  int nb = (slice + CTHREADS - 1) / CTHREADS;
+  if ((long long)2 * nb * lt > 2 * device_sm_count()) nb = (slice + 2 * CTHREADS - 1) / (2 * CTHREADS);
+  const int nblk = 2 * nb;  // per slice
+  const size_t npart = (size_t)nblk * lt * NGRAM;
+  const int nout = 2 * ngamma * lt;
+  LQCD_TRY(ctx_staging(c, (npart + nout) * sizeof(double)));
   double* d_part = c->staging;
-  const double2** d_props = reinterpret_cast<const double2**>(d_part + nd);
-  LQCD_CK(cudaMemcpyAsync(d_props, hp.data(), 24 * sizeof(void*), cudaMemcpyHostToDevice, c->stream));
-  const size_t smem = (size_t)CSITES * 144 * sizeof(double2);
-  LQCD_CK(cudaFuncSetAttribute(k_meson, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   double* d_corr = d_part + npart;  // ngamma x Lt complex, after the partials
-  k_meson<<<nblk, CTHREADS, smem, c->stream>>>(d_props, g, ngamma, tps, d_part);
-  const int nout = 2 * ngamma * g.L[3];
-  k_meson_slices<<<(nout + 127) / 128, 128, 0, c->stream>>>(d_part, ngamma, tps, g.L[3], d_corr);
+  k_meson<<<(unsigned)(nblk * lt), CTHREADS, 0, c->stream>>>(props_arg, g.Vh, slice, nb, tab.use, d_part);
+  k_meson_slices<<<lt, 4 * NGRAM, 0, c->stream>>>(d_part, ngamma, nblk, lt, tab, d_corr);
   LQCD_CK(cudaGetLastError());
   c->launches += 2;
   LQCD_CK(cudaMemcpyAsync(host_corr, d_corr, (size_t)nout * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
