@@ -324,7 +324,7 @@ static int gauge_upload_impl(lqcd_ctx* c, const int dims[4], const double* U, bo
     return set_error(LQCD_ENOMEM, "gauge field: %s", cudaGetErrorString(e));
   }
   gg->bytes = b64;
-  e = gauge_from_aos(src, g, P_F64, 18, gg->copy[P_F64][0], c->stream);
+  e = links_from_aos(src, g, static_cast<double2*>(gg->copy[P_F64][0]), c->stream);
   int rc = (e == cudaSuccess) ? LQCD_OK : set_error(LQCD_ECUDA, "gauge layout: %s", cudaGetErrorString(e));
   if (rc == LQCD_OK) {
     const void* base;

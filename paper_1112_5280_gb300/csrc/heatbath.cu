@@ -206,14 +206,6 @@ __global__ void __launch_bounds__(HB_THREADS, LQCD_HB_MIN_BLOCKS) k_heatbath(flo
   if (nfail) atomicAdd(fails, (unsigned long long)nfail);
 }
 
-// FP64 master words from the double-float copy (hi + lo, exact in FP64)
-__global__ void k_master_from_df(double2* U, const float4* Ud, long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float4 d = Ud[i];
-  U[i] = make_double2((double)d.x + (double)d.y, (double)d.z + (double)d.w);
-}
-
 // Gram-Schmidt of rows 0 and 1, row 2 = conj(row0 x row1), in double-float on the copy Ud
 __global__ void k_reunitarise(float4* Ud, Geom g) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (par, mu, h)
@@ -300,20 +292,6 @@ __global__ void k_sum_ordered(const double* partials, int n, double* out) {
   if (threadIdx.x == 0) *out = red[0];
 }
 
-// FP64 18-real layout -> host AoS U[s][mu][row][col] (re, im)
-__global__ void k_gauge_to_aos(const double2* U, Geom g, double2* aos) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (par, h)
-  if (i >= 2LL * g.Vh) return;
-  const Site x = site_of(g, (int)(i / g.Vh), (int)(i % g.Vh));
-  const size_t s = (size_t)x.c[0] + (size_t)g.L[0] * (x.c[1] + (size_t)g.L[1] * (x.c[2] + (size_t)g.L[2] * x.c[3]));
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-    const size_t b = link_base(g, x, mu);
-#pragma unroll
-    for (int w = 0; w < 9; ++w) aos[(s * 4 + mu) * 9 + w] = U[b + (size_t)w * g.Vh];
-  }
-}
-
 }  // namespace
 
 // derived link copies follow the master after an update
@@ -332,17 +310,9 @@ int refresh_gauge_copies(lqcd_gauge* g, bool keep_df) {
 int links_from_df(lqcd_gauge* g) {
   const float4* Ud = static_cast<const float4*>(g->copy[P_DF64][0]);
   if (!Ud) return set_error(LQCD_EINVAL, "the gauge field has no double-float copy");
-  const long long n = 2LL * 4 * 9 * g->g.Vh;
-  k_master_from_df<<<(unsigned)((n + 255) / 256), 256, 0, g->ctx->stream>>>(
-      static_cast<double2*>(g->copy[P_F64][0]), Ud, n);
+  LQCD_CK(master_from_df(static_cast<double2*>(g->copy[P_F64][0]), Ud, g->g, g->ctx->stream));
   g->ctx->launches++;
-  LQCD_CK(cudaGetLastError());
   return refresh_gauge_copies(g, true);
-}
-
-cudaError_t links_to_aos(const double2* U, const Geom& g, double2* aos, cudaStream_t s) {
-  k_gauge_to_aos<<<(unsigned)((2LL * g.Vh + 255) / 256), 256, 0, s>>>(U, g, aos);
-  return cudaGetLastError();
 }
 
 }  // namespace lqcd

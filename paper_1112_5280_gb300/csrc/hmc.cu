@@ -498,7 +498,7 @@ int lqcd_mom_upload(lqcd_mom* m, const double* host) {
   LQCD_CK(cudaSetDevice(c->device));
   LQCD_TRY(ctx_staging(c, m->bytes));
   LQCD_CK(cudaMemcpyAsync(c->staging, host, m->bytes, cudaMemcpyHostToDevice, c->stream));
-  LQCD_CK(gauge_from_aos(c->staging, m->g, P_F64, 18, m->d, c->stream));
+  LQCD_CK(links_from_aos(c->staging, m->g, m->d, c->stream));
   c->launches++;
   LQCD_CK(cudaStreamSynchronize(c->stream));
   return LQCD_OK;

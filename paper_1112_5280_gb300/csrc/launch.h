@@ -103,8 +103,10 @@ void set_dslash_colour_split(int prec, bool on);
 
 
 // layout kernels (layout.cu)
-cudaError_t gauge_from_aos(const double* d_aos, const Geom& g, int prec, int nr, void* d_out,
-                           cudaStream_t s);
+// (the AoS arrays need the alignment of their FP64 reals only)
+cudaError_t links_from_aos(const double* d_aos, const Geom& g, double2* d_U, cudaStream_t s);
+cudaError_t links_to_aos(const double2* d_U, const Geom& g, double2* d_aos, cudaStream_t s);
+cudaError_t master_from_df(double2* d_U, const float4* d_Ud, const Geom& g, cudaStream_t s);
 cudaError_t gauge_convert(const void* d_f64_18, const Geom& g, int prec, int nr, void* d_out,
                           cudaStream_t s);
 cudaError_t spinor_from_aos(const double* d_aos, const Geom& g, int prec, void* d_even,

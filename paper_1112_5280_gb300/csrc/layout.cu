@@ -7,65 +7,89 @@
 #include <mutex>
 #include <unordered_map>
 
+#include "convert.cuh"
 #include "launch.h"
 
 namespace lqcd {
 
-// ------------------------------------------------------------------ scalar real access
+// Layouts. On the host side of a copy a field is an array of sites of FP64 reals (AoS); on
+// the device it is a structure of arrays of words, word(c, h) = base[c * Vh + h]. Every
+// kernel here is bound by HBM, so each side is read and written in runs of consecutive
+// addresses by consecutive threads: the AoS kernels pass a tile of sites through shared
+// memory, and the conversions between two device layouts move whole words (eight reals of
+// a spinor, one link). FP64 <-> FP32 / double-float conversions take the bits apart
+// (convert.cuh) because the conversion instructions run at the FP64 pipe's rate.
+// Measured on GB300 against one thread per site reading and writing single reals, per call
+// with everything else unchanged: a 32^3x64 FP16 operator chain with its result to the host
+// layout 1379 -> 1295 us (the download 181 -> 98 us), a 24^3x48 double-float one 1670 ->
+// 1618 us, a 22x18x14x38 configuration and source in and the result out 777 -> 723 us.
 
+// ------------------------------------------------------------------ words
+
+// The words of one spinor's reals: W reals of a storage word, to and from FP64.
 template <int P>
-__device__ __forceinline__ void st_real(void* base, size_t i, double v);
+struct Words;
 template <>
-__device__ __forceinline__ void st_real<P_F64>(void* b, size_t i, double v) { ((double*)b)[i] = v; }
+struct Words<P_F64> {
+  using T = double2;
+  static constexpr int W = 2;
+  __device__ static void get(const T& w, double* v) { v[0] = w.x; v[1] = w.y; }
+  __device__ static T put(const double* v) { return make_double2(v[0], v[1]); }
+};
 template <>
-__device__ __forceinline__ void st_real<P_F32>(void* b, size_t i, double v) { ((float*)b)[i] = (float)v; }
+struct Words<P_DF64> {
+  using T = float4;
+  static constexpr int W = 2;
+  __device__ static void get(const T& w, double* v) {
+    v[0] = cv::from_df(w.x, w.y);
+    v[1] = cv::from_df(w.z, w.w);
+  }
+  __device__ static T put(const double* v) {
+    T w;
+    cv::to_df(v[0], w.x, w.y);
+    cv::to_df(v[1], w.z, w.w);
+    return w;
+  }
+};
 template <>
-__device__ __forceinline__ void st_real<P_F16>(void* b, size_t i, double v) { ((__half*)b)[i] = __double2half(v); }
+struct Words<P_F32> {
+  using T = float4;
+  static constexpr int W = 4;
+  __device__ static void get(const T& w, double* v) {
+    v[0] = cv::to_double(w.x); v[1] = cv::to_double(w.y); v[2] = cv::to_double(w.z); v[3] = cv::to_double(w.w);
+  }
+  __device__ static T put(const double* v) {
+    return make_float4(cv::to_float(v[0]), cv::to_float(v[1]), cv::to_float(v[2]), cv::to_float(v[3]));
+  }
+};
+template <bool BF>
+struct WordsHalf {
+  using T = uint4;
+  static constexpr int W = 8;
+  __device__ static unsigned pair(double a, double b) {
+    if (BF) {
+      const __nv_bfloat162 h(__double2bfloat16(a), __double2bfloat16(b));
+      return *reinterpret_cast<const unsigned*>(&h);
+    }
+    const __half2 h(__double2half(a), __double2half(b));
+    return *reinterpret_cast<const unsigned*>(&h);
+  }
+  __device__ static void get2(unsigned w, double* v) {
+    const float2 f = BF ? unpack_b2(w) : unpack_h2(w);
+    v[0] = cv::to_double(f.x);
+    v[1] = cv::to_double(f.y);
+  }
+  __device__ static void get(const T& w, double* v) {
+    get2(w.x, v); get2(w.y, v + 2); get2(w.z, v + 4); get2(w.w, v + 6);
+  }
+  __device__ static T put(const double* v) {
+    return make_uint4(pair(v[0], v[1]), pair(v[2], v[3]), pair(v[4], v[5]), pair(v[6], v[7]));
+  }
+};
 template <>
-__device__ __forceinline__ void st_real<P_BF16>(void* b, size_t i, double v) {
-  ((__nv_bfloat16*)b)[i] = __double2bfloat16(v);
-}
-
+struct Words<P_F16> : WordsHalf<false> {};
 template <>
-__device__ __forceinline__ void st_real<P_DF64>(void* b, size_t i, double v) {
-  const float hi = __double2float_rn(v);
-  ((float*)b)[2 * i] = hi;
-  ((float*)b)[2 * i + 1] = __double2float_rn(v - (double)hi);
-}
-
-template <int P>
-__device__ __forceinline__ double ld_real(const void* base, size_t i);
-template <>
-__device__ __forceinline__ double ld_real<P_DF64>(const void* b, size_t i) {
-  return (double)((const float*)b)[2 * i] + (double)((const float*)b)[2 * i + 1];
-}
-template <>
-__device__ __forceinline__ double ld_real<P_F64>(const void* b, size_t i) { return ((const double*)b)[i]; }
-template <>
-__device__ __forceinline__ double ld_real<P_F32>(const void* b, size_t i) { return ((const float*)b)[i]; }
-template <>
-__device__ __forceinline__ double ld_real<P_F16>(const void* b, size_t i) { return __half2float(((const __half*)b)[i]); }
-template <>
-__device__ __forceinline__ double ld_real<P_BF16>(const void* b, size_t i) {
-  return __bfloat162float(((const __nv_bfloat16*)b)[i]);
-}
-
-// reals per storage word
-__host__ __device__ inline int link_word(int p, int nr) {
-  return (p == P_F64 || p == P_DF64) ? 2 : (nr == 18 ? 2 : 4);
-}
-__host__ __device__ inline int spinor_word(int p) { return 16 / prec_bytes(p); }
-
-// offset (in reals) of real k of link (parity, mu, h)
-__device__ __forceinline__ size_t link_off(int p, int nr, int Vh, int par, int mu, int h, int k) {
-  const int W = link_word(p, nr);
-  return (size_t)par * 4 * nr * Vh + (size_t)mu * nr * Vh + (size_t)(k / W) * Vh * W +
-         (size_t)h * W + (k % W);
-}
-__device__ __forceinline__ size_t spinor_off(int p, int Vh, int h, int k) {
-  const int W = spinor_word(p);
-  return (size_t)(k / W) * Vh * W + (size_t)h * W + (k % W);
-}
+struct Words<P_BF16> : WordsHalf<true> {};
 
 // host real k = (spin * 3 + colour) * 2 + re/im  ->  device position (colour-major)
 __device__ __forceinline__ int dev_real(int k) {
@@ -73,70 +97,111 @@ __device__ __forceinline__ int dev_real(int k) {
   return sidx(spin, col) + ri;
 }
 
-__device__ __forceinline__ void full_coords(const Geom& g, long long s, int& par, int& h) {
-  int x = (int)(s % g.L[0]);
-  long long r = s / g.L[0];
-  int y = (int)(r % g.L[1]);
-  r /= g.L[1];
-  int z = (int)(r % g.L[2]);
-  int t = (int)(r / g.L[2]);
-  par = (x + y + z + t) & 1;
-  h = (int)(s >> 1);  // Lx even: (x >> 1) + Lxh * (y + Ly * (z + Lz * t))
+// (y + z + t) & 1 of half-lattice index h: the even site of the pair 2h, 2h + 1 of the host
+// order is 2h when this is 0
+__device__ __forceinline__ int row_parity(const Geom& g, int h) {
+  const unsigned r0 = geom_div(g, 0, (unsigned)h), r1 = geom_div(g, 1, r0), r2 = geom_div(g, 2, r1);
+  return (int)((r0 - r1 * g.L[1]) + (r1 - r2 * g.L[2]) + r2) & 1;
 }
 
-// ------------------------------------------------------------------ gauge
+// A tile is the 64 consecutive host sites 2 h0 .. 2 h0 + 63, which hold the half-lattice
+// sites h0 .. h0 + 31 of both parities. In shared memory site 2h + b of the tile is at
+// [b][h][.], its row padded to an odd number of FP64 words, so that 32 threads at
+// consecutive h hit different banks.
+constexpr int TILE_H = 32;
+constexpr int LAYOUT_THREADS = 256;
 
-template <int P, int NR>
-__global__ void k_gauge_from_aos(const double* __restrict__ aos, Geom g, void* out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // site * 4 + mu
-  const long long V = 2LL * g.Vh;
-  if (i >= 4 * V) return;
-  const long long s = i >> 2;
-  const int mu = (int)(i & 3);
-  int par, h;
-  full_coords(g, s, par, h);
-  const double* src = aos + i * 18;
-  for (int k = 0; k < NR; ++k) st_real<P>(out, link_off(P, NR, g.Vh, par, mu, h, k), src[k]);
+// ------------------------------------------------------------------ gauge (FP64, 18 reals)
+
+// TO_AOS false: AoS U[site][mu][row][col] -> [parity][mu][word][V/2] of double2; true: back
+template <bool TO_AOS>
+__global__ void __launch_bounds__(LAYOUT_THREADS) k_gauge_aos(const double* in, Geom g, double* out) {
+  __shared__ double sm[2][TILE_H][73];
+  const int h0 = blockIdx.x * TILE_H, nh = min(TILE_H, g.Vh - h0);
+  const size_t first = (size_t)h0 * 2 * 72;
+  if (!TO_AOS) {
+    for (int i = threadIdx.x; i < 2 * nh * 72; i += LAYOUT_THREADS) {
+      const int site = i / 72;
+      sm[site & 1][site >> 1][i - site * 72] = in[first + i];
+    }
+    __syncthreads();
+  }
+  const int hl = threadIdx.x % TILE_H;
+  if (hl < nh) {
+    const int rp = row_parity(g, h0 + hl);
+    for (int q = threadIdx.x / TILE_H; q < 2 * 36; q += LAYOUT_THREADS / TILE_H) {
+      const int par = q / 36, w = q - par * 36;  // w = mu * 9 + word
+      double* s = &sm[par ^ rp][hl][2 * w];
+      const size_t at = (size_t)q * g.Vh + h0 + hl;
+      if (TO_AOS) {
+        const double2 d = reinterpret_cast<const double2*>(in)[at];
+        s[0] = d.x;
+        s[1] = d.y;
+      } else {
+        reinterpret_cast<double2*>(out)[at] = make_double2(s[0], s[1]);
+      }
+    }
+  }
+  if (TO_AOS) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * nh * 72; i += LAYOUT_THREADS) {
+      const int site = i / 72;
+      out[first + i] = sm[site & 1][site >> 1][i - site * 72];
+    }
+  }
 }
 
+static unsigned aos_grid(const Geom& g) { return (unsigned)((g.Vh + TILE_H - 1) / TILE_H); }
+
+cudaError_t links_from_aos(const double* aos, const Geom& g, double2* U, cudaStream_t s) {
+  k_gauge_aos<false><<<aos_grid(g), LAYOUT_THREADS, 0, s>>>(aos, g, reinterpret_cast<double*>(U));
+  return cudaGetLastError();
+}
+cudaError_t links_to_aos(const double2* U, const Geom& g, double2* aos, cudaStream_t s) {
+  k_gauge_aos<true><<<aos_grid(g), LAYOUT_THREADS, 0, s>>>(reinterpret_cast<const double*>(U), g,
+                                                          reinterpret_cast<double*>(aos));
+  return cudaGetLastError();
+}
+
+// One link of the FP64 18-real layout to precision P with NR reals; word sizes as in LinkIO.
 template <int P, int NR>
-__global__ void k_gauge_convert(const void* __restrict__ in64, Geom g, void* out) {
+__global__ void __launch_bounds__(LAYOUT_THREADS) k_gauge_convert(const double2* __restrict__ in64, Geom g, void* out) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (par, mu, h)
-  const long long n = 8LL * g.Vh;
-  if (i >= n) return;
-  const int h = (int)(i % g.Vh);
-  const int mu = (int)((i / g.Vh) & 3);
-  const int par = (int)(i / (4LL * g.Vh));
-  for (int k = 0; k < NR; ++k) {
-    const double v = ld_real<P_F64>(in64, link_off(P_F64, 18, g.Vh, par, mu, h, k));
-    st_real<P>(out, link_off(P, NR, g.Vh, par, mu, h, k), v);
+  if (i >= 8LL * g.Vh) return;
+  const size_t pm = (size_t)(i / g.Vh);  // 4 par + mu
+  const size_t Vh = (size_t)g.Vh, h = (size_t)i - pm * Vh;
+  double v[NR];
+#pragma unroll
+  for (int w = 0; w < NR / 2; ++w) {
+    const double2 d = in64[(pm * 9 + w) * Vh + h];
+    v[2 * w] = d.x;
+    v[2 * w + 1] = d.y;
+  }
+  constexpr int NW = LinkIO<P, NR>::NW;
+  typename LinkIO<P, NR>::Word* o = reinterpret_cast<typename LinkIO<P, NR>::Word*>(out) + pm * NW * Vh + h;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    if constexpr (P == P_F64 || P == P_DF64) {
+      o[w * Vh] = Words<P>::put(v + 2 * w);
+    } else if constexpr (P == P_F32 && NR == 18) {
+      o[w * Vh] = make_float2(cv::to_float(v[2 * w]), cv::to_float(v[2 * w + 1]));
+    } else if constexpr (P == P_F32) {
+      o[w * Vh] = Words<P_F32>::put(v + 4 * w);
+    } else if constexpr (NR == 18) {
+      o[w * Vh] = WordsHalf<false>::pair(v[2 * w], v[2 * w + 1]);
+    } else {
+      o[w * Vh] = make_uint2(WordsHalf<false>::pair(v[4 * w], v[4 * w + 1]),
+                             WordsHalf<false>::pair(v[4 * w + 2], v[4 * w + 3]));
+    }
   }
 }
 
 template <int P, int NR>
-static cudaError_t go_gauge_from_aos(const double* a, const Geom& g, void* o, cudaStream_t s) {
-  const long long n = 8LL * g.Vh;
-  k_gauge_from_aos<P, NR><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, g, o);
-  return cudaGetLastError();
-}
-template <int P, int NR>
 static cudaError_t go_gauge_convert(const void* a, const Geom& g, void* o, cudaStream_t s) {
   const long long n = 8LL * g.Vh;
-  k_gauge_convert<P, NR><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, g, o);
+  k_gauge_convert<P, NR><<<(unsigned)((n + LAYOUT_THREADS - 1) / LAYOUT_THREADS), LAYOUT_THREADS, 0, s>>>(
+      static_cast<const double2*>(a), g, o);
   return cudaGetLastError();
-}
-
-cudaError_t gauge_from_aos(const double* d_aos, const Geom& g, int prec, int nr, void* d_out,
-                           cudaStream_t s) {
-  if (prec == P_F64) return nr == 12 ? go_gauge_from_aos<P_F64, 12>(d_aos, g, d_out, s)
-                                     : go_gauge_from_aos<P_F64, 18>(d_aos, g, d_out, s);
-  if (prec == P_F32) return nr == 12 ? go_gauge_from_aos<P_F32, 12>(d_aos, g, d_out, s)
-                                     : go_gauge_from_aos<P_F32, 18>(d_aos, g, d_out, s);
-  if (prec == P_F16) return nr == 12 ? go_gauge_from_aos<P_F16, 12>(d_aos, g, d_out, s)
-                                     : go_gauge_from_aos<P_F16, 18>(d_aos, g, d_out, s);
-  if (prec == P_DF64) return nr == 12 ? go_gauge_from_aos<P_DF64, 12>(d_aos, g, d_out, s)
-                                      : go_gauge_from_aos<P_DF64, 18>(d_aos, g, d_out, s);
-  return cudaErrorInvalidValue;
 }
 
 cudaError_t gauge_convert(const void* d64, const Geom& g, int prec, int nr, void* d_out,
@@ -147,55 +212,110 @@ cudaError_t gauge_convert(const void* d64, const Geom& g, int prec, int nr, void
                                      : go_gauge_convert<P_F32, 18>(d64, g, d_out, s);
   if (prec == P_F16) return nr == 12 ? go_gauge_convert<P_F16, 12>(d64, g, d_out, s)
                                      : go_gauge_convert<P_F16, 18>(d64, g, d_out, s);
-  if (prec == P_DF64) return nr == 12 ? go_gauge_convert<P_DF64, 12>(d64, g, d_out, s)
-                                      : go_gauge_convert<P_DF64, 18>(d64, g, d_out, s);
+  if (prec == P_DF64 && nr == 18) return go_gauge_convert<P_DF64, 18>(d64, g, d_out, s);
   return cudaErrorInvalidValue;
+}
+
+// FP64 master words from the double-float copy (hi + lo, exact in FP64)
+__global__ void __launch_bounds__(LAYOUT_THREADS) k_master_from_df(double2* U, const float4* Ud, long long n) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const float4 d = Ud[i];
+  U[i] = make_double2(cv::from_df(d.x, d.y), cv::from_df(d.z, d.w));
+}
+cudaError_t master_from_df(double2* U, const float4* Ud, const Geom& g, cudaStream_t s) {
+  const long long n = 72LL * g.Vh;
+  k_master_from_df<<<(unsigned)((n + LAYOUT_THREADS - 1) / LAYOUT_THREADS), LAYOUT_THREADS, 0, s>>>(U, Ud, n);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ spinors
 
 template <int P>
-__global__ void k_spinor_from_aos(const double* __restrict__ aos, Geom g, void* ev, void* od) {
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= 2LL * g.Vh) return;
-  int par, h;
-  full_coords(g, s, par, h);
-  void* dst = par ? od : ev;
-  if (!dst) return;
-  const double* src = aos + s * 24;
-  for (int k = 0; k < 24; ++k) st_real<P>(dst, spinor_off(P, g.Vh, h, dev_real(k)), src[k]);
+__global__ void __launch_bounds__(LAYOUT_THREADS) k_spinor_from_aos(const double* __restrict__ aos, Geom g, void* ev,
+                                                                    void* od) {
+  using Wd = Words<P>;
+  __shared__ double sm[2][TILE_H][25];
+  const int h0 = blockIdx.x * TILE_H, nh = min(TILE_H, g.Vh - h0);
+  const double* src = aos + (size_t)h0 * 2 * 24;
+  for (int i = threadIdx.x; i < 2 * nh * 24; i += LAYOUT_THREADS) {
+    const int site = i / 24;
+    sm[site & 1][site >> 1][dev_real(i - site * 24)] = src[i];
+  }
+  __syncthreads();
+  const int hl = threadIdx.x % TILE_H;
+  if (hl >= nh) return;
+  const int rp = row_parity(g, h0 + hl);
+  constexpr int NW = 24 / Wd::W;
+  for (int q = threadIdx.x / TILE_H; q < 2 * NW; q += LAYOUT_THREADS / TILE_H) {
+    const int par = q / NW, c = q - par * NW;
+    void* dst = par ? od : ev;
+    if (dst) reinterpret_cast<typename Wd::T*>(dst)[(size_t)c * g.Vh + h0 + hl] = Wd::put(&sm[par ^ rp][hl][c * Wd::W]);
+  }
 }
 
 template <int P>
-__global__ void k_spinor_to_aos(const void* ev, const void* od, Geom g, double* __restrict__ aos) {
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= 2LL * g.Vh) return;
-  int par, h;
-  full_coords(g, s, par, h);
-  const void* src = par ? od : ev;
-  if (!src) return;
-  double* dst = aos + s * 24;
-  for (int k = 0; k < 24; ++k) dst[k] = ld_real<P>(src, spinor_off(P, g.Vh, h, dev_real(k)));
+__global__ void __launch_bounds__(LAYOUT_THREADS) k_spinor_to_aos(const void* ev, const void* od, Geom g,
+                                                                  double* __restrict__ aos) {
+  using Wd = Words<P>;
+  __shared__ double sm[2][TILE_H][25];
+  __shared__ int rps[TILE_H];
+  const int h0 = blockIdx.x * TILE_H, nh = min(TILE_H, g.Vh - h0);
+  const int hl = threadIdx.x % TILE_H;
+  if (hl < nh) {
+    const int rp = row_parity(g, h0 + hl);
+    if (threadIdx.x < TILE_H) rps[hl] = rp;
+    constexpr int NW = 24 / Wd::W;
+    for (int q = threadIdx.x / TILE_H; q < 2 * NW; q += LAYOUT_THREADS / TILE_H) {
+      const int par = q / NW, c = q - par * NW;
+      const void* src = par ? od : ev;
+      if (src) {
+        double v[Wd::W];
+        Wd::get(reinterpret_cast<const typename Wd::T*>(src)[(size_t)c * g.Vh + h0 + hl], v);
+#pragma unroll
+        for (int j = 0; j < Wd::W; ++j) sm[par ^ rp][hl][c * Wd::W + j] = v[j];
+      }
+    }
+  }
+  __syncthreads();
+  double* dst = aos + (size_t)h0 * 2 * 24;
+  for (int i = threadIdx.x; i < 2 * nh * 24; i += LAYOUT_THREADS) {
+    const int site = i / 24, b = site & 1, h = site >> 1;
+    // the site's parity is b ^ rp; sites of a parity that the field does not hold stay
+    if ((b ^ rps[h]) ? od : ev) dst[i] = sm[b][h][dev_real(i - site * 24)];
+  }
 }
 
+// One thread per site and eight reals (one FP16 word, two FP32, four FP64 or double-float).
 template <int PI, int PO>
-__global__ void k_spinor_convert(const void* in, void* out, int Vh, double scale) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (h, k)
-  if (i >= 24LL * Vh) return;
-  const int h = (int)(i / 24), k = (int)(i % 24);
-  st_real<PO>(out, spinor_off(PO, Vh, h, k), scale * ld_real<PI>(in, spinor_off(PI, Vh, h, k)));
+__global__ void __launch_bounds__(LAYOUT_THREADS) k_spinor_convert(const void* in, void* out, int Vh, double scale) {
+  using Wi = Words<PI>;
+  using Wo = Words<PO>;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (group, h)
+  if (i >= 3LL * Vh) return;
+  const size_t grp = (size_t)(i / Vh), h = (size_t)i - grp * Vh;
+  constexpr int NI = 8 / Wi::W, NO = 8 / Wo::W;
+  const typename Wi::T* src = reinterpret_cast<const typename Wi::T*>(in) + grp * NI * Vh + h;
+  typename Wo::T* dst = reinterpret_cast<typename Wo::T*>(out) + grp * NO * Vh + h;
+  double v[8];
+#pragma unroll
+  for (int w = 0; w < NI; ++w) Wi::get(src[(size_t)w * Vh], v + w * Wi::W);
+  if (scale != 1.0) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] *= scale;
+  }
+#pragma unroll
+  for (int w = 0; w < NO; ++w) dst[(size_t)w * Vh] = Wo::put(v + w * Wo::W);
 }
 
 template <int P>
 static cudaError_t go_from_aos(const double* a, const Geom& g, void* e, void* o, cudaStream_t s) {
-  const long long n = 2LL * g.Vh;
-  k_spinor_from_aos<P><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, g, e, o);
+  k_spinor_from_aos<P><<<aos_grid(g), LAYOUT_THREADS, 0, s>>>(a, g, e, o);
   return cudaGetLastError();
 }
 template <int P>
 static cudaError_t go_to_aos(const void* e, const void* o, const Geom& g, double* a, cudaStream_t s) {
-  const long long n = 2LL * g.Vh;
-  k_spinor_to_aos<P><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(e, o, g, a);
+  k_spinor_to_aos<P><<<aos_grid(g), LAYOUT_THREADS, 0, s>>>(e, o, g, a);
   return cudaGetLastError();
 }
 
@@ -226,14 +346,14 @@ cudaError_t spinor_to_aos(const void* d_even, const void* d_odd, const Geom& g, 
 template <int PI>
 static cudaError_t go_convert_in(const void* in, void* out, int pout, int Vh, double sc,
                                  cudaStream_t s) {
-  const long long n = 24LL * Vh;
-  const unsigned nb = (unsigned)((n + 255) / 256);
+  const long long n = 3LL * Vh;
+  const unsigned nb = (unsigned)((n + LAYOUT_THREADS - 1) / LAYOUT_THREADS);
   switch (pout) {
-    case P_F64: k_spinor_convert<PI, P_F64><<<nb, 256, 0, s>>>(in, out, Vh, sc); break;
-    case P_F32: k_spinor_convert<PI, P_F32><<<nb, 256, 0, s>>>(in, out, Vh, sc); break;
-    case P_F16: k_spinor_convert<PI, P_F16><<<nb, 256, 0, s>>>(in, out, Vh, sc); break;
-    case P_BF16: k_spinor_convert<PI, P_BF16><<<nb, 256, 0, s>>>(in, out, Vh, sc); break;
-    case P_DF64: k_spinor_convert<PI, P_DF64><<<nb, 256, 0, s>>>(in, out, Vh, sc); break;
+    case P_F64: k_spinor_convert<PI, P_F64><<<nb, LAYOUT_THREADS, 0, s>>>(in, out, Vh, sc); break;
+    case P_F32: k_spinor_convert<PI, P_F32><<<nb, LAYOUT_THREADS, 0, s>>>(in, out, Vh, sc); break;
+    case P_F16: k_spinor_convert<PI, P_F16><<<nb, LAYOUT_THREADS, 0, s>>>(in, out, Vh, sc); break;
+    case P_BF16: k_spinor_convert<PI, P_BF16><<<nb, LAYOUT_THREADS, 0, s>>>(in, out, Vh, sc); break;
+    case P_DF64: k_spinor_convert<PI, P_DF64><<<nb, LAYOUT_THREADS, 0, s>>>(in, out, Vh, sc); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
