@@ -359,94 +359,149 @@ __device__ __forceinline__ void dslash_site(const Geom& g, int h, int out_par, c
 // U^dag = conj(column col of U(x - mu)) (backward). The accumulator and the link
 // data per thread shrink three-fold; this pays where the per-site work is latency
 // bound at low occupancy (double-float), not where it is memory bound.
-
+//
 // The three threads of a site (colour col = 0, 1, 2, in different warps of the CTA) each
 // need the projected half spinor h of all three colours of a neighbour. Each thread loads
 // and projects only its own colour and publishes it in shared memory; after a barrier it
 // reads the other two. Per hop that is one third of the spinor loads and projections of
-// the unshared form, at the cost of one CTA barrier per hop (two buffers alternate, so one
-// barrier per hop suffices). Every thread of the CTA must run all 8 hops: threads past
-// the end of the lattice pass a clamped site and discard the result.
+// the unshared form, at the cost of one CTA barrier per direction, whose forward and
+// backward hops share it (two buffers alternate over the directions, so one barrier
+// suffices). Every thread of the CTA must run all 8 hops: threads past the end of the
+// lattice pass a clamped site and discard the result.
+//
+// The arithmetic is packed (field.cuh): the lanes are the two spin rows of h, which meet the
+// same link entry. Bound by the FP32 pipe (9482 operations per site; the pipe's rate in long
+// chains of these operations is 31 T/s, 0.10 ms at 24^3x48) and by the latency of the loads
+// before each barrier. Scalar arithmetic with one barrier per hop took 174.7 us per
+// application at 24^3x48 and 531 at 32^3x64; packed 145.9 and 475; with a direction's two
+// hops on one barrier 144.4 and 464 (39.4, 36.7 and 36.1 us at 16^3x32). Staging the next
+// hop's words in shared memory with cp.async measured slower than plain loads (158 us at
+// 24^3x48), and so did 3 or 5 CTAs per SM (152 and 178 us against 144 at 4).
 
-// one buffer: [colour][h0 | h1][tile site] of (re.hi, re.lo, im.hi, im.lo)
+// NT sites: two buffers (alternating over the directions) of the forward and the backward
+// hop's [colour][re | im][site], each word (h0.hi, h1.hi, h0.lo, h1.lo)
 template <int NT>
 struct ProjShare {
-  float4 h[2][3][2][NT];
+  ulonglong2 h[2][2][3][2][NT];
 };
 
-__device__ __forceinline__ float4 pack_c(const Cx<df64>& a) { return make_float4(a.re.hi, a.re.lo, a.im.hi, a.im.lo); }
-__device__ __forceinline__ Cx<df64> unpack_c(const float4& d) { return {df64(d.x, d.y), df64(d.z, d.w)}; }
+// S a on both lanes
+template <int S>
+__device__ __forceinline__ df64x2 df2_sgn(df64x2 a) {
+  if (S > 0) return a;
+  return {p_neg(a.hi), p_neg(a.lo)};
+}
+// (S a, -S b) of the lanes (a, b)
+template <int S>
+__device__ __forceinline__ f32x2 p_alt(f32x2 v) {
+  float a, b;
+  p_unpack(v, a, b);
+  return S > 0 ? p_pack(a, -b) : p_pack(-a, b);
+}
+template <int S>
+__device__ __forceinline__ df64x2 df2_alt(df64x2 a) { return {p_alt<S>(a.hi), p_alt<S>(a.lo)}; }
+__device__ __forceinline__ f32x2 p_swap(f32x2 v) {
+  float a, b;
+  p_unpack(v, a, b);
+  return p_pack(b, a);
+}
 
-template <int K, int LP, bool DAG, int NT>
-__device__ __forceinline__ void hop3s_df(const Geom& g, int h, const int nf[4], const int nb[4], int t,
-                                         const void* in, const void* Uout, const void* Uin, int col, int j,
-                                         df64 acc[8], ProjShare<NT>& sh) {
-  constexpr int MU = K / 2;
-  constexpr bool FWD = (K % 2) == 0;
-  constexpr int S = FWD ? (DAG ? 1 : -1) : (DAG ? -1 : 1);
-  const int n = FWD ? nf[MU] : nb[MU];
-  df64 v[8];
-  SpinorIO<P_DF64>::load_colour(in, g.Vh, n, col, v);
-  const Cx<df64> p0{v[0], v[1]}, p1{v[2], v[3]}, p2{v[4], v[5]}, p3{v[6], v[7]};
-  Cx<df64> h0, h1;
+// acc: packed sums of the site's colour col. up: spins (0, 1), low: spins (3, 2) through the
+// x and y hops, whose lower components are crossed, and (2, 3) after them.
+struct Acc3 {
+  df64x2 up_re, up_im, low_re, low_im;
+};
+
+// projected half spinor of one colour's words (lanes h0, h1)
+template <int MU, int S>
+__device__ __forceinline__ void project3(const float4 d[4], df64x2& hr, df64x2& hi) {
+  auto re = [&](int sp) { return df64(d[sp].x, d[sp].y); };
+  auto im = [&](int sp) { return df64(d[sp].z, d[sp].w); };
+  const df64x2 pr = df2_pack(re(0), re(1)), pi = df2_pack(im(0), im(1));
   if (MU == 0) {
-    h0 = {df_add_u(p0.re, S * p3.im), df_add_u(p0.im, S * -p3.re)};
-    h1 = {df_add_u(p1.re, S * p2.im), df_add_u(p1.im, S * -p2.re)};
+    hr = df2_add_u(pr, df2_pack(S * im(3), S * im(2)));
+    hi = df2_add_u(pi, df2_pack(S * -re(3), S * -re(2)));
   } else if (MU == 1) {
-    h0 = {df_add_u(p0.re, S * -p3.re), df_add_u(p0.im, S * -p3.im)};
-    h1 = {df_add_u(p1.re, S * p2.re), df_add_u(p1.im, S * p2.im)};
+    hr = df2_add_u(pr, df2_pack(S * -re(3), S * re(2)));
+    hi = df2_add_u(pi, df2_pack(S * -im(3), S * im(2)));
   } else if (MU == 2) {
-    h0 = {df_add_u(p0.re, S * p2.im), df_add_u(p0.im, S * -p2.re)};
-    h1 = {df_add_u(p1.re, S * -p3.im), df_add_u(p1.im, S * p3.re)};
+    hr = df2_add_u(pr, df2_pack(S * im(2), S * -im(3)));
+    hi = df2_add_u(pi, df2_pack(S * -re(2), S * re(3)));
   } else {
-    h0 = {df_add_u(p0.re, S * p2.re), df_add_u(p0.im, S * p2.im)};
-    h1 = {df_add_u(p1.re, S * p3.re), df_add_u(p1.im, S * p3.im)};
+    hr = df2_add_u(pr, df2_pack(S * re(2), S * re(3)));
+    hi = df2_add_u(pi, df2_pack(S * im(2), S * im(3)));
   }
-  float4 (&buf)[3][2][NT] = sh.h[K & 1];
-  buf[col][0][j] = pack_c(h0);
-  buf[col][1][j] = pack_c(h1);
-  // row col of U (forward) or of U(x - mu)^dag (backward)
-  df64 r[6];
-  {
-    const char* base = link_dir<LP, 18>(FWD ? Uout : Uin, g.Vh, MU);
-    const int hl = FWD ? h : n;
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int word = FWD ? (3 * col + b) : (3 * b + col);
-      const float4 d = ld_stream(reinterpret_cast<const float4*>(base) + hl + (size_t)word * g.Vh);
-      r[2 * b] = df64(d.x, d.y);
-      r[2 * b + 1] = FWD ? df64(d.z, d.w) : df64(-d.z, -d.w);
-    }
-  }
-  __syncthreads();
-  Cx<df64> w0{df64(0.0f, 0.0f), df64(0.0f, 0.0f)}, w1 = w0;
+}
+
+// acc += (1 + S g_MU) applied to the link row u times the published h, times eta = +-1
+template <int MU, int S, bool ADJ, int NT>
+__device__ __forceinline__ void hop3_mac(const float4 u[3], const ulonglong2 (&buf)[3][2][NT], int j, int eta, Acc3& acc) {
+  df64x2 wr{0ull, 0ull}, wi{0ull, 0ull};  // lanes (w0, w1)
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
-    const Cx<df64> hb0 = unpack_c(buf[b][0][j]), hb1 = unpack_c(buf[b][1][j]);
-    const df64 rr = r[2 * b], ri = r[2 * b + 1];
-    df_mac_u(w0.re, rr, hb0.re);
-    df_mac_u(w0.re, -ri, hb0.im);
-    df_mac_u(w0.im, rr, hb0.im);
-    df_mac_u(w0.im, ri, hb0.re);
-    df_mac_u(w1.re, rr, hb1.re);
-    df_mac_u(w1.re, -ri, hb1.im);
-    df_mac_u(w1.im, rr, hb1.im);
-    df_mac_u(w1.im, ri, hb1.re);
+    const ulonglong2 a = buf[b][0][j], c = buf[b][1][j];
+    const df64x2 hr{a.x, a.y}, hi{c.x, c.y};
+    const df64 r(u[b].x, u[b].y), i = ADJ ? df64(-u[b].z, -u[b].w) : df64(u[b].z, u[b].w);
+    const df64x2 rr = df2_pack(r, r), ri = df2_pack(i, i);
+    df2_mac_u(wr, rr, hr);
+    df2_mac_u(wr, df2_sgn<-1>(ri), hi);
+    df2_mac_u(wi, rr, hi);
+    df2_mac_u(wi, ri, hr);
   }
-  const int eta = (MU == 3 && t == (FWD ? g.L[3] - 1 : 0)) ? g.t_bc : 1;
   if (MU == 3 && eta < 0) {
-    w0 = sgn<-1>(w0);
-    w1 = sgn<-1>(w1);
+    wr = df2_sgn<-1>(wr);
+    wi = df2_sgn<-1>(wi);
   }
-  acc[0] = df_add_u(acc[0], w0.re); acc[1] = df_add_u(acc[1], w0.im);
-  acc[2] = df_add_u(acc[2], w1.re); acc[3] = df_add_u(acc[3], w1.im);
-  Cx<df64> l2, l3;
-  if (MU == 0) { l2 = sgn<S>(mul_i(w1)); l3 = sgn<S>(mul_i(w0)); }
-  else if (MU == 1) { l2 = sgn<S>(w1); l3 = sgn<-S>(w0); }
-  else if (MU == 2) { l2 = sgn<S>(mul_i(w0)); l3 = sgn<-S>(mul_i(w1)); }
-  else { l2 = sgn<S>(w0); l3 = sgn<S>(w1); }
-  acc[4] = df_add_u(acc[4], l2.re); acc[5] = df_add_u(acc[5], l2.im);
-  acc[6] = df_add_u(acc[6], l3.re); acc[7] = df_add_u(acc[7], l3.im);
+  acc.up_re = df2_add_u(acc.up_re, wr);
+  acc.up_im = df2_add_u(acc.up_im, wi);
+  if (MU == 0) {  // (l3, l2) = S i (w0, w1)
+    acc.low_re = df2_add_u(acc.low_re, df2_sgn<-S>(wi));
+    acc.low_im = df2_add_u(acc.low_im, df2_sgn<S>(wr));
+  } else if (MU == 1) {  // (l3, l2) = (-S w0, S w1)
+    acc.low_re = df2_add_u(acc.low_re, df2_alt<-S>(wr));
+    acc.low_im = df2_add_u(acc.low_im, df2_alt<-S>(wi));
+  } else if (MU == 2) {  // (l2, l3) = S i (w0, -w1)
+    acc.low_re = df2_add_u(acc.low_re, df2_alt<-S>(wi));
+    acc.low_im = df2_add_u(acc.low_im, df2_alt<S>(wr));
+  } else {  // (l2, l3) = S (w0, w1)
+    acc.low_re = df2_add_u(acc.low_re, df2_sgn<S>(wr));
+    acc.low_im = df2_add_u(acc.low_im, df2_sgn<S>(wi));
+  }
+}
+
+// the forward and the backward hop of direction MU, with one barrier for both
+template <int MU, int LP, bool DAG, int NT>
+__device__ __forceinline__ void hops3s_df(const Geom& g, int h, const int nf[4], const int nb[4], int t,
+                                          const void* in, const void* Uout, const void* Uin, int col, int j,
+                                          Acc3& acc, ProjShare<NT>& sh) {
+  constexpr int SF = DAG ? 1 : -1;
+  const int f = LQCD_SITE(nf[MU], g.Vh), b = LQCD_SITE(nb[MU], g.Vh), hs = LQCD_SITE(h, g.Vh);
+  const float4* s = reinterpret_cast<const float4*>(in) + (size_t)(4 * col) * g.Vh;
+  float4 df[4], db[4], uf[3], ub[3];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) df[c] = ld_ro(s + f + (size_t)c * g.Vh);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) db[c] = ld_ro(s + b + (size_t)c * g.Vh);
+  // row col of U(x) and of U(x - mu)^dag
+  const float4* pf = reinterpret_cast<const float4*>(link_dir<LP, 18>(Uout, g.Vh, MU)) + hs;
+  const float4* pb = reinterpret_cast<const float4*>(link_dir<LP, 18>(Uin, g.Vh, MU)) + b;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) uf[c] = ld_stream(pf + (size_t)(3 * col + c) * g.Vh);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) ub[c] = ld_stream(pb + (size_t)(3 * c + col) * g.Vh);
+  ulonglong2 (&buf)[2][3][2][NT] = sh.h[MU & 1];
+  {
+    df64x2 hr, hi;
+    project3<MU, SF>(df, hr, hi);
+    buf[0][col][0][j] = make_ulonglong2(hr.hi, hr.lo);
+    buf[0][col][1][j] = make_ulonglong2(hi.hi, hi.lo);
+    project3<MU, -SF>(db, hr, hi);
+    buf[1][col][0][j] = make_ulonglong2(hr.hi, hr.lo);
+    buf[1][col][1][j] = make_ulonglong2(hi.hi, hi.lo);
+  }
+  __syncthreads();
+  hop3_mac<MU, SF, false, NT>(uf, buf[0], j, (MU == 3 && t == g.L[3] - 1) ? g.t_bc : 1, acc);
+  hop3_mac<MU, -SF, true, NT>(ub, buf[1], j, (MU == 3 && t == 0) ? g.t_bc : 1, acc);
 }
 
 // acc = colour col of (D_{p,1-p} in)(h) in double-float, 18-real double-float links; all
@@ -457,18 +512,17 @@ __device__ __forceinline__ void dslash_site3s_df(const Geom& g, int h, int out_p
                                                  df64 acc[8], ProjShare<NT>& sh) {
   int nf[4], nb[4], t;
   neighbours(g, h, out_par, nf, nb, t);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) acc[i] = df64(0.0f, 0.0f);
-  hop3s_df<0, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, acc, sh);
-  hop3s_df<1, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, acc, sh);
-  hop3s_df<2, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, acc, sh);
-  hop3s_df<3, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, acc, sh);
-  hop3s_df<4, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, acc, sh);
-  hop3s_df<5, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, acc, sh);
-  hop3s_df<6, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, acc, sh);
-  hop3s_df<7, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, acc, sh);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) acc[i] = df_norm(acc[i]);
+  Acc3 s{{0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}};
+  hops3s_df<0, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, s, sh);
+  hops3s_df<1, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, s, sh);
+  s.low_re = {p_swap(s.low_re.hi), p_swap(s.low_re.lo)};
+  s.low_im = {p_swap(s.low_im.hi), p_swap(s.low_im.lo)};
+  hops3s_df<2, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, s, sh);
+  hops3s_df<3, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, s, sh);
+  df2_unpack(df2_norm(s.up_re), acc[0], acc[2]);
+  df2_unpack(df2_norm(s.up_im), acc[1], acc[3]);
+  df2_unpack(df2_norm(s.low_re), acc[4], acc[6]);
+  df2_unpack(df2_norm(s.low_im), acc[5], acc[7]);
 }
 
 }  // namespace lqcd

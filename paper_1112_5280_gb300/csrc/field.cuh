@@ -117,6 +117,77 @@ __device__ __forceinline__ df64 df_norm(df64 a) {
   return df64(s, __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, v)), __fsub_rn(a.lo, v)));
 }
 
+// Packed double-float: two df64 in the lanes of 64-bit register pairs (hi words in one,
+// lo words in the other), with FP32 pairs per instruction (add / mul / fma.rn.f32x2, each
+// lane rounded as the scalar instruction). A packed instruction takes the FMA pipe twice
+// as long as a scalar one, so the pipe's rate is the same; what it halves is the issue
+// slots, the code size and the number of independent instructions needed to fill the pipe.
+// Every function below does lane by lane the same operations as its scalar counterpart.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 p_pack(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void p_unpack(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 p_neg(f32x2 v) {
+  float a, b;
+  p_unpack(v, a, b);
+  return p_pack(-a, -b);
+}
+__device__ __forceinline__ f32x2 p_add(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 p_sub(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 p_mul(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 p_fma(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+struct df64x2 {
+  f32x2 hi, lo;
+};
+__device__ __forceinline__ df64x2 df2_pack(df64 a, df64 b) { return {p_pack(a.hi, b.hi), p_pack(a.lo, b.lo)}; }
+__device__ __forceinline__ void df2_unpack(df64x2 v, df64& a, df64& b) {
+  p_unpack(v.hi, a.hi, b.hi);
+  p_unpack(v.lo, a.lo, b.lo);
+}
+// df_add_u, df_mac_u and df_norm on both lanes
+__device__ __forceinline__ df64x2 df2_add_u(df64x2 a, df64x2 b) {
+  const f32x2 s = p_add(a.hi, b.hi);
+  const f32x2 v = p_sub(s, a.hi);
+  const f32x2 e = p_add(p_sub(a.hi, p_sub(s, v)), p_sub(b.hi, v));
+  return {s, p_add(e, p_add(a.lo, b.lo))};
+}
+__device__ __forceinline__ void df2_mac_u(df64x2& acc, df64x2 a, df64x2 b) {
+  const f32x2 p = p_mul(a.hi, b.hi);
+  f32x2 pe = p_fma(a.hi, b.hi, p_neg(p));
+  pe = p_fma(a.hi, b.lo, p_fma(a.lo, b.hi, pe));
+  const f32x2 s = p_add(acc.hi, p);
+  const f32x2 v = p_sub(s, acc.hi);
+  const f32x2 e = p_add(p_sub(acc.hi, p_sub(s, v)), p_sub(p, v));
+  acc.hi = s;
+  acc.lo = p_add(acc.lo, p_add(e, pe));
+}
+__device__ __forceinline__ df64x2 df2_norm(df64x2 a) {
+  const f32x2 s = p_add(a.hi, a.lo);
+  const f32x2 v = p_sub(s, a.hi);
+  return {s, p_add(p_sub(a.hi, p_sub(s, v)), p_sub(a.lo, v))};
+}
+
 // Arithmetic with a fixed rounding sequence. nvcc fuses a * b + c into one FMA where it
 // sees fit, and the same source inlined into two different kernels may be fused in two
 // different ways, which round differently. The site arithmetic of the Dslash, which must
