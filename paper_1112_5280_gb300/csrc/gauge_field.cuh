@@ -13,9 +13,6 @@ struct C2 {
   double re, im;
 };
 __device__ __forceinline__ C2 cmul(C2 a, C2 b) { return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
-__device__ __forceinline__ C2 cmulc(C2 a, C2 b) {  // a * conj(b)
-  return {a.re * b.re + a.im * b.im, a.im * b.re - a.re * b.im};
-}
 __device__ __forceinline__ C2 cadd(C2 a, C2 b) { return {a.re + b.re, a.im + b.im}; }
 
 struct M3 {
@@ -62,12 +59,6 @@ __device__ __forceinline__ M3 load_link(const double2* U, const Geom& g, const S
   }
   return m;
 }
-__device__ __forceinline__ void store_link(double2* U, const Geom& g, const Site& s, int mu, const M3& m) {
-  const size_t b = link_base(g, s, mu);
-#pragma unroll
-  for (int w = 0; w < 9; ++w) U[b + (size_t)w * g.Vh] = make_double2(m.e[w].re, m.e[w].im);
-}
-
 __device__ __forceinline__ M3 mul_nn(const M3& a, const M3& b) {
   M3 c;
 #pragma unroll
@@ -81,33 +72,6 @@ __device__ __forceinline__ M3 mul_nn(const M3& a, const M3& b) {
     }
   return c;
 }
-__device__ __forceinline__ M3 mul_nd(const M3& a, const M3& b) {  // a b^dag
-  M3 c;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      C2 s = cmulc(a.e[i * 3], b.e[j * 3]);
-      s = cadd(s, cmulc(a.e[i * 3 + 1], b.e[j * 3 + 1]));
-      s = cadd(s, cmulc(a.e[i * 3 + 2], b.e[j * 3 + 2]));
-      c.e[i * 3 + j] = s;
-    }
-  return c;
-}
-__device__ __forceinline__ M3 mul_dn(const M3& a, const M3& b) {  // a^dag b
-  M3 c;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      C2 s = cmulc(b.e[j], a.e[i]);
-      s = cadd(s, cmulc(b.e[3 + j], a.e[3 + i]));
-      s = cadd(s, cmulc(b.e[6 + j], a.e[6 + i]));
-      c.e[i * 3 + j] = s;
-    }
-  return c;
-}
-
 // ---------------------------------------------------------------- double-float matrices
 // The FP64 pipes of this part run at 1/64 of the FP32 rate, so the SU(3) products of the
 // gauge kernels run in double-float (pairs of FP32, 48-bit significand) on the FP32 pipes,
@@ -157,46 +121,40 @@ __device__ __forceinline__ void store_link_df(float4* U, const Geom& g, const Si
 #pragma unroll
   for (int w = 0; w < 9; ++w) U[b + (size_t)w * g.Vh] = make_float4(m.e[w].re.hi, m.e[w].re.lo, m.e[w].im.hi, m.e[w].im.lo);
 }
-__device__ __forceinline__ M3d to_df(const M3& a) {
-  M3d m;
-#pragma unroll
-  for (int w = 0; w < 9; ++w) m.e[w] = {df64(a.e[w].re), df64(a.e[w].im)};
-  return m;
+// Complex double-float scalars and matrices in packed arithmetic: the lanes are the real
+// and the imaginary part, so c += x y takes two packed multiply-accumulates, x.re (y.re, y.im)
+// and x.im (-y.im, y.re), in the order of the scalar form's four.
+__device__ __forceinline__ df64x2 c_pack(const C2d& a) { return df2_pack(a.re, a.im); }
+__device__ __forceinline__ df64x2 c_rot(const C2d& a) { return df2_pack(-a.im, a.re); }  // i a
+__device__ __forceinline__ df64x2 c_dup(df64 a) { return df2_pack(a, a); }
+__device__ __forceinline__ C2d c_unpack(df64x2 v) {
+  C2d r;
+  df2_unpack(v, r.re, r.im);
+  return r;
 }
-__device__ __forceinline__ M3 to_double(const M3d& a) {
-  M3 m;
-#pragma unroll
-  for (int w = 0; w < 9; ++w) m.e[w] = {(double)a.e[w].re, (double)a.e[w].im};
-  return m;
+__device__ __forceinline__ df64x2 c_zero() { return {0ull, 0ull}; }
+__device__ __forceinline__ void c_mac(df64x2& acc, const C2d& x, const C2d& y) {  // acc += x y
+  df2_mac_u(acc, c_dup(x.re), c_pack(y));
+  df2_mac_u(acc, c_dup(x.im), c_rot(y));
 }
 
-// complex double-float scalars
 __device__ __forceinline__ C2d cmul_d(const C2d& a, const C2d& b) {
-  df64 re(0.0f, 0.0f), im(0.0f, 0.0f);
-  df_mac_u(re, a.re, b.re);
-  df_mac_u(re, -a.im, b.im);
-  df_mac_u(im, a.re, b.im);
-  df_mac_u(im, a.im, b.re);
-  return {df_norm(re), df_norm(im)};
+  df64x2 s = c_zero();
+  c_mac(s, a, b);
+  return c_unpack(df2_norm(s));
 }
 __device__ __forceinline__ C2d cadd_d(const C2d& a, const C2d& b) {
-  return {df_norm(df_add_u(a.re, b.re)), df_norm(df_add_u(a.im, b.im))};
+  return c_unpack(df2_norm(df2_add_u(c_pack(a), c_pack(b))));
 }
 __device__ __forceinline__ C2d csub_d(const C2d& a, const C2d& b) { return cadd_d(a, {-b.re, -b.im}); }
 __device__ __forceinline__ C2d cscale_d(df64 f, const C2d& a) { return {f * a.re, f * a.im}; }
 
 // a x + b y in double-float
 __device__ __forceinline__ C2d cmix_d(const C2d& a, const C2d& x, const C2d& b, const C2d& y) {
-  df64 re(0.0f, 0.0f), im(0.0f, 0.0f);
-  df_mac_u(re, a.re, x.re);
-  df_mac_u(re, -a.im, x.im);
-  df_mac_u(re, b.re, y.re);
-  df_mac_u(re, -b.im, y.im);
-  df_mac_u(im, a.re, x.im);
-  df_mac_u(im, a.im, x.re);
-  df_mac_u(im, b.re, y.im);
-  df_mac_u(im, b.im, y.re);
-  return {df_norm(re), df_norm(im)};
+  df64x2 s = c_zero();
+  c_mac(s, a, x);
+  c_mac(s, b, y);
+  return c_unpack(df2_norm(s));
 }
 
 // 1/sqrt(n) for n > 0 in double-float: the FP32 estimate and two Newton-Raphson steps
@@ -211,65 +169,46 @@ __device__ __forceinline__ df64 df_rsqrt(df64 n) {
   return y;
 }
 
-// c = a op(b) with op(b) = b (DAGB false) or b^dag; a^dag b when DAGA
+// w += op(a) op(b) with op the adjoint where asked: each entry accumulates unnormalised
+// over k and is normalised once. Per k, an entry of b serves the three rows i at once.
+template <bool DAGA, bool DAGB>
+__device__ __forceinline__ void mac_d(M3d& w, const M3d& a, const M3d& b) {
+  df64x2 s[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) s[i] = c_pack(w.e[i]);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    df64x2 xr[3], xi[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const C2d x = DAGA ? a.e[k * 3 + i] : a.e[i * 3 + k];
+      xr[i] = c_dup(x.re);
+      xi[i] = c_dup(DAGA ? -x.im : x.im);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      C2d y = DAGB ? b.e[j * 3 + k] : b.e[k * 3 + j];
+      if (DAGB) y.im = -y.im;
+      const df64x2 yp = c_pack(y), yr = c_rot(y);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        df2_mac_u(s[i * 3 + j], xr[i], yp);
+        df2_mac_u(s[i * 3 + j], xi[i], yr);
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) w.e[i] = c_unpack(df2_norm(s[i]));
+}
+
+// op(a) op(b)
 template <bool DAGA, bool DAGB>
 __device__ __forceinline__ M3d mul_d(const M3d& a, const M3d& b) {
   M3d c;
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      df64 re(0.0f, 0.0f), im(0.0f, 0.0f);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const C2d x = DAGA ? a.e[k * 3 + i] : a.e[i * 3 + k];
-        const C2d y = DAGB ? b.e[j * 3 + k] : b.e[k * 3 + j];
-        // x' y' with x' = conj(x) when DAGA, y' = conj(y) when DAGB
-        const df64 xi = DAGA ? -x.im : x.im, yi = DAGB ? -y.im : y.im;
-        df_mac_u(re, x.re, y.re);
-        df_mac_u(re, -xi, yi);
-        df_mac_u(im, x.re, yi);
-        df_mac_u(im, xi, y.re);
-      }
-      c.e[i * 3 + j] = {df_norm(re), df_norm(im)};
-    }
+  for (int i = 0; i < 9; ++i) c.e[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
+  mac_d<DAGA, DAGB>(c, a, b);
   return c;
-}
-
-// w += a op(b) in double-float: each entry accumulates unnormalised over k and is
-// normalised once (the layout of mul_d, without the intermediate matrix)
-template <bool DAGA, bool DAGB>
-__device__ __forceinline__ void mac_d(M3d& w, const M3d& a, const M3d& b) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      df64 re = w.e[i * 3 + j].re, im = w.e[i * 3 + j].im;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const C2d x = DAGA ? a.e[k * 3 + i] : a.e[i * 3 + k];
-        const C2d y = DAGB ? b.e[j * 3 + k] : b.e[k * 3 + j];
-        const df64 xi = DAGA ? -x.im : x.im, yi = DAGB ? -y.im : y.im;
-        df_mac_u(re, x.re, y.re);
-        df_mac_u(re, -xi, yi);
-        df_mac_u(im, x.re, yi);
-        df_mac_u(im, xi, y.re);
-      }
-      w.e[i * 3 + j] = {df_norm(re), df_norm(im)};
-    }
-}
-
-// m or m^dag, chosen at run time (selects on registers)
-__device__ __forceinline__ M3d dagger_if(const M3d& m, bool dag) {
-  M3d r;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const C2d a = m.e[i * 3 + j], b = m.e[j * 3 + i];
-      r.e[i * 3 + j] = dag ? C2d{b.re, -b.im} : a;
-    }
-  return r;
 }
 
 // coordinate nu of s and the site shifted by d in direction nu, for a direction known only
@@ -286,30 +225,127 @@ __device__ __forceinline__ Site shifted_rt(const Geom& g, Site s, int nu, int d)
   return s;
 }
 
-// The staple sum W_mu(x) = sum_{nu != mu} U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-//                                         + U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)
-// for a direction mu known at run time, in double-float from the copy Ud. The six staples
-// run through one loop body of two products
+// ---------------------------------------------------------------- row-split products
+// Three threads per link, thread i holding row i of the matrix that is built up. A row of
+// a b needs row i of a and all of b, so a chain of products splits over rows without extra
+// arithmetic, and a thread needs a third of the accumulators: 24 warps per SM can be
+// resident where one thread per link took 254 registers (8 warps), which left the loads and
+// the chains of dependent operations uncovered (FMA pipe 60% busy). Entries are packed
+// (lanes re, im), each accumulated in the same order as in mac_d.
+struct RowD {
+  df64x2 e[3];
+};
+constexpr int SPLIT_LINKS = 64;                 // links per CTA
+constexpr int SPLIT_THREADS = 3 * SPLIT_LINKS;  // thread 64 i + j: row (or column) i of link j
+
+// one entry (re.hi, re.lo, im.hi, im.lo) as a packed pair, its imaginary part's sign flipped
+// by flip (0 or 0x80000000)
+__device__ __forceinline__ df64x2 c_entry(const float4& d, unsigned flip) {
+  const float ih = __uint_as_float(__float_as_uint(d.z) ^ flip), il = __uint_as_float(__float_as_uint(d.w) ^ flip);
+  return {p_pack(d.x, ih), p_pack(d.y, il)};
+}
+__device__ __forceinline__ df64x2 c_times_i(df64x2 a) {
+  C2d c = c_unpack(a);
+  return c_rot(c);
+}
+__device__ __forceinline__ void c_dups(df64x2 a, df64x2& re, df64x2& im) {
+  const C2d c = c_unpack(a);
+  re = c_dup(c.re);
+  im = c_dup(c.im);
+}
+
+// Row i of the staple sum
+//   W_mu(x) = sum_{nu != mu} U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
+//                          + U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)
+// for a direction mu known at run time, from the double-float copy Ud. The six staples run
+// through one loop body of two products
 //   up (nu):   T = U_nu(x+mu) U_mu(x+nu)^dag,          W += T U_nu(x)^dag
 //   down (nu): T = U_nu(x+mu-nu)^dag U_mu(x-nu)^dag,   W += T U_nu(x-nu)
-// so that the instructions of the loop stay in the instruction cache (fully unrolled, at
-// about 1400 instructions per double-float product, the staple sum did not).
-__device__ __forceinline__ M3d staple_df(const float4* Ud, const Geom& g, const Site& x, int mu) {
-  M3d W;
+// so that its instructions stay in the instruction cache; an adjoint is a choice of the
+// words read and of the sign of the imaginary parts.
+__device__ __forceinline__ RowD staple_row(const float4* Ud, const Geom& g, const Site& x, int mu, int i) {
+  RowD W;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) W.e[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
+  for (int c = 0; c < 3; ++c) W.e[c] = c_zero();
   const Site xp = shifted_rt(g, x, mu, 1);
+  const size_t vh = (size_t)g.Vh;
 #pragma unroll 1
   for (int t = 0; t < 6; ++t) {
-    const int k = t >> 1, nu = k + (k >= mu ? 1 : 0);
+    const int k0 = t >> 1, nu = k0 + (k0 >= mu ? 1 : 0);
     const bool up = (t & 1) == 0;
     const Site s0 = up ? xp : shifted_rt(g, xp, nu, -1);
     const Site s1 = shifted_rt(g, x, nu, up ? 1 : -1);
     const Site s2 = up ? x : s1;
-    const M3d T = mul_d<false, true>(dagger_if(load_link_df(Ud, g, s0, nu), !up), load_link_df(Ud, g, s1, mu));
-    mac_d<false, false>(W, T, dagger_if(load_link_df(Ud, g, s2, nu), up));
+    const unsigned flip_a = up ? 0u : 0x80000000u, flip_c = up ? 0x80000000u : 0u;
+    const size_t row = vh * 3, one = vh;
+    const float4* a = Ud + link_base(g, s0, nu) + (size_t)i * (up ? row : one);
+    const float4* b = Ud + link_base(g, s1, mu);
+    const float4* c = Ud + link_base(g, s2, nu);
+    const size_t a_step = up ? one : row;                        // over k
+    const size_t c_row = up ? one : row, c_col = up ? row : one;  // over k and over the column
+    RowD T;
+    {
+      df64x2 xr[3], xi[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) c_dups(c_entry(a[k * a_step], flip_a), xr[k], xi[k]);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        df64x2 s = c_zero();
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const df64x2 y = c_entry(b[(size_t)(3 * j + k) * vh], 0x80000000u);
+          df2_mac_u(s, xr[k], y);
+          df2_mac_u(s, xi[k], c_times_i(y));
+        }
+        T.e[j] = df2_norm(s);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      df64x2 xr, xi;
+      c_dups(T.e[k], xr, xi);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const df64x2 y = c_entry(c[k * c_row + q * c_col], flip_c);
+        df2_mac_u(W.e[q], xr, y);
+        df2_mac_u(W.e[q], xi, c_times_i(y));
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) W.e[q] = df2_norm(W.e[q]);
   }
   return W;
+}
+
+// A CTA's matrices in shared memory, one per link: entry [row][column][link]
+struct SplitM {
+  ulonglong2 e[3][3][SPLIT_LINKS];
+  __device__ __forceinline__ void put(int r, int c, int j, df64x2 v) { e[r][c][j] = make_ulonglong2(v.hi, v.lo); }
+  __device__ __forceinline__ df64x2 get(int r, int c, int j) const {
+    const ulonglong2 v = e[r][c][j];
+    return {v.x, v.y};
+  }
+};
+
+// row i of U W for the thread's link j: U's words from u (stride vh), W in shared memory
+__device__ __forceinline__ RowD split_row_times(const float4* u, size_t vh, int i, const SplitM& w, int j) {
+  RowD r;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) r.e[q] = c_zero();
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    df64x2 xr, xi;
+    c_dups(c_entry(u[(size_t)(3 * i + k) * vh], 0u), xr, xi);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const df64x2 y = w.get(k, q, j);
+      df2_mac_u(r.e[q], xr, y);
+      df2_mac_u(r.e[q], xi, c_times_i(y));
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) r.e[q] = df2_norm(r.e[q]);
+  return r;
 }
 
 }  // namespace gf

@@ -32,7 +32,6 @@ namespace {
 
 using namespace gf;
 
-constexpr int HB_THREADS = 128;
 constexpr int HB_MAX_ATTEMPTS = 1000;
 
 // ---------------------------------------------------------------- Philox4x64-10
@@ -133,18 +132,44 @@ __device__ __noinline__ bool su2_draw(double alpha, uint64_t seed, uint64_t c0, 
   return true;
 }
 
-// The SU(3) and SU(2) algebra (staple sum, V = U W, the subgroup projection c and its
-// direction v = c / |c|, a = b v, the rotations of U and V) in double-float from the copy Ud
-// on the FP32 pipes; the draw of b (Creutz) and |c| in FP64. The updated link goes to Ud
-// only: the caller rebuilds the FP64 master from it.
-// 3 CTAs of 128 threads per SM (168 registers, a 100-byte spill) against 2 (254 registers,
-// no spill): measured on GB300 at 32^3x64 beta 6, 39.7 against 43.2 ms per sweep with the
-// same chain; the update is latency bound, so the extra warps outweigh the spill. At 4 CTAs
-// (128 registers) the spill grows and the sweep takes 40.1 ms.
+// A class is updated in two launches. The algebra (staple sum, V = U W, the subgroup
+// projection c and its direction v = c / |c|, a = b v, the rotations of U and V) runs in
+// double-float from the copy Ud on the FP32 pipes; the draw of b (Creutz) and |c| in FP64.
+// The updated link goes to Ud only: the caller rebuilds the FP64 master from it.
+//
+// k_heatbath_v: V = U W of every link of the class, three threads per link (row-split
+// products in gauge_field.cuh), FP32 bound like the gauge force. V [word][V/2] stays in L2.
+// k_heatbath: the three subgroups, one thread per link, FP64 bound (about 200 FP64
+// instructions per draw). At 24^3x48, beta 6, a sweep takes 5.83 ms; as one kernel with one
+// thread per link (168 registers, staple code and draws sharing 12 warps per SM) 6.63 ms, and
+// as one kernel with three threads per link, where two thirds of the CTA wait at a barrier
+// during the draws, 6.27 ms.
+__global__ void __launch_bounds__(SPLIT_THREADS, 4) k_heatbath_v(const float4* Ud, Geom g, int mu, int par, float4* V) {
+  __shared__ SplitM sw;
+  const int j = threadIdx.x % SPLIT_LINKS, i = threadIdx.x / SPLIT_LINKS;
+  // threads past the last link repeat it (they share barriers and rows) and store nothing
+  const int at = blockIdx.x * SPLIT_LINKS + j, h = min(at, g.Vh - 1);
+  const Site x = site_of(g, par, h);
+  const size_t base = link_base(g, x, mu), vh = (size_t)g.Vh;
+  const RowD W = staple_row(Ud, g, x, mu, i);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) sw.put(i, q, j, W.e[q]);
+  __syncthreads();
+  const RowD r = split_row_times(Ud + base, vh, i, sw, j);
+  if (at >= g.Vh) return;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const C2d e = c_unpack(r.e[q]);
+    V[(size_t)(3 * i + q) * vh + h] = make_float4(e.re.hi, e.re.lo, e.im.hi, e.im.lo);
+  }
+}
+
+constexpr int HB_THREADS = 128;
+// 4 CTAs per SM (128 registers, a 108-byte spill): 3 and 5 measured the same.
 #ifndef LQCD_HB_MIN_BLOCKS
-#define LQCD_HB_MIN_BLOCKS 3
+#define LQCD_HB_MIN_BLOCKS 4
 #endif
-__global__ void __launch_bounds__(HB_THREADS, LQCD_HB_MIN_BLOCKS) k_heatbath(float4* Ud, Geom g, int mu,
+__global__ void __launch_bounds__(HB_THREADS, LQCD_HB_MIN_BLOCKS) k_heatbath(float4* Ud, const float4* Vd, Geom g, int mu,
                                                                              int par, double beta, uint64_t seed,
                                                                              uint64_t sweep,
                                                                              unsigned long long* fails) {
@@ -152,7 +177,12 @@ __global__ void __launch_bounds__(HB_THREADS, LQCD_HB_MIN_BLOCKS) k_heatbath(flo
   if (h >= g.Vh) return;
   const Site x = site_of(g, par, h);
   M3d u = load_link_df(Ud, g, x, mu);
-  M3d V = mul_d<false, false>(u, staple_df(Ud, g, x, mu));
+  M3d V;
+#pragma unroll
+  for (int w = 0; w < 9; ++w) {
+    const float4 d = Vd[(size_t)w * g.Vh + h];
+    V.e[w] = {df64(d.x, d.y), df64(d.z, d.w)};
+  }
   const uint64_t s = (uint64_t)x.c[0] + (uint64_t)g.L[0] * ((uint64_t)x.c[1] + (uint64_t)g.L[1] *
                      ((uint64_t)x.c[2] + (uint64_t)g.L[2] * (uint64_t)x.c[3]));
   const uint64_t link_id = 4 * s + (uint64_t)mu;
@@ -249,25 +279,23 @@ __global__ void k_reunitarise(float4* Ud, Geom g) {
     Ud[base + (size_t)w * g.Vh] = make_float4(r[w].re.hi, r[w].re.lo, r[w].im.hi, r[w].im.lo);
 }
 
-// per-CTA partial of sum_{x, mu<nu} Re Tr U_munu(x) over the sites of both parities
+// per-CTA partial of sum_x Re Tr U_munu(x) over the sites of both parities; blockIdx.y: the
+// plane mu < nu. Bound by the FP64 pipe (234 FMAs per plaquette, 1.5 ms at 24^3x48): one
+// thread per plaquette leaves registers for 16 warps per SM. One
+// thread per site held 254 registers: 2.43 ms at 24^3x48, this form 2.34 ms.
 constexpr int PLAQ_THREADS = 256;
-__global__ void __launch_bounds__(PLAQ_THREADS) k_plaquette(const double2* U, Geom g, double* partials) {
+__global__ void __launch_bounds__(PLAQ_THREADS, 2) k_plaquette(const double2* U, Geom g, double* partials) {
   __shared__ double red[PLAQ_THREADS];
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (par, h)
+  const int plane = blockIdx.y;                                           // 01 02 03 12 13 23
+  const int mu = plane < 3 ? 0 : (plane < 5 ? 1 : 2), nu = plane < 3 ? plane + 1 : (plane < 5 ? plane - 1 : 3);
   double acc = 0.0;
   if (i < 2LL * g.Vh) {
     const Site x = site_of(g, (int)(i / g.Vh), (int)(i % g.Vh));
+    const M3 a = mul_nn(load_link(U, g, x, mu), load_link(U, g, shifted_rt(g, x, mu, 1), nu));
+    const M3 b = mul_nn(load_link(U, g, x, nu), load_link(U, g, shifted_rt(g, x, nu, 1), mu));
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu)
-#pragma unroll
-      for (int nu = mu + 1; nu < 4; ++nu) {
-        const M3 a = mul_nn(load_link(U, g, x, mu), load_link(U, g, shifted(g, x, mu, 1), nu));
-        const M3 b = mul_nn(load_link(U, g, x, nu), load_link(U, g, shifted(g, x, nu, 1), mu));
-        double tr = 0.0;
-#pragma unroll
-        for (int w = 0; w < 9; ++w) tr += a.e[w].re * b.e[w].re + a.e[w].im * b.e[w].im;  // Re Tr a b^dag
-        acc += tr;
-      }
+    for (int w = 0; w < 9; ++w) acc += a.e[w].re * b.e[w].re + a.e[w].im * b.e[w].im;  // Re Tr a b^dag
   }
   red[threadIdx.x] = acc;
   __syncthreads();
@@ -275,7 +303,7 @@ __global__ void __launch_bounds__(PLAQ_THREADS) k_plaquette(const double2* U, Ge
     if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
     __syncthreads();
   }
-  if (threadIdx.x == 0) partials[blockIdx.x] = red[0];
+  if (threadIdx.x == 0) partials[(size_t)plane * gridDim.x + blockIdx.x] = red[0];
 }
 
 // out = sum of n partials in a fixed order (one CTA, strided then tree)
@@ -341,14 +369,18 @@ int lqcd_heatbath(lqcd_gauge* g, double beta, int nsweeps, unsigned long long se
   LQCD_TRY(gauge_links(g, P_DF64, &dfbase, &dfnr));
   float4* Ud = static_cast<float4*>(const_cast<void*>(dfbase));
   LQCD_CK(gauge_convert(U, g->g, P_DF64, 18, Ud, st));
+  const unsigned vgrid = (unsigned)((g->g.Vh + SPLIT_LINKS - 1) / SPLIT_LINKS);
   const unsigned grid = (unsigned)((g->g.Vh + HB_THREADS - 1) / HB_THREADS);
+  LQCD_TRY(ctx_staging(c, (size_t)9 * g->g.Vh * sizeof(float4)));
+  float4* V = reinterpret_cast<float4*>(c->staging);
   const unsigned rgrid = (unsigned)((8LL * g->g.Vh + 255) / 256);
   for (int sw = 0; sw < nsweeps; ++sw) {
     const uint64_t sweep = (uint64_t)(sweep0 + (unsigned long long)sw);
     for (int mu = 0; mu < 4; ++mu)
       for (int par = 0; par < 2; ++par) {
-        k_heatbath<<<grid, HB_THREADS, 0, st>>>(Ud, g->g, mu, par, beta, seed, sweep, d_fails);
-        c->launches++;
+        k_heatbath_v<<<vgrid, SPLIT_THREADS, 0, st>>>(Ud, g->g, mu, par, V);
+        k_heatbath<<<grid, HB_THREADS, 0, st>>>(Ud, V, g->g, mu, par, beta, seed, sweep, d_fails);
+        c->launches += 2;
       }
     if (reunit) {
       k_reunitarise<<<rgrid, 256, 0, st>>>(Ud, g->g);
@@ -372,13 +404,14 @@ int lqcd_plaquette(const lqcd_gauge* g, double* plaq) {
   LQCD_CK(cudaSetDevice(c->device));
   cudaStream_t st = c->stream;
   const int nb = (int)((2LL * g->g.Vh + PLAQ_THREADS - 1) / PLAQ_THREADS);
-  LQCD_TRY(ctx_partials(c, (size_t)nb + 1));
-  k_plaquette<<<nb, PLAQ_THREADS, 0, st>>>(static_cast<const double2*>(g->copy[P_F64][0]), g->g, c->partials);
-  k_sum_ordered<<<1, PLAQ_THREADS, 0, st>>>(c->partials, nb, c->partials + nb);
+  const int n = 6 * nb;
+  LQCD_TRY(ctx_partials(c, (size_t)n + 1));
+  k_plaquette<<<dim3(nb, 6), PLAQ_THREADS, 0, st>>>(static_cast<const double2*>(g->copy[P_F64][0]), g->g, c->partials);
+  k_sum_ordered<<<1, PLAQ_THREADS, 0, st>>>(c->partials, n, c->partials + n);
   c->launches += 2;
   LQCD_CK(cudaGetLastError());
   double sum = 0.0;
-  LQCD_CK(cudaMemcpyAsync(&sum, c->partials + nb, sizeof sum, cudaMemcpyDeviceToHost, st));
+  LQCD_CK(cudaMemcpyAsync(&sum, c->partials + n, sizeof sum, cudaMemcpyDeviceToHost, st));
   LQCD_CK(cudaStreamSynchronize(st));
   *plaq = sum / (18.0 * 2.0 * (double)g->g.Vh);
   return LQCD_OK;

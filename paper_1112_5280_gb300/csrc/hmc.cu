@@ -40,13 +40,9 @@ __device__ __forceinline__ int eo_index(const Geom& g, const Site& s) {
 
 // P_mu(x) += c TA(V) for a double-float V: TA(V)_ii = i (Im V_ii - Im tr V / 3),
 // TA(V)_ij = (V_ij - conj V_ji) / 2, TA_ji = -conj TA_ij; only the accumulation into the FP64
-// momenta runs in FP64
-__device__ __forceinline__ void add_ta(double2* P, const Geom& g, const Site& x, int mu, const M3d& V, double c) {
-  const size_t b = link_base(g, x, mu);
-  const size_t vh = (size_t)g.Vh;
-  double d[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) d[k] = (double)V.e[k * 4].im;
+// momenta runs in FP64. b: word 0 of the link (link_base).
+__device__ __forceinline__ void ta_diag(double2* P, size_t b, size_t vh, df64 i0, df64 i1, df64 i2, double c) {
+  const double d[3] = {(double)i0, (double)i1, (double)i2};
   const double tr = (d[0] + d[1] + d[2]) / 3.0;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -54,38 +50,70 @@ __device__ __forceinline__ void add_ta(double2* P, const Geom& g, const Site& x,
     q.y += c * (d[k] - tr);
     P[b + (size_t)(k * 4) * vh] = q;
   }
+}
+__device__ __forceinline__ void ta_pair(double2* P, size_t b, size_t vh, int r, int col, const C2d& x1, const C2d& y1,
+                                        double c) {
+  const double re = 0.5 * (double)df_add_u(x1.re, -y1.re), im = 0.5 * (double)df_add_u(x1.im, y1.im);
+  double2 q = P[b + (size_t)(r * 3 + col) * vh];
+  q.x += c * re;
+  q.y += c * im;
+  P[b + (size_t)(r * 3 + col) * vh] = q;
+  q = P[b + (size_t)(col * 3 + r) * vh];
+  q.x -= c * re;
+  q.y += c * im;
+  P[b + (size_t)(col * 3 + r) * vh] = q;
+}
+__device__ __forceinline__ void add_ta(double2* P, const Geom& g, const Site& x, int mu, const M3d& V, double c) {
+  const size_t b = link_base(g, x, mu), vh = (size_t)g.Vh;
+  ta_diag(P, b, vh, V.e[0].im, V.e[4].im, V.e[8].im, c);
 #pragma unroll
   for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int col = r + 1; col < 3; ++col) {
-      const C2d x1 = V.e[r * 3 + col], y1 = V.e[col * 3 + r];
-      const double re = 0.5 * (double)df_add_u(x1.re, -y1.re), im = 0.5 * (double)df_add_u(x1.im, y1.im);
-      double2 q = P[b + (size_t)(r * 3 + col) * vh];
-      q.x += c * re;
-      q.y += c * im;
-      P[b + (size_t)(r * 3 + col) * vh] = q;
-      q = P[b + (size_t)(col * 3 + r) * vh];
-      q.x -= c * re;
-      q.y += c * im;
-      P[b + (size_t)(col * 3 + r) * vh] = q;
-    }
+    for (int col = r + 1; col < 3; ++col) ta_pair(P, b, vh, r, col, V.e[r * 3 + col], V.e[col * 3 + r], c);
 }
 
 // P_mu(x) += c TA(U W), c = coeff beta / 3: the staple sum, U W and the anti-Hermitian
 // part in double-float from the copy Ud (FP32 pipes), only the accumulation into the FP64
-// momenta in FP64. All four directions in one launch (blockIdx.y = mu), one thread per
-// link, mu a run-time value so that the four share one instruction stream.
-// 2 CTAs per SM (254 registers, no spill): 3 (168 registers, a 68-byte spill) measured 3%
-// slower over a 16^3x32 HMC trajectory on GB300.
+// momenta in FP64. All four directions in one launch (blockIdx.y = mu), three threads per
+// link (one row each; row-split products in gauge_field.cuh), mu a run-time value so that
+// the four share one instruction stream. Bound by FP32 arithmetic, 18.5 k operations per
+// link: 385 us at 16^3x32 (25 T/s; the FMA pipe 65% busy, the rest of the issue slots going
+// to sign flips and lane packing) against 458 us with one thread per link at 254 registers,
+// 421 us of which was packed arithmetic alone. At 3 CTAs per SM 418 us.
 #ifndef LQCD_GF_MIN_BLOCKS
-#define LQCD_GF_MIN_BLOCKS 2
+#define LQCD_GF_MIN_BLOCKS 4
 #endif
-__global__ void __launch_bounds__(HMC_THREADS, LQCD_GF_MIN_BLOCKS) k_gauge_force(const float4* Ud, Geom g, double c, double2* P) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 2LL * g.Vh) return;
+__global__ void __launch_bounds__(SPLIT_THREADS, LQCD_GF_MIN_BLOCKS) k_gauge_force(const float4* Ud, Geom g, double c,
+                                                                                   double2* P) {
+  __shared__ SplitM sw, sv;
+  const int j = threadIdx.x % SPLIT_LINKS, i = threadIdx.x / SPLIT_LINKS;
   const int mu = blockIdx.y;
-  const Site x = site_of(g, (int)(i / g.Vh), (int)(i % g.Vh));
-  add_ta(P, g, x, mu, mul_d<false, false>(load_link_df(Ud, g, x, mu), staple_df(Ud, g, x, mu)), c);
+  // threads past the last link repeat it (they share barriers and rows) and store nothing
+  const long long at = (long long)blockIdx.x * SPLIT_LINKS + j, n = 2LL * g.Vh;
+  const bool live = at < n;
+  const long long l = live ? at : n - 1;
+  const int par = l >= g.Vh ? 1 : 0;
+  const Site x = site_of(g, par, (int)(l - (long long)par * g.Vh));
+  const size_t base = link_base(g, x, mu), vh = (size_t)g.Vh;
+  const RowD W = staple_row(Ud, g, x, mu, i);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) sw.put(i, q, j, W.e[q]);
+  __syncthreads();
+  const RowD V = split_row_times(Ud + base, vh, i, sw, j);  // V = U W
+#pragma unroll
+  for (int q = 0; q < 3; ++q) sv.put(i, q, j, V.e[q]);
+  __syncthreads();
+  if (!live) return;
+  // TA(V): thread 0 the diagonal, threads 1 and 2 the pairs of entries off it
+  auto entry = [&](int r, int q) { return c_unpack(sv.get(r, q, j)); };
+  if (i == 0) {
+    ta_diag(P, base, vh, entry(0, 0).im, entry(1, 1).im, entry(2, 2).im, c);
+  } else if (i == 1) {
+    ta_pair(P, base, vh, 0, 1, entry(0, 1), entry(1, 0), c);
+    ta_pair(P, base, vh, 0, 2, entry(0, 2), entry(2, 0), c);
+  } else {
+    ta_pair(P, base, vh, 1, 2, entry(1, 2), entry(2, 1), c);
+  }
 }
 
 // gamma_mu v on one colour's four spins in double-float (chiral basis, as in the Dslash:
@@ -106,12 +134,10 @@ __device__ __forceinline__ void gamma_mul_d(const C2d v[4], C2d o[4]) {
   }
 }
 
-// acc += a conj(b), unnormalised double-float
-__device__ __forceinline__ void cmacc_d(C2d& acc, const C2d& a, const C2d& b) {
-  df_mac_u(acc.re, a.re, b.re);
-  df_mac_u(acc.re, a.im, b.im);
-  df_mac_u(acc.im, a.im, b.re);
-  df_mac_u(acc.im, -a.re, b.im);
+// acc += a conj(b), unnormalised packed double-float (lanes re, im)
+__device__ __forceinline__ void cmacc_d(df64x2& acc, const C2d& a, const C2d& b) {
+  df2_mac_u(acc, c_pack(a), c_dup(b.re));
+  df2_mac_u(acc, df2_pack(a.im, -a.re), c_dup(b.im));
 }
 
 // P_mu(x) += c eta TA(U B), B = ((1 - g_mu) Phi(x+mu))^T conj(Psi(x)) + Psi(x+mu)^T conj((1 + g_mu) Phi(x)),
@@ -131,9 +157,9 @@ __global__ void __launch_bounds__(HMC_THREADS) k_fermion_force(const float4* Ud,
   const void* psi_x = par ? psi_o : psi_e;
   const void* phi_n = par ? phi_e : phi_o;
   const void* psi_n = par ? psi_e : psi_o;
-  M3d Bm;
+  df64x2 acc[9];
 #pragma unroll
-  for (int k = 0; k < 9; ++k) Bm.e[k] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
+  for (int k = 0; k < 9; ++k) acc[k] = c_zero();
   {
     df64 s[24];  // Psi(x)
     SpinorIO<P_DF64>::load(psi_x, g.Vh, h, s);
@@ -151,7 +177,7 @@ __global__ void __launch_bounds__(HMC_THREADS) k_fermion_force(const float4* Ud,
       for (int a = 0; a < 3; ++a)
 #pragma unroll
         for (int sp = 0; sp < 4; ++sp)
-          cmacc_d(Bm.e[b * 3 + a], v[sp], C2d{s[sidx(sp, a)], s[sidx(sp, a) + 1]});
+          cmacc_d(acc[b * 3 + a], v[sp], C2d{s[sidx(sp, a)], s[sidx(sp, a) + 1]});
     }
   }
   {
@@ -170,13 +196,14 @@ __global__ void __launch_bounds__(HMC_THREADS) k_fermion_force(const float4* Ud,
 #pragma unroll
         for (int sp = 0; sp < 4; ++sp) {
           const C2d w{df_add_u(v[sp].re, gv[sp].re), df_add_u(v[sp].im, gv[sp].im)};  // (1 + g_mu) Phi(x)
-          cmacc_d(Bm.e[a * 3 + b], C2d{t[2 * sp], t[2 * sp + 1]}, w);
+          cmacc_d(acc[a * 3 + b], C2d{t[2 * sp], t[2 * sp + 1]}, w);
         }
       }
     }
   }
+  M3d Bm;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) Bm.e[k] = {df_norm(Bm.e[k].re), df_norm(Bm.e[k].im)};
+  for (int k = 0; k < 9; ++k) Bm.e[k] = c_unpack(df2_norm(acc[k]));
   const double eta = (MU == 3 && x.c[3] == g.L[3] - 1) ? (double)g.t_bc : 1.0;
   add_ta(P, g, x, MU, mul_d<false, false>(load_link_df(Ud, g, x, MU), Bm), c * eta);
 }
@@ -204,7 +231,12 @@ __constant__ DFConst kInvFact[18] = {
 // product (X^2) for any degree. Everything runs on the FP32 pipes: P is split into
 // double-float pairs by integer operations, and the norm and the degree, which only need
 // to bound the Taylor tail, are taken in FP32 with a margin.
-__global__ void k_expm_update(double2* U, float4* Ud, Geom g, const double2* P, double eps, bool write_master) {
+// 128 registers, 4 CTAs per SM: 156 us at 16^3x32 (197 us in scalar arithmetic), 173 us at 3
+// CTAs per SM and 168 us at 5.
+#ifndef LQCD_EX_MIN_BLOCKS
+#define LQCD_EX_MIN_BLOCKS 4
+#endif
+__global__ void __launch_bounds__(HMC_THREADS, LQCD_EX_MIN_BLOCKS) k_expm_update(double2* U, float4* Ud, Geom g, const double2* P, double eps, bool write_master) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (par, mu, h)
   if (i >= 8LL * g.Vh) return;
   const int h = (int)(i % g.Vh);
@@ -340,9 +372,9 @@ int gauge_force_impl(const lqcd_gauge* g, double beta, double coeff, lqcd_mom* m
   const double c = coeff * beta / 3.0;
   float4* Ud = nullptr;
   LQCD_TRY(df_links(g, &Ud));
-  const unsigned nb = blocks(2LL * g->g.Vh, HMC_THREADS);
+  const unsigned nb = blocks(2LL * g->g.Vh, SPLIT_LINKS);
   cudaStream_t st = g->ctx->stream;
-  k_gauge_force<<<dim3(nb, 4), HMC_THREADS, 0, st>>>(Ud, g->g, c, m->d);
+  k_gauge_force<<<dim3(nb, 4), SPLIT_THREADS, 0, st>>>(Ud, g->g, c, m->d);
   g->ctx->launches++;
   LQCD_CK(cudaGetLastError());
   return LQCD_OK;
