@@ -488,7 +488,8 @@ typedef struct lqcd_tune_result {
   int ctas_per_sm;  /* chosen persistent grid, CTAs per SM (0: occupancy limit) */
   int form;         /* chosen kernel form: 0 one thread per site, 1 colour split (DF64),
                        2 shared-link multi-RHS, 3 one thread per site compiled for 8 CTAs
-                       per SM (FP32: 128 registers, more warps with fewer loads each) */
+                       per SM (FP32: 128 registers, more warps with fewer loads each; the
+                       FP32 default, but for twisted launches of more tiles than that) */
   int candidates;   /* configurations timed */
   double us_best;   /* per launch, chosen configuration */
   double us_default;/* per launch, untuned default (shared-link entries: the own-link launch) */

@@ -195,12 +195,13 @@ bool get_num(const JVal& o, const char* k, double& out) {
 }  // namespace
 
 TuneChoice tune_choice(int sp, int nr, int ntiles) {
-  TuneChoice c{0, dslash_colour_split(sp) ? 1 : 0};
+  TuneChoice c{0, default_dslash_form(sp), false};
   std::lock_guard<std::mutex> lk(g_mu);
   auto it = g_table.find({sp, nr, 0, bucket_of(ntiles)});
   if (it != g_table.end()) {
     c.ctas_per_sm = it->second.ctas_per_sm;
     c.form = it->second.form;
+    c.tuned = true;
   }
   return c;
 }
@@ -309,7 +310,7 @@ int lqcd_autotune_dslash(int n, const lqcd_gauge* const* g, int prec, int compre
   if (err == cudaSuccess) err = cudaEventCreate(&e0);
   if (err == cudaSuccess) err = cudaEventCreate(&e1);
   const int nsm = device_sm_count();
-  const int def_form = dslash_colour_split(prec) ? 1 : 0;
+  const int def_form = default_dslash_form(prec);
   // time `reps` launches of one configuration: best average of three trials (us)
   auto time_cfg = [&](const Launch& LL, int grid, int form, double* us) -> cudaError_t {
     cudaError_t e = cudaSuccess;
