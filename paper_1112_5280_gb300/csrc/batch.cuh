@@ -67,7 +67,8 @@ struct Scalars {
   int state, status, iter, maxiter, last, n_updates, restart_p;
   int normal;       // 1: solve Mhat^dag Mhat x = phi; converged on |phi - Mhat^dag Mhat x|
   unsigned ticket;  // k_finish groups done (reset by the last)
-  unsigned pad2[3];
+  int bad;          // FIN_ALPHA found the step impossible (ST_*); FIN_BETA stops the slot
+  unsigned pad2[2];
 };
 
 // One slot's operands for one batched kernel.
@@ -110,10 +111,17 @@ struct Launch {
                            // 2: shared-link multi-RHS Dslash (all slots on one gauge field):
                            //    tile t -> (slot group t % mrhs_groups, block t / mrhs_groups)
   double* partials;
-  int finish;              // 1: the slots' Works reduce or finish; k_finish follows the launch
+  int finish;              // 1: the slots' Works reduce or finish; k_finish follows the launch;
+                           // 2: they reduce, and the next launch finishes them (fin_works)
   int mrhs_group;          // interleave 2: slots per group (group g holds [g G, (g + 1) G))
   int mrhs_groups;         // interleave 2: number of slot groups
   int gated;               // 1: some slot runs only in a given solver state (Work::run_if >= 0)
+  // FIN_ALPHA of the launch before, run by the first nslots * fin_groups CTAs of this one
+  // (Dslash kernels; the step it belongs to needs alpha only two launches later)
+  const Work* fin_works;
+  int fin_groups;
+  // CUDA graph: the conditional node to enable when some slot waits for a reliable update
+  unsigned long long cond;
 };
 
 // Programmatic dependent launch. The batched kernels are launched with programmatic stream
@@ -132,9 +140,10 @@ __device__ __forceinline__ void pdl_entry() {
   pdl_wait();
   pdl_trigger();
 }
-// a persistent CTA about to take `tile`: its last one triggers the dependents
-__device__ __forceinline__ void pdl_last_tile(int tile, int ntiles) {
-  if (tile + (int)gridDim.x >= ntiles) pdl_trigger();
+// a persistent CTA about to take `tile` of a grid of `stride` CTAs: its last one triggers the
+// dependents
+__device__ __forceinline__ void pdl_last_tile(int tile, int ntiles, int stride) {
+  if (tile + stride >= ntiles) pdl_trigger();
 }
 
 __device__ __forceinline__ const Work& work_of(const Launch& L, int slot) {
@@ -275,6 +284,16 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 // The scalar programs. Run by one thread of k_finish for the slot.
 __device__ __noinline__ static void run_fin_bicg(const Work& w, const double* v);
 
+// alpha = <r,r> / <p, Mhat^dag Mhat p> = rr / |Mhat p|^2. This may run beside the next
+// Dslash launch, whose CTAs each read the slots' states: so it changes no state, and leaves
+// what it finds for FIN_BETA.
+__device__ __forceinline__ void fin_alpha(const Work& w, double sum) {
+  Scalars* s = w.sc;
+  s->qq = sum;
+  s->bad = !isfinite(sum) ? ST_NONFINITE : (!(sum > 0.0) ? ST_BREAKDOWN : ST_OK);
+  s->alpha = s->bad ? 0.0 : s->rr / sum;
+}
+
 __device__ __noinline__ static void run_fin(const Work& w, const double* v) {
   Scalars* s = w.sc;
   const double sum = v[0];
@@ -285,19 +304,15 @@ __device__ __noinline__ static void run_fin(const Work& w, const double* v) {
     case FIN_STORE1:
       s->res[1] = sum;
       break;
-    case FIN_ALPHA:  // alpha = <r,r> / <p, Mhat^dag Mhat p> = rr / |Mhat p|^2
-      s->qq = sum;
-      if (!isfinite(sum)) {
-        s->state = S_FAILED;
-        s->status = ST_NONFINITE;
-      } else if (!(sum > 0.0)) {
-        s->state = S_FAILED;
-        s->status = ST_BREAKDOWN;
-      } else {
-        s->alpha = s->rr / sum;
-      }
+    case FIN_ALPHA:
+      fin_alpha(w, sum);
       break;
     case FIN_BETA: {  // new |r|^2: beta, and whether to leave for a reliable update
+      if (s->bad) {
+        s->state = S_FAILED;
+        s->status = s->bad;
+        break;
+      }
       s->rr_prev = s->rr;
       s->rr = sum;
       s->iter += 1;
@@ -493,6 +508,112 @@ __device__ __forceinline__ double block_sum_f32(double v, double* sh) {
   }
   __syncthreads();
   return s;
+}
+
+// ------------------------------------------------------------------ reduction totals
+// A slot of n tiles is summed by G = finish_groups(n) CTAs, fixed by n alone, so the result
+// never depends on the batch or the grid: CTA q adds tiles [q c, (q + 1) c), c = ceil(n / G),
+// lane t of 256 taking tiles q c + t, q c + t + 256, ... in that order, then a fixed tree
+// (warps, then the eight warp sums in order). NT threads hold 256 / NT lanes each. With G > 1
+// the CTA's sum replaces its first partial, and the last CTA to finish (an atomic ticket on
+// Scalars::ticket after a fence) adds the G sums in order. True in the thread that holds the
+// slot's totals.
+constexpr int FINISH_LANES = 256;
+constexpr int FINISH_GROUPS = 16;     // most CTAs per slot
+constexpr int FINISH_TILES = 1024;    // tiles per CTA before a slot takes another CTA
+
+__host__ __device__ inline int finish_groups(int ntiles) {
+  const int g = (ntiles + FINISH_TILES - 1) / FINISH_TILES;
+  return g < 1 ? 1 : (g > FINISH_GROUPS ? FINISH_GROUPS : g);
+}
+
+// NS: sums per tile (1 or 3)
+template <int NT, int NS>
+__device__ __forceinline__ bool slot_totals(const Work& w, int q, double* partials, double tot[3]) {
+  static_assert(FINISH_LANES % NT == 0 || NT % FINISH_LANES == 0 || NT == 192, "lanes per thread");
+  constexpr int LPT = (FINISH_LANES + NT - 1) / NT;  // lanes per thread (NT 192: warps 0, 1 hold two)
+  __shared__ double sh[NS][FINISH_LANES / 32];
+  const int G = finish_groups(w.ntiles);
+  const int chunk = (w.ntiles + G - 1) / G;
+  const int lo = q * chunk, hi = min(w.ntiles, lo + chunk);
+  double* part = partials + 3 * (size_t)w.tile0;
+  constexpr int UNR = 4;
+#pragma unroll
+  for (int l = 0; l < LPT; ++l) {
+    const int lane = (int)threadIdx.x + l * NT;
+    if (lane >= FINISH_LANES) break;
+    double acc[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) acc[k] = 0.0;
+    for (int i0 = lo + lane; i0 < hi; i0 += UNR * FINISH_LANES) {
+      double x[UNR][NS];
+#pragma unroll
+      for (int u = 0; u < UNR; ++u) {
+        const int i = i0 + u * FINISH_LANES;
+        const double* src = part + 3 * (size_t)(i < hi ? i : lo);
+#pragma unroll
+        for (int k = 0; k < NS; ++k) x[u][k] = __ldcg(src + k);
+      }
+#pragma unroll
+      for (int u = 0; u < UNR; ++u)
+        if (i0 + u * FINISH_LANES < hi)
+#pragma unroll
+          for (int k = 0; k < NS; ++k) acc[k] += x[u][k];
+    }
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      double v = acc[k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if ((lane & 31) == 0) sh[k][lane >> 5] = v;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return false;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < FINISH_LANES / 32; ++i) s += sh[k][i];
+    tot[k] = s;
+  }
+  if (G == 1) return true;
+  if (lo < hi)
+#pragma unroll
+    for (int k = 0; k < NS; ++k) part[3 * (size_t)lo + k] = tot[k];
+  __threadfence();
+  if (atomicAdd(&w.sc->ticket, 1u) != (unsigned)G - 1) return false;
+  __threadfence();
+  for (int k = 0; k < NS; ++k) tot[k] = 0.0;
+  for (int g = 0; g < G; ++g) {
+    const int glo = g * chunk;
+    if (glo >= w.ntiles) break;
+    for (int k = 0; k < NS; ++k) tot[k] += __ldcg(part + 3 * (size_t)glo + k);
+  }
+  w.sc->ticket = 0;
+  return true;
+}
+
+// The first CTAs of a launch with fin_works: true in a CTA that was one of them (it is done).
+// Otherwise `block` and `stride` are the CTA's place among the launch's own.
+template <int NT, bool FINISHES>
+__device__ __forceinline__ bool finish_before(const Launch& L, int& block, int& stride) {
+  block = blockIdx.x;
+  stride = gridDim.x;
+  if (!FINISHES || !L.fin_works) return false;
+  const int n = L.nslots * L.fin_groups;
+  if (block >= n) {
+    block -= n;
+    stride -= n;
+    return false;
+  }
+  const Work& w = L.fin_works[block / L.fin_groups];
+  const int q = block % L.fin_groups;
+  if (q < finish_groups(w.ntiles) && slot_runs(w)) {
+    double tot[3];
+    if (slot_totals<NT, 1>(w, q, L.partials, tot)) fin_alpha(w, tot[0]);
+  }
+  return true;
 }
 
 // Called by all threads of the CTA after its tile: records the tile's partial sums

@@ -14,6 +14,8 @@ struct EpiTraits {
   static constexpr bool lin = (EPI == EPI_LIN || EPI == EPI_LIN_TW || EPI == EPI_PLAIN);
   static constexpr bool tw = (EPI == EPI_LIN_TW || EPI == EPI_CG_TW);
   static constexpr bool red = (EPI != EPI_PLAIN);
+  // the launch may finish the one before it (K3 of the CG: no reduction of its own)
+  static constexpr bool finishes = (EPI == EPI_PLAIN || EPI == EPI_LIN_TW);
 };
 
 // Occupancy target (CTAs of TILE threads per SM) of the Dslash: 6 leaves 168
@@ -152,13 +154,15 @@ __device__ __forceinline__ void dslash_epilogue(const Work& w, int h, typename S
     if (!EpiTraits<EPI>::red) {
     } else if (w.red == 1) {
       v0 = site_norm2(acc);
-    } else if (w.red == 2) {
-      R z[24];
-      SpinorIO<SP>::load(w.zin, w.g.Vh, h, z);
-      site_dot(z, acc, v0, v1);
-    } else if (w.red == 3) {  // <out, y1>, |out|^2
-      site_dot(acc, y, v0, v1);
-      v2 = site_norm2(acc);
+    } else if constexpr (SP != P_F16 && SP != P_BF16) {  // BiCGStab's, which no half precision runs
+      if (w.red == 2) {
+        R z[24];
+        SpinorIO<SP>::load(w.zin, w.g.Vh, h, z);
+        site_dot(z, acc, v0, v1);
+      } else if (w.red == 3) {  // <out, y1>, |out|^2
+        site_dot(acc, y, v0, v1);
+        v2 = site_norm2(acc);
+      }
     }
   } else {
     const R alpha = (R)w.sc->alpha;
@@ -210,20 +214,22 @@ __device__ __forceinline__ void dslash_tile(const Launch& L, int slot, int start
 template <int SP, int LP, int NR, bool DAG, int EPI, int MB = DslashMinBlocks<SP>::value>
 __global__ void __launch_bounds__(TILE, MB) k_dslash(const Launch L) {
   pdl_wait();
+  int block, stride;
+  if (finish_before<TILE, EpiTraits<EPI>::finishes>(L, block, stride)) return;
   if (single_slot_idle(L)) return;
   extern __shared__ int4 dyn_smem[];  // the slot view, launched with view_smem(L) bytes
   SlotView& sv = *reinterpret_cast<SlotView*>(dyn_smem);
   if (view_load(L, sv)) {
-    for (int tile = blockIdx.x; tile < sv.total; tile += gridDim.x) {
-      pdl_last_tile(tile, sv.total);
+    for (int tile = block; tile < sv.total; tile += stride) {
+      pdl_last_tile(tile, sv.total, stride);
       int slot, start;
       view_tile(L, sv, tile, slot, start);
       dslash_tile<SP, LP, NR, DAG, EPI>(L, slot, start);
     }
     return;
   }
-  for (int tile = blockIdx.x; tile < L.ntiles; tile += gridDim.x) {
-    pdl_last_tile(tile, L.ntiles);
+  for (int tile = block; tile < L.ntiles; tile += stride) {
+    pdl_last_tile(tile, L.ntiles, stride);
     int slot, start;
     tile_of(L, tile, slot, start);
     if (!slot_runs(work_of(L, slot))) continue;
@@ -316,6 +322,8 @@ struct MrhsPipe<8, D, SP, NR, DAG> {
 template <int SP, int LP, int NR, bool DAG, int EPI>
 __global__ void __launch_bounds__(TILE, Mrhs<NR>::MIN_BLOCKS) k_dslash_mrhs(const Launch L) {
   pdl_wait();
+  int cta, stride;
+  if (finish_before<TILE, EpiTraits<EPI>::finishes>(L, cta, stride)) return;
   static_assert(SP == P_F32 || SP == P_F16 || SP == P_BF16, "multi-RHS form: FP32 arithmetic");
   using IO = SpinorIO<SP>;
   constexpr int D = DslashDepth<SP>::value;
@@ -323,8 +331,8 @@ __global__ void __launch_bounds__(TILE, Mrhs<NR>::MIN_BLOCKS) k_dslash_mrhs(cons
   __shared__ SlotView sv;
   const bool view = view_load(L, sv);
   float4* s = su + threadIdx.x;
-  for (int tile = blockIdx.x; tile < L.ntiles; tile += gridDim.x) {
-    pdl_last_tile(tile, L.ntiles);
+  for (int tile = cta; tile < L.ntiles; tile += stride) {
+    pdl_last_tile(tile, L.ntiles, stride);
     const int group = tile % L.mrhs_groups;
     const int block = tile / L.mrhs_groups;
     const int s0 = group * L.mrhs_group;
@@ -399,14 +407,16 @@ __global__ void __launch_bounds__(3 * TILE, LQCD_DSLASH3_MIN_BLOCKS) k_dslash3(c
   using R = typename SpinorIO<SP>::Real;
   static_assert(SP == P_DF64 && LP == P_DF64, "the colour-split form is built for double-float");
   __shared__ ProjShare<TILE> sh;
+  int block, stride;
+  if (finish_before<3 * TILE, EpiTraits<EPI>::finishes>(L, block, stride)) return;
   if (single_slot_idle(L)) return;
   __shared__ SlotView sv;
   const bool view = view_load(L, sv);
   const int ntiles = view ? sv.total : L.ntiles;
   const int col = threadIdx.x / TILE;
   const int j = threadIdx.x - col * TILE;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    pdl_last_tile(tile, ntiles);
+  for (int tile = block; tile < ntiles; tile += stride) {
+    pdl_last_tile(tile, ntiles, stride);
     int slot, start;
     if (view) {
       view_tile(L, sv, tile, slot, start);
@@ -501,6 +511,14 @@ enum Blas {
   B_RDOT,         // Re <in, y1>
 };
 
+// The last launch of an iteration enables the graph's reliable-update node when some slot has
+// left for one (the default, set at each launch of the graph, is to skip it).
+__device__ __forceinline__ void request_update(const Launch& L) {
+  if (!L.cond || blockIdx.x != 0) return;
+  for (int i = threadIdx.x; i < L.nslots; i += TILE)
+    if (*((volatile int*)&work_of(L, i).sc->state) == S_UPDATE) cudaGraphSetConditional(L.cond, 1);
+}
+
 // out = x + c * y (complex c)
 template <typename R>
 __device__ __forceinline__ void caxpy(R* out, const R* x, R cr, R ci, const R* y) {
@@ -519,12 +537,13 @@ __global__ void __launch_bounds__(TILE) k_blas(const Launch L) {
   pdl_wait();
   using R = typename SpinorIO<SP>::Real;
   using TR = typename SpinorIO<TP>::Real;
+  if constexpr (OP == B_CG_P) request_update(L);
   if (single_slot_idle(L)) return;
   __shared__ SlotView sv;
   const bool view = view_load(L, sv);
   const int ntiles = view ? sv.total : L.ntiles;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    pdl_last_tile(tile, ntiles);
+    pdl_last_tile(tile, ntiles, gridDim.x);
     int slot, start;
     if (view) {
       view_tile(L, sv, tile, slot, start);

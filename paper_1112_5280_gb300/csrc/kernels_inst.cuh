@@ -17,6 +17,9 @@ namespace {
 constexpr int SPX = LQCD_SP;
 constexpr int LPX = (SPX == P_F64 || SPX == P_DF64 || SPX == P_F32) ? SPX : P_F16;
 
+// CTAs before the launch's own that finish the launch before it
+int fin_ctas(const Launch& L) { return L.fin_works ? L.nslots * L.fin_groups : 0; }
+
 template <int NR, bool DAG, int EPI>
 cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
   if (L.ntiles <= 0) return cudaSuccess;
@@ -40,7 +43,7 @@ cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
         tune_shared_links(SPX, NR, L.nslots, L.ntiles / L.mrhs_groups, &scps);
         grid = grid_for((const void*)fm, L.ntiles, 0, TILE, scps);
       }
-      return launch_k(fm, dim3(grid), dim3(TILE), 0, s, L);
+      return launch_k(fm, dim3(grid + fin_ctas(L)), dim3(TILE), 0, s, L);
     } else {
       return cudaErrorInvalidValue;
     }
@@ -53,20 +56,20 @@ cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
       // double-float: the colour-split form (latency bound at one thread per site)
       auto fn3 = k_dslash3<SPX, LPX, DAG, EPI>;
       if (grid <= 0) grid = grid_for((const void*)fn3, L.ntiles, 0, 3 * TILE, cps);
-      return launch_k(fn3, dim3(grid), dim3(3 * TILE), 0, s, L);
+      return launch_k(fn3, dim3(grid + fin_ctas(L)), dim3(3 * TILE), 0, s, L);
     }
   }
   if constexpr (SPX == P_F32) {
     if (form == 3) {  // the FP32 Dslash at the second register budget
       auto fh = k_dslash<SPX, LPX, NR, DAG, EPI, DSLASH_MIN_BLOCKS_HI>;
       if (grid <= 0) grid = grid_for((const void*)fh, L.ntiles, 0, TILE, cps);
-      return launch_k(fh, dim3(grid), dim3(TILE), view_smem(L), s, L);
+      return launch_k(fh, dim3(grid + fin_ctas(L)), dim3(TILE), view_smem(L), s, L);
     }
   }
   if constexpr (!split_only) {
     auto fn = k_dslash<SPX, LPX, NR, DAG, EPI>;
     if (grid <= 0) grid = grid_for((const void*)fn, L.ntiles, 0, TILE, cps);
-    return launch_k(fn, dim3(grid), dim3(TILE), view_smem(L), s, L);
+    return launch_k(fn, dim3(grid + fin_ctas(L)), dim3(TILE), view_smem(L), s, L);
   } else {
     return cudaErrorInvalidValue;
   }

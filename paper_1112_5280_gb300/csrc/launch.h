@@ -73,6 +73,15 @@ cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t dyn
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// The next launch of this thread is an ordinary one (true): programmatic dependence is
+// between kernels, and what it follows in a captured graph is another kind of node.
+void pdl_skip_next(bool skip);
+
+// Counts changes of what decides a launch's shape (tuner table, grid caps, kernel form): a
+// captured graph is good for as long as it stands.
+unsigned launch_config_epoch();
+void launch_config_changed();
+
 // Number of SMs of the current device and the persistent-grid multiplier.
 int device_sm_count();
 void set_grid_multiplier(int kernel_family, int mult);  // 0 = occupancy limit

@@ -3,6 +3,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <atomic>
 #include <cstdlib>
 #include <mutex>
 #include <unordered_map>
@@ -375,7 +376,7 @@ cudaError_t spinor_convert(const void* in, int pin, void* out, int pout, int Vh,
 
 // the slots' reduction totals and scalar finishers of the launch just issued on s
 static cudaError_t then_finish(cudaError_t err, const Launch& L, cudaStream_t s) {
-  if (err != cudaSuccess || !L.finish) return err;
+  if (err != cudaSuccess || L.finish != 1) return err;
   return launch_finish(L, s);
 }
 
@@ -413,7 +414,16 @@ PdlSolverScope::~PdlSolverScope() {
   if (off_) --t_solver_depth;
 }
 
+namespace {
+thread_local bool t_pdl_skip = false;  // the next launch depends on a node that is no kernel
+}
+void pdl_skip_next(bool skip) { t_pdl_skip = skip; }
+
 bool pdl_enabled() {
+  if (t_pdl_skip) {
+    t_pdl_skip = false;
+    return false;
+  }
   static const int mode = [] {
     const char* v = std::getenv("LQCD_PDL");
     if (!v || !v[0]) return -1;
@@ -465,7 +475,12 @@ int device_sm_count() {
   return g_nsm;
 }
 
+std::atomic<unsigned> g_config_epoch{0};
+unsigned launch_config_epoch() { return g_config_epoch.load(); }
+void launch_config_changed() { ++g_config_epoch; }
+
 void set_grid_multiplier(int family, int mult) {
+  launch_config_changed();
   if (family >= 0 && family < 4) g_mult[family] = mult;
 }
 
@@ -475,6 +490,7 @@ bool g_split[NPREC] = {false, false, false, false, true};
 
 bool dslash_colour_split(int prec) { return prec >= 0 && prec < NPREC && g_split[prec]; }
 void set_dslash_colour_split(int prec, bool on) {
+  launch_config_changed();
   if (prec >= 0 && prec < NPREC) g_split[prec] = on;
 }
 

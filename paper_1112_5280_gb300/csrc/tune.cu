@@ -427,6 +427,7 @@ int lqcd_autotune_dslash(int n, const lqcd_gauge* const* g, int prec, int compre
   {
     std::lock_guard<std::mutex> lk(g_mu);
     g_table[k0] = ent;
+    launch_config_changed();
     if (try_shared) g_table[ks] = sh;
   }
   if (out) {
@@ -453,6 +454,7 @@ int lqcd_tune_entries(lqcd_tune_result* out, int max, int* n) {
 void lqcd_tune_clear(void) {
   std::lock_guard<std::mutex> lk(g_mu);
   g_table.clear();
+  launch_config_changed();
 }
 
 int lqcd_tune_save(const char* path) {
@@ -526,6 +528,7 @@ int lqcd_tune_load(const char* path) {
   }
   std::lock_guard<std::mutex> lk(g_mu);
   for (auto& kv : add) g_table[kv.first] = kv.second;
+  launch_config_changed();
   return LQCD_OK;
 }
 
