@@ -2,6 +2,7 @@
 #include <cstdio>
 #include <cmath>
 #include <cstring>
+#include <set>
 #include <vector>
 
 #include "kernels.cuh"
@@ -692,6 +693,11 @@ int lqcd_dslash_batch_create(int n, const lqcd_gauge* const* g, const lqcd_field
   b->L.ntiles = prefix[n];
   b->L.interleave = (same_vh && n > 1) ? 1 : 0;
   b->L.partials = nullptr;  // no reduction
+  size_t link_bytes = 0;
+  std::set<const lqcd_gauge*> gauges;
+  for (int i = 0; i < n; ++i)
+    if (gauges.insert(g[i]).second) link_bytes += gauge_copy_bytes(link_prec_for(prec), nr, g[i]->g.Vh);
+  b->L.stream_links = stream_links((int)gauges.size(), link_bytes);
   if (n == 1) {
     b->L.works = nullptr;
     b->L.inline_work = w[0];

@@ -32,6 +32,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <set>
 #include <vector>
 
 #include "kernels.cuh"
@@ -126,6 +127,7 @@ struct lqcd_engine {
   bool dirty = true;
   int ntiles_total = 0;
   int interleave = 0;
+  int stream_links = 0;  // of the sloppy Dslash launches
   // shared-link multi-RHS Dslash for the sloppy steps (interleave mode 2): slots per group,
   // groups, and tiles (site blocks x groups); mrhs_groups == 0: not used
   int mrhs_group = 0, mrhs_groups = 0, mrhs_tiles = 0;
@@ -318,6 +320,7 @@ Launch batch_launch(const lqcd_engine* e, int s) {
   L.interleave = e->interleave;
   L.partials = e->d_partials;
   const StepKind k = kind_of(s);
+  if (k.dslash && !k.f64) L.stream_links = e->stream_links;
   if (e->mrhs_groups > 0 && k.dslash && !k.f64) {
     L.interleave = 2;
     L.ntiles = e->mrhs_tiles;
@@ -440,6 +443,13 @@ int rebuild(lqcd_engine* e) {
     else e->any_plain = true;
   }
   e->interleave = (same && n > 1) ? 1 : 0;
+  size_t link_bytes = 0;
+  std::set<const lqcd_gauge*> gauges;
+  for (long long id : e->active) {
+    const Request& q = e->reqs[id];
+    if (gauges.insert(q.gauge).second) link_bytes += gauge_copy_bytes(link_prec_for(e->sp), e->nr, q.g.Vh);
+  }
+  e->stream_links = stream_links((int)gauges.size(), link_bytes);
   // Slots on one gauge field may share each site block's link loads in the sloppy Dslash
   // steps (k_dslash_mrhs): a CTA applies the block's links to a group of slots. The group
   // size is the autotuner's measured choice for this key. Without one the slots load their

@@ -36,9 +36,12 @@ inline std::vector<int (*)(unsigned long long*)>& bounds_word_readers() {
 // (8 bytes, like FP64) and computes in double-float arithmetic (below).
 enum Prec { P_F64 = 0, P_F32 = 1, P_F16 = 2, P_BF16 = 3, P_DF64 = 4 };
 constexpr int NPREC = 5;  // number of storage precisions (size of per-precision tables)
+// FP32 links read past L1: the storage of P_F32 under another LinkIO (a template argument of
+// the kernels, never a field's precision)
+constexpr int P_F32_STREAM = NPREC;
 
-__host__ __device__ inline int prec_bytes(int p) {
-  return (p == P_F64 || p == P_DF64) ? 8 : (p == P_F32 ? 4 : 2);
+__host__ __device__ constexpr int prec_bytes(int p) {
+  return (p == P_F64 || p == P_DF64) ? 8 : ((p == P_F32 || p == P_F32_STREAM) ? 4 : 2);
 }
 
 // ------------------------------------------------------------------ double-float
@@ -274,8 +277,18 @@ struct BoundsWordRegistration {
 #endif
 
 // ------------------------------------------------------------------ raw loads
-// Read-only data is loaded through the non-coherent path. Links are read
-// exactly once per half-lattice sweep, so they bypass L1 allocation.
+// Read-only data is loaded through the non-coherent path. Each link word is read once per
+// half-lattice sweep. FP64-class links bypass L1; FP32 and FP16 links are
+// loaded through it: a warp whose neighbours start off a sector boundary shares its end
+// sectors with the next tile, and slots on one gauge field share whole words, so the L2 to L1
+// traffic, which bounds the launches whose data lies in L2, is smaller. Measured on GB300
+// against L1::no_allocate, per application: 16^3x32 FP32-18 8.6 -> 7.6 us, FP32-12 7.6 -> 7.1,
+// FP16-12 8.0 -> 7.3; 24^3x48, 12 sources, the whole FP32 solve 238 -> 217 ms; at 32^3x64,
+// where HBM bounds, FP32-12 96.4 -> 95.9, FP16-12 71.2 -> 71.3, FP32-18 121.4 -> 122.5.
+// L1::evict_first measured as no_allocate. Many different gauge fields in one launch, more
+// link bytes than L2 holds, are the exception: nothing is found again, and the links push
+// spinors out of L1 (18 mixed FP32 systems 57.7 -> 58.9 ms), so such FP32 launches keep
+// no_allocate (P_F32_STREAM, Launch::stream_links).
 
 __device__ __forceinline__ double2 ld_ro(const double2* p) { return __ldg(p); }
 __device__ __forceinline__ float4 ld_ro(const float4* p) { return __ldg(p); }
@@ -289,34 +302,17 @@ __device__ __forceinline__ double2 ld_stream(const double2* p) {
   asm volatile("ld.global.nc.L1::no_allocate.v2.f64 {%0,%1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
   return v;
 }
+__device__ __forceinline__ float2 ld_stream(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
 __device__ __forceinline__ float4 ld_stream(const float4* p) {
   float4 v;
   asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
                : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
   return v;
 }
-__device__ __forceinline__ float2 ld_stream(const float2* p) {
-  float2 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ uint4 ld_stream(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ uint2 ld_stream(const uint2* p) {
-  uint2 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ unsigned ld_stream(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
-  return v;
-}
-
 // half2 / bfloat162 packed in a 32-bit word
 __device__ __forceinline__ float2 unpack_h2(unsigned w) {
   __half2 h = *reinterpret_cast<__half2*>(&w);
@@ -576,7 +572,7 @@ struct SpinorIO<P_BF16> : SpinorIO16<true> {};
 template <int LP, int NR>
 struct LinkIO;
 
-// Raw words of one link (loaded once, bypassing L1) and their unpacking.
+// Raw words of one link and their unpacking.
 template <int NR>
 struct LinkIO<P_F64, NR> {
   using Real = double;
@@ -638,7 +634,7 @@ struct LinkIO<P_F32, 18> {
     h = LQCD_SITE(h, Vh);
     const float2* p = reinterpret_cast<const float2*>(base_mu) + h;
 #pragma unroll
-    for (int c = 0; c < NW; ++c) w[c] = ld_stream(p + (size_t)c * Vh);
+    for (int c = 0; c < NW; ++c) w[c] = ld_ro(p + (size_t)c * Vh);
   }
   __device__ static void unpack(const Word w[NW], float u[18]) {
 #pragma unroll
@@ -664,7 +660,7 @@ struct LinkIO<P_F32, 12> {
     h = LQCD_SITE(h, Vh);
     const float4* p = reinterpret_cast<const float4*>(base_mu) + h;
 #pragma unroll
-    for (int c = 0; c < NW; ++c) w[c] = ld_stream(p + (size_t)c * Vh);
+    for (int c = 0; c < NW; ++c) w[c] = ld_ro(p + (size_t)c * Vh);
   }
   __device__ static void unpack(const Word w[NW], float u[18]) {
 #pragma unroll
@@ -683,6 +679,18 @@ struct LinkIO<P_F32, 12> {
   }
 };
 
+template <int NR>
+struct LinkIO<P_F32_STREAM, NR> : LinkIO<P_F32, NR> {
+  using Word = typename LinkIO<P_F32, NR>::Word;
+  static constexpr int NW = LinkIO<P_F32, NR>::NW;
+  __device__ static void load_raw(const void* base_mu, int Vh, int h, Word w[NW]) {
+    h = LQCD_SITE(h, Vh);
+    const Word* p = reinterpret_cast<const Word*>(base_mu) + h;
+#pragma unroll
+    for (int c = 0; c < NW; ++c) w[c] = ld_stream(p + (size_t)c * Vh);
+  }
+};
+
 template <>
 struct LinkIO<P_F16, 18> {
   using Real = float;
@@ -692,7 +700,7 @@ struct LinkIO<P_F16, 18> {
     h = LQCD_SITE(h, Vh);
     const unsigned* p = reinterpret_cast<const unsigned*>(base_mu) + h;
 #pragma unroll
-    for (int c = 0; c < NW; ++c) w[c] = ld_stream(p + (size_t)c * Vh);
+    for (int c = 0; c < NW; ++c) w[c] = ld_ro(p + (size_t)c * Vh);
   }
   __device__ static void unpack(const Word w[NW], float u[18]) {
 #pragma unroll
@@ -719,7 +727,7 @@ struct LinkIO<P_F16, 12> {
     h = LQCD_SITE(h, Vh);
     const uint2* p = reinterpret_cast<const uint2*>(base_mu) + h;
 #pragma unroll
-    for (int c = 0; c < NW; ++c) w[c] = ld_stream(p + (size_t)c * Vh);
+    for (int c = 0; c < NW; ++c) w[c] = ld_ro(p + (size_t)c * Vh);
   }
   __device__ static void unpack(const Word w[NW], float u[18]) {
 #pragma unroll

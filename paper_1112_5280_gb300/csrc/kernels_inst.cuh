@@ -1,6 +1,10 @@
 // Instantiates the batched kernels for one spinor precision LQCD_SP with
 // launch-function suffix LQCD_SFX. Included by kernels_<prec>.cu.
 //
+// LQCD_STREAM_UNIT: this translation unit holds the FP32 Dslash with links read past L1
+// (launch_dslash_stream_<sfx>), to which the dispatcher of the LQCD_STREAM_EXTERN unit
+// forwards the launches with stream_links.
+//
 // LQCD_TW_UNIT: this translation unit holds only the twisted-mass Dslash epilogues
 // (launch_dslash_tw_<sfx>); LQCD_TW_EXTERN: the dispatcher of this unit forwards the
 // twisted epilogues to such a unit. Double-float uses the pair, so that its two
@@ -15,7 +19,11 @@ namespace lqcd {
 
 namespace {
 constexpr int SPX = LQCD_SP;
+#ifdef LQCD_STREAM_UNIT
+constexpr int LPX = P_F32_STREAM;
+#else
 constexpr int LPX = (SPX == P_F64 || SPX == P_DF64 || SPX == P_F32) ? SPX : P_F16;
+#endif
 
 // CTAs before the launch's own that finish the launch before it
 int fin_ctas(const Launch& L) { return L.fin_works ? L.nslots * L.fin_groups : 0; }
@@ -36,7 +44,7 @@ cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
   // shared-link multi-RHS launches (every slot on one gauge field): FP32-arithmetic
   // precisions, Wilson epilogues
   if (L.interleave == 2) {
-    if constexpr ((SPX == P_F32 || SPX == P_F16 || SPX == P_BF16) && !EpiTraits<EPI>::tw) {
+    if constexpr (LPX != P_F32_STREAM && (SPX == P_F32 || SPX == P_F16 || SPX == P_BF16) && !EpiTraits<EPI>::tw) {
       auto fm = k_dslash_mrhs<SPX, LPX, NR, DAG, EPI>;
       if (grid <= 0) {
         int scps = 0;
@@ -85,6 +93,7 @@ cudaError_t dispatch_tw(bool dag, int epi, const Launch& L, int grid, cudaStream
   return cudaErrorInvalidValue;
 }
 
+#ifndef LQCD_STREAM_UNIT
 template <int OP, int P, int TP = P_F64>
 cudaError_t go_blas(const Launch& L, int grid, cudaStream_t s) {
   auto fn = k_blas<P, OP, TP>;
@@ -92,6 +101,7 @@ cudaError_t go_blas(const Launch& L, int grid, cudaStream_t s) {
   if (grid <= 0) grid = grid_for((const void*)fn, L.ntiles, 1, TILE);
   return launch_k(fn, dim3(grid), dim3(TILE), 0, s, L);
 }
+#endif
 }  // namespace
 
 #ifdef LQCD_TW_UNIT
@@ -141,11 +151,29 @@ cudaError_t dispatch_12(bool dag, int epi, const Launch& L, int grid, cudaStream
 }
 }  // namespace
 
+#ifdef LQCD_STREAM_UNIT
+
+cudaError_t LQCD_CAT(launch_dslash_stream_, LQCD_SFX)(int nr, bool dag, int epi, const Launch& L,
+                                                       int grid, cudaStream_t s, int form) {
+  return nr == 18 ? dispatch_nr<18>(dag, epi, L, grid, s, form) : dispatch_nr<12>(dag, epi, L, grid, s, form);
+}
+
+#else
+
+#ifdef LQCD_STREAM_EXTERN
+cudaError_t LQCD_CAT(launch_dslash_stream_, LQCD_SFX)(int nr, bool dag, int epi, const Launch& L,
+                                                       int grid, cudaStream_t s, int form);
+#endif
+
 cudaError_t LQCD_CAT(launch_dslash_, LQCD_SFX)(int nr, bool dag, int epi, const Launch& L,
                                                 int grid, cudaStream_t s, int form) {
   // a twisted single-slot work needs the twisted epilogue (a batched launch's works live
   // on the device; their callers pick the epilogue from the slots they hold)
   if (!L.works && L.inline_work.twist && epi != EPI_LIN_TW && epi != EPI_CG_TW) return cudaErrorInvalidValue;
+#ifdef LQCD_STREAM_EXTERN
+  if (L.stream_links && (nr == 18 || nr == 12))
+    return LQCD_CAT(launch_dslash_stream_, LQCD_SFX)(nr, dag, epi, L, grid, s, form);
+#endif
   if (nr == 18) return dispatch_nr<18>(dag, epi, L, grid, s, form);
   if (nr == 12) return dispatch_12<SPX>(dag, epi, L, grid, s, form);
   return cudaErrorInvalidValue;
@@ -231,6 +259,7 @@ cudaError_t LQCD_CAT(launch_blas_, LQCD_SFX)(int op, int tp, const Launch& L, in
   }
 }
 
+#endif  // LQCD_STREAM_UNIT
 #endif  // LQCD_TW_UNIT
 
 }  // namespace lqcd

@@ -77,6 +77,10 @@ cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t dyn
 // between kernels, and what it follows in a captured graph is another kind of node.
 void pdl_skip_next(bool skip);
 
+// Launch::stream_links: the slots' link copies (bytes in all, over `gauges` different gauge
+// fields) are more than half of L2 (126 MB), which the launch's spinors share.
+inline int stream_links(int gauges, size_t link_bytes) { return gauges > 1 && link_bytes > ((size_t)64 << 20); }
+
 // Counts changes of what decides a launch's shape (tuner table, grid caps, kernel form): a
 // captured graph is good for as long as it stands.
 unsigned launch_config_epoch();
