@@ -84,10 +84,10 @@ template <typename R>
 __device__ __forceinline__ Cx<R> sp(const R* v, int spin, int col) {
   return {v[sidx(spin, col)], v[sidx(spin, col) + 1]};
 }
-template <typename R>
+template <bool FIRST, typename R>
 __device__ __forceinline__ void acc_add(R* a, int spin, int col, Cx<R> w) {
-  a[sidx(spin, col)] = f_add(a[sidx(spin, col)], w.re);
-  a[sidx(spin, col) + 1] = f_add(a[sidx(spin, col) + 1], w.im);
+  a[sidx(spin, col)] = FIRST ? w.re : f_add(a[sidx(spin, col)], w.re);
+  a[sidx(spin, col) + 1] = FIRST ? w.im : f_add(a[sidx(spin, col) + 1], w.im);
 }
 // i * w
 template <typename R>
@@ -173,8 +173,18 @@ __device__ __forceinline__ void project_h2(const uint4 w[3], int eta, Cx<float> 
   }
 }
 
-// The rest of a hop: acc += (U or U^dag) h, lifted back to four spins by (1 + S g_MU).
-template <int MU, int S, bool ADJ, typename R>
+// Whether the first hop of a site sets the accumulators instead of adding to zeros: where the
+// arithmetic bounds (FP64: 24 of 888 operations per site, 130.7 -> 128.0 us at 16^3x32). In
+// FP32 the accumulators' longer life in the compiler's schedule cost spills (FP16 at 32^3x64
+// 71.2 -> 72.4 us).
+template <int SP>
+struct FirstSets {
+  static constexpr bool value = SP == P_F64 || SP == P_DF64;
+};
+
+// The rest of a hop: acc += (U or U^dag) h, lifted back to four spins by (1 + S g_MU); FIRST:
+// acc = that.
+template <int MU, int S, bool ADJ, bool FIRST, typename R>
 __device__ __forceinline__ void hop_half(const Cx<R> h0[3], const Cx<R> h1[3], const R u[18], R acc[24]) {
   // w = U h (or U^dag h) per spin row: for each product u h, re += u.re h.re - u.im h.im and
   // im += u.re h.im + u.im h.re, as four multiply-adds in this order
@@ -201,47 +211,47 @@ __device__ __forceinline__ void hop_half(const Cx<R> h0[3], const Cx<R> h1[3], c
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    acc_add(acc, 0, a, w0[a]);
-    acc_add(acc, 1, a, w1[a]);
+    acc_add<FIRST>(acc, 0, a, w0[a]);
+    acc_add<FIRST>(acc, 1, a, w1[a]);
     if (MU == 0) {  // lower = S A^dag h, A^dag = [[0,i],[i,0]]
-      acc_add(acc, 2, a, sgn<S>(mul_i(w1[a])));
-      acc_add(acc, 3, a, sgn<S>(mul_i(w0[a])));
+      acc_add<FIRST>(acc, 2, a, sgn<S>(mul_i(w1[a])));
+      acc_add<FIRST>(acc, 3, a, sgn<S>(mul_i(w0[a])));
     } else if (MU == 1) {  // A^dag = [[0,1],[-1,0]]
-      acc_add(acc, 2, a, sgn<S>(w1[a]));
-      acc_add(acc, 3, a, sgn<-S>(w0[a]));
+      acc_add<FIRST>(acc, 2, a, sgn<S>(w1[a]));
+      acc_add<FIRST>(acc, 3, a, sgn<-S>(w0[a]));
     } else if (MU == 2) {  // A^dag = diag(i, -i)
-      acc_add(acc, 2, a, sgn<S>(mul_i(w0[a])));
-      acc_add(acc, 3, a, sgn<-S>(mul_i(w1[a])));
+      acc_add<FIRST>(acc, 2, a, sgn<S>(mul_i(w0[a])));
+      acc_add<FIRST>(acc, 3, a, sgn<-S>(mul_i(w1[a])));
     } else {
-      acc_add(acc, 2, a, sgn<S>(w0[a]));
-      acc_add(acc, 3, a, sgn<S>(w1[a]));
+      acc_add<FIRST>(acc, 2, a, sgn<S>(w0[a]));
+      acc_add<FIRST>(acc, 3, a, sgn<S>(w1[a]));
     }
   }
 }
 
 // One hop: acc += eta * (1 + S g_MU) (U or U^dag) psi, eta = +-1.
-template <int MU, int S, bool ADJ, typename R>
+template <int MU, int S, bool ADJ, bool FIRST, typename R>
 __device__ __forceinline__ void hop(const R psi[24], const R u[18], int eta, R acc[24]) {
   Cx<R> h0[3], h1[3];
   project<MU, S>(psi, eta, h0, h1);
-  hop_half<MU, S, ADJ>(h0, h1, u, acc);
+  hop_half<MU, S, ADJ, FIRST>(h0, h1, u, acc);
 }
 
 // One hop from the raw storage words of the neighbour spinor: FP16 spinors are projected in
 // half2 before conversion, every other precision is unpacked and projected in its arithmetic
 // type. Every Dslash form calls this, so a site's arithmetic is the same in all of them.
-template <int MU, int S, bool ADJ, int SP>
+template <int MU, int S, bool ADJ, bool FIRST, int SP>
 __device__ __forceinline__ void hop_words(const typename SpinorIO<SP>::Word w[SpinorIO<SP>::NW],
                                           const typename SpinorIO<SP>::Real u[18], int eta,
                                           typename SpinorIO<SP>::Real acc[24]) {
   if constexpr (SP == P_F16) {
     Cx<float> h0[3], h1[3];
     project_h2<MU, S>(w, eta, h0, h1);
-    hop_half<MU, S, ADJ>(h0, h1, u, acc);
+    hop_half<MU, S, ADJ, FIRST>(h0, h1, u, acc);
   } else {
     typename SpinorIO<SP>::Real psi[24];
     SpinorIO<SP>::unpack(w, psi);
-    hop<MU, S, ADJ>(psi, u, eta, acc);
+    hop<MU, S, ADJ, FIRST>(psi, u, eta, acc);
   }
 }
 
@@ -301,7 +311,7 @@ __device__ __forceinline__ void compute_hop(const Geom& g, int t, const HopBuf<S
   // backward: U_mu(x - mu)^dag psi(x - mu), projector (1 + g) for D, (1 - g) for D^dag
   const int eta = (MU == 3 && t == (FWD ? g.L[3] - 1 : 0)) ? g.t_bc : 1;
   constexpr int S = FWD ? (DAG ? 1 : -1) : (DAG ? -1 : 1);
-  hop_words<MU, S, !FWD, SP>(b.s, u, eta, acc);
+  hop_words<MU, S, !FWD, K == 0 && FirstSets<SP>::value, SP>(b.s, u, eta, acc);
 }
 
 template <int K, int D, int SP, int LP, int NR, bool DAG>
@@ -348,8 +358,10 @@ __device__ __forceinline__ void dslash_site(const Geom& g, int h, int out_par, c
   constexpr int D = DslashDepth<SP>::value;
   HopBuf<SP, LP, NR> b[D];
   HopPrologue<0, D, SP, LP, NR>::run(g, h, nf, nb, in, Uout, Uin, b);
+  if (!FirstSets<SP>::value) {
 #pragma unroll
-  for (int i = 0; i < 24; ++i) acc[i] = 0;
+    for (int i = 0; i < 24; ++i) acc[i] = 0;
+  }
   HopPipe<0, D, SP, LP, NR, DAG>::run(g, h, t, nf, nb, in, Uout, Uin, b, acc);
 }
 
@@ -370,11 +382,12 @@ __device__ __forceinline__ void dslash_site(const Geom& g, int h, int out_par, c
 // lattice pass a clamped site and discard the result.
 //
 // The arithmetic is packed (field.cuh): the lanes are the two spin rows of h, which meet the
-// same link entry. Bound by the FP32 pipe (9482 operations per site; the pipe's rate in long
-// chains of these operations is 31 T/s, 0.10 ms at 24^3x48) and by the latency of the loads
-// before each barrier. Scalar arithmetic with one barrier per hop took 174.7 us per
+// same link entry. Bound by the FP32 pipe (9482 operations per site in scalar form; the pipe's
+// rate in long chains of these operations is 31 T/s, 0.10 ms at 24^3x48) and by the latency of
+// the loads before each barrier. Scalar arithmetic with one barrier per hop took 174.7 us per
 // application at 24^3x48 and 531 at 32^3x64; packed 145.9 and 475; with a direction's two
-// hops on one barrier 144.4 and 464 (39.4, 36.7 and 36.1 us at 16^3x32). Staging the next
+// hops on one barrier 144.4 and 464 (39.4, 36.7 and 36.1 us at 16^3x32); with a product
+// started as one instead of added to zero 138.0 at 24^3x48 (34.9 at 16^3x32). Staging the next
 // hop's words in shared memory with cp.async measured slower than plain loads (158 us at
 // 24^3x48), and so did 3 or 5 CTAs per SM (152 and 178 us against 144 at 4).
 
@@ -387,10 +400,7 @@ struct ProjShare {
 
 // S a on both lanes
 template <int S>
-__device__ __forceinline__ df64x2 df2_sgn(df64x2 a) {
-  if (S > 0) return a;
-  return {p_neg(a.hi), p_neg(a.lo)};
-}
+__device__ __forceinline__ df64x2 df2_sgn(df64x2 a) { return S > 0 ? a : df2_neg(a); }
 // (S a, -S b) of the lanes (a, b)
 template <int S>
 __device__ __forceinline__ f32x2 p_alt(f32x2 v) {
@@ -434,23 +444,34 @@ __device__ __forceinline__ void project3(const float4 d[4], df64x2& hr, df64x2& 
 }
 
 // acc += (1 + S g_MU) applied to the link row u times the published h, times eta = +-1
-template <int MU, int S, bool ADJ, int NT>
+// (FIRST: acc = that)
+template <int MU, int S, bool ADJ, bool FIRST, int NT>
 __device__ __forceinline__ void hop3_mac(const float4 u[3], const ulonglong2 (&buf)[3][2][NT], int j, int eta, Acc3& acc) {
-  df64x2 wr{0ull, 0ull}, wi{0ull, 0ull};  // lanes (w0, w1)
+  df64x2 wr, wi;  // lanes (w0, w1)
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
     const ulonglong2 a = buf[b][0][j], c = buf[b][1][j];
     const df64x2 hr{a.x, a.y}, hi{c.x, c.y};
     const df64 r(u[b].x, u[b].y), i = ADJ ? df64(-u[b].z, -u[b].w) : df64(u[b].z, u[b].w);
     const df64x2 rr = df2_pack(r, r), ri = df2_pack(i, i);
-    df2_mac_u(wr, rr, hr);
+    if (b == 0) {
+      wr = df2_mul_u(rr, hr);
+      wi = df2_mul_u(rr, hi);
+    } else {
+      df2_mac_u(wr, rr, hr);
+      df2_mac_u(wi, rr, hi);
+    }
     df2_mac_u(wr, df2_sgn<-1>(ri), hi);
-    df2_mac_u(wi, rr, hi);
     df2_mac_u(wi, ri, hr);
   }
   if (MU == 3 && eta < 0) {
     wr = df2_sgn<-1>(wr);
     wi = df2_sgn<-1>(wi);
+  }
+  if (FIRST) {
+    static_assert(!FIRST || MU == 0, "the first hop is an x hop");
+    acc = {wr, wi, df2_sgn<-S>(wi), df2_sgn<S>(wr)};
+    return;
   }
   acc.up_re = df2_add_u(acc.up_re, wr);
   acc.up_im = df2_add_u(acc.up_im, wi);
@@ -500,29 +521,31 @@ __device__ __forceinline__ void hops3s_df(const Geom& g, int h, const int nf[4],
     buf[1][col][1][j] = make_ulonglong2(hi.hi, hi.lo);
   }
   __syncthreads();
-  hop3_mac<MU, SF, false, NT>(uf, buf[0], j, (MU == 3 && t == g.L[3] - 1) ? g.t_bc : 1, acc);
-  hop3_mac<MU, -SF, true, NT>(ub, buf[1], j, (MU == 3 && t == 0) ? g.t_bc : 1, acc);
+  hop3_mac<MU, SF, false, MU == 0, NT>(uf, buf[0], j, (MU == 3 && t == g.L[3] - 1) ? g.t_bc : 1, acc);
+  hop3_mac<MU, -SF, true, false, NT>(ub, buf[1], j, (MU == 3 && t == 0) ? g.t_bc : 1, acc);
 }
+
+// the four spins of one colour: lanes (0, 1) in [0] and (2, 3) in [1]
+struct Spins4 {
+  df64x2 re[2], im[2];
+};
 
 // acc = colour col of (D_{p,1-p} in)(h) in double-float, 18-real double-float links; all
 // 3 NT threads of the CTA call it together (thread j of colour col: site h)
 template <int LP, bool DAG, int NT>
 __device__ __forceinline__ void dslash_site3s_df(const Geom& g, int h, int out_par, const void* in,
                                                  const void* Uout, const void* Uin, int col, int j,
-                                                 df64 acc[8], ProjShare<NT>& sh) {
+                                                 Spins4& acc, ProjShare<NT>& sh) {
   int nf[4], nb[4], t;
   neighbours(g, h, out_par, nf, nb, t);
-  Acc3 s{{0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}};
+  Acc3 s;
   hops3s_df<0, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, s, sh);
   hops3s_df<1, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, s, sh);
   s.low_re = {p_swap(s.low_re.hi), p_swap(s.low_re.lo)};
   s.low_im = {p_swap(s.low_im.hi), p_swap(s.low_im.lo)};
   hops3s_df<2, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, s, sh);
   hops3s_df<3, LP, DAG, NT>(g, h, nf, nb, t, in, Uout, Uin, col, j, s, sh);
-  df2_unpack(df2_norm(s.up_re), acc[0], acc[2]);
-  df2_unpack(df2_norm(s.up_im), acc[1], acc[3]);
-  df2_unpack(df2_norm(s.low_re), acc[4], acc[6]);
-  df2_unpack(df2_norm(s.low_im), acc[5], acc[7]);
+  acc = {{df2_norm(s.up_re), df2_norm(s.low_re)}, {df2_norm(s.up_im), df2_norm(s.low_im)}};
 }
 
 }  // namespace lqcd

@@ -185,11 +185,27 @@ __device__ __forceinline__ void df2_mac_u(df64x2& acc, df64x2 a, df64x2 b) {
   acc.hi = s;
   acc.lo = p_add(acc.lo, p_add(e, pe));
 }
+// a b, the value that df2_mac_u leaves in an accumulator of zero: 4 operations instead of 12
+__device__ __forceinline__ df64x2 df2_mul_u(df64x2 a, df64x2 b) {
+  const f32x2 p = p_mul(a.hi, b.hi);
+  f32x2 pe = p_fma(a.hi, b.hi, p_neg(p));
+  pe = p_fma(a.hi, b.lo, p_fma(a.lo, b.hi, pe));
+  return {p, pe};
+}
 __device__ __forceinline__ df64x2 df2_norm(df64x2 a) {
   const f32x2 s = p_add(a.hi, a.lo);
   const f32x2 v = p_sub(s, a.hi);
   return {s, p_add(p_sub(a.hi, p_sub(s, v)), p_sub(a.lo, v))};
 }
+
+// df64's +, - and * on both lanes
+__device__ __forceinline__ df64x2 df2_renorm(df64x2 a) {
+  const f32x2 h = p_add(a.hi, a.lo);
+  return {h, p_sub(a.lo, p_sub(h, a.hi))};
+}
+__device__ __forceinline__ df64x2 df2_neg(df64x2 a) { return {p_neg(a.hi), p_neg(a.lo)}; }
+__device__ __forceinline__ df64x2 df2_add(df64x2 a, df64x2 b) { return df2_renorm(df2_add_u(a, b)); }
+__device__ __forceinline__ df64x2 df2_mul(df64x2 a, df64x2 b) { return df2_renorm(df2_mul_u(a, b)); }
 
 // Arithmetic with a fixed rounding sequence. nvcc fuses a * b + c into one FMA where it
 // sees fit, and the same source inlined into two different kernels may be fused in two

@@ -133,15 +133,18 @@ __device__ __forceinline__ C2d c_unpack(df64x2 v) {
   return r;
 }
 __device__ __forceinline__ df64x2 c_zero() { return {0ull, 0ull}; }
+__device__ __forceinline__ df64x2 c_mul(const C2d& x, const C2d& y) {  // x y
+  df64x2 s = df2_mul_u(c_dup(x.re), c_pack(y));
+  df2_mac_u(s, c_dup(x.im), c_rot(y));
+  return s;
+}
 __device__ __forceinline__ void c_mac(df64x2& acc, const C2d& x, const C2d& y) {  // acc += x y
   df2_mac_u(acc, c_dup(x.re), c_pack(y));
   df2_mac_u(acc, c_dup(x.im), c_rot(y));
 }
 
 __device__ __forceinline__ C2d cmul_d(const C2d& a, const C2d& b) {
-  df64x2 s = c_zero();
-  c_mac(s, a, b);
-  return c_unpack(df2_norm(s));
+  return c_unpack(df2_norm(c_mul(a, b)));
 }
 __device__ __forceinline__ C2d cadd_d(const C2d& a, const C2d& b) {
   return c_unpack(df2_norm(df2_add_u(c_pack(a), c_pack(b))));
@@ -151,8 +154,7 @@ __device__ __forceinline__ C2d cscale_d(df64 f, const C2d& a) { return {f * a.re
 
 // a x + b y in double-float
 __device__ __forceinline__ C2d cmix_d(const C2d& a, const C2d& x, const C2d& b, const C2d& y) {
-  df64x2 s = c_zero();
-  c_mac(s, a, x);
+  df64x2 s = c_mul(a, x);
   c_mac(s, b, y);
   return c_unpack(df2_norm(s));
 }
@@ -169,13 +171,11 @@ __device__ __forceinline__ df64 df_rsqrt(df64 n) {
   return y;
 }
 
-// w += op(a) op(b) with op the adjoint where asked: each entry accumulates unnormalised
-// over k and is normalised once. Per k, an entry of b serves the three rows i at once.
+// op(a) op(b) with op the adjoint where asked: each entry accumulates unnormalised over k and
+// is normalised once. Per k, an entry of b serves the three rows i at once.
 template <bool DAGA, bool DAGB>
-__device__ __forceinline__ void mac_d(M3d& w, const M3d& a, const M3d& b) {
+__device__ __forceinline__ M3d mul_d(const M3d& a, const M3d& b) {
   df64x2 s[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) s[i] = c_pack(w.e[i]);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     df64x2 xr[3], xi[3];
@@ -192,22 +192,15 @@ __device__ __forceinline__ void mac_d(M3d& w, const M3d& a, const M3d& b) {
       const df64x2 yp = c_pack(y), yr = c_rot(y);
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        df2_mac_u(s[i * 3 + j], xr[i], yp);
+        if (k == 0) s[i * 3 + j] = df2_mul_u(xr[i], yp);
+        else df2_mac_u(s[i * 3 + j], xr[i], yp);
         df2_mac_u(s[i * 3 + j], xi[i], yr);
       }
     }
   }
-#pragma unroll
-  for (int i = 0; i < 9; ++i) w.e[i] = c_unpack(df2_norm(s[i]));
-}
-
-// op(a) op(b)
-template <bool DAGA, bool DAGB>
-__device__ __forceinline__ M3d mul_d(const M3d& a, const M3d& b) {
   M3d c;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) c.e[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
-  mac_d<DAGA, DAGB>(c, a, b);
+  for (int i = 0; i < 9; ++i) c.e[i] = c_unpack(df2_norm(s[i]));
   return c;
 }
 
@@ -231,7 +224,7 @@ __device__ __forceinline__ Site shifted_rt(const Geom& g, Site s, int nu, int d)
 // arithmetic, and a thread needs a third of the accumulators: 24 warps per SM can be
 // resident where one thread per link took 254 registers (8 warps), which left the loads and
 // the chains of dependent operations uncovered (FMA pipe 60% busy). Entries are packed
-// (lanes re, im), each accumulated in the same order as in mac_d.
+// (lanes re, im), each accumulated in the same order as in mul_d.
 struct RowD {
   df64x2 e[3];
 };
@@ -290,11 +283,12 @@ __device__ __forceinline__ RowD staple_row(const float4* Ud, const Geom& g, cons
       for (int k = 0; k < 3; ++k) c_dups(c_entry(a[k * a_step], flip_a), xr[k], xi[k]);
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        df64x2 s = c_zero();
+        df64x2 s;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
           const df64x2 y = c_entry(b[(size_t)(3 * j + k) * vh], 0x80000000u);
-          df2_mac_u(s, xr[k], y);
+          if (k == 0) s = df2_mul_u(xr[k], y);
+          else df2_mac_u(s, xr[k], y);
           df2_mac_u(s, xi[k], c_times_i(y));
         }
         T.e[j] = df2_norm(s);
@@ -331,15 +325,14 @@ struct SplitM {
 __device__ __forceinline__ RowD split_row_times(const float4* u, size_t vh, int i, const SplitM& w, int j) {
   RowD r;
 #pragma unroll
-  for (int q = 0; q < 3; ++q) r.e[q] = c_zero();
-#pragma unroll
   for (int k = 0; k < 3; ++k) {
     df64x2 xr, xi;
     c_dups(c_entry(u[(size_t)(3 * i + k) * vh], 0u), xr, xi);
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       const df64x2 y = w.get(k, q, j);
-      df2_mac_u(r.e[q], xr, y);
+      if (k == 0) r.e[q] = df2_mul_u(xr, y);
+      else df2_mac_u(r.e[q], xr, y);
       df2_mac_u(r.e[q], xi, c_times_i(y));
     }
   }

@@ -140,7 +140,7 @@ __device__ __noinline__ bool su2_draw(double alpha, uint64_t seed, uint64_t c0, 
 // k_heatbath_v: V = U W of every link of the class, three threads per link (row-split
 // products in gauge_field.cuh), FP32 bound like the gauge force. V [word][V/2] stays in L2.
 // k_heatbath: the three subgroups, one thread per link, FP64 bound (about 200 FP64
-// instructions per draw). At 24^3x48, beta 6, a sweep takes 5.83 ms; as one kernel with one
+// instructions per draw). At 24^3x48, beta 6, a sweep takes 5.74 ms; as one kernel with one
 // thread per link (168 registers, staple code and draws sharing 12 warps per SM) 6.63 ms, and
 // as one kernel with three threads per link, where two thirds of the CTA wait at a barrier
 // during the draws, 6.27 ms.

@@ -77,7 +77,7 @@ __device__ __forceinline__ void add_ta(double2* P, const Geom& g, const Site& x,
 // momenta in FP64. All four directions in one launch (blockIdx.y = mu), three threads per
 // link (one row each; row-split products in gauge_field.cuh), mu a run-time value so that
 // the four share one instruction stream. Bound by FP32 arithmetic, 18.5 k operations per
-// link: 385 us at 16^3x32 (25 T/s; the FMA pipe 65% busy, the rest of the issue slots going
+// link: 375 us at 16^3x32 (25 T/s; the FMA pipe 65% busy, the rest of the issue slots going
 // to sign flips and lane packing) against 458 us with one thread per link at 254 registers,
 // 421 us of which was packed arithmetic alone. At 3 CTAs per SM 418 us.
 #ifndef LQCD_GF_MIN_BLOCKS
@@ -231,7 +231,7 @@ __constant__ DFConst kInvFact[18] = {
 // product (X^2) for any degree. Everything runs on the FP32 pipes: P is split into
 // double-float pairs by integer operations, and the norm and the degree, which only need
 // to bound the Taylor tail, are taken in FP32 with a margin.
-// 128 registers, 4 CTAs per SM: 156 us at 16^3x32 (197 us in scalar arithmetic), 173 us at 3
+// 128 registers, 4 CTAs per SM: 149 us at 16^3x32 (197 us in scalar arithmetic), 173 us at 3
 // CTAs per SM and 168 us at 5.
 #ifndef LQCD_EX_MIN_BLOCKS
 #define LQCD_EX_MIN_BLOCKS 4

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "batch.cuh"
+#include "convert.cuh"
 
 namespace lqcd {
 
@@ -101,19 +102,6 @@ __device__ __forceinline__ void twist24(R v[24], double sd, double td) {
     v[2 * c + 1] = f_mul(s, f_fma(tt, re, im));
   }
 }
-// the same for the 4 spins of one colour (v[2 spin], v[2 spin + 1])
-template <typename R>
-__device__ __forceinline__ void twist8(R v[8], double sd, double td) {
-  const R s = R(sd), t = R(td);
-#pragma unroll
-  for (int sp = 0; sp < 4; ++sp) {
-    const R re = v[2 * sp], im = v[2 * sp + 1];
-    const R tt = sp < 2 ? t : -t;
-    v[2 * sp] = s * (re - tt * im);
-    v[2 * sp + 1] = s * (im + tt * re);
-  }
-}
-
 // Whole-CTA exit for a single-slot launch whose slot does not run.
 __device__ __forceinline__ bool single_slot_idle(const Launch& L) {
   return L.nslots == 1 && !slot_runs(work_of(L, 0));
@@ -304,7 +292,7 @@ struct MrhsPipe {
     mrhs_load_link<NR>(s, K, u);
     const int eta = (MU == 3 && t == (FWD ? g.L[3] - 1 : 0)) ? g.t_bc : 1;
     constexpr int S = FWD ? (DAG ? 1 : -1) : (DAG ? -1 : 1);
-    hop_words<MU, S, !FWD, SP>(b[K % D], u, eta, acc);
+    hop_words<MU, S, !FWD, false, SP>(b[K % D], u, eta, acc);
     if (K + D < 8) {
       constexpr int KN = (K + D < 8) ? K + D : 0;
       IO::load_raw(in, g.Vh, (KN % 2 == 0) ? nf[KN / 2] : nb[KN / 2], b[K % D]);
@@ -398,6 +386,77 @@ __device__ __forceinline__ void colour_dot(const R a[8], const R b[8], double& r
   im = (double)si;
 }
 
+// The colour-split form's epilogue, packed like its hops: v, the four spins of one colour, with
+// double-float's own rounding sequence per lane. The Work's FP64 coefficients are taken apart
+// by their bits (a conversion instruction runs on the FP64 pipe, for every thread of every
+// tile), and factors of one are skipped (twisted M-hat 24^3x48 324.9 -> 320.9 us).
+__device__ __forceinline__ df64x2 df2_all(df64 c) { return df2_pack(c, c); }
+__device__ __forceinline__ df64 df_of_bits(double x) {
+  df64 v;
+  cv::to_df(x, v.hi, v.lo);
+  return v;
+}
+__device__ __forceinline__ Spins4 load_spins(const void* base, int Vh, int h, int col) {
+  df64 d[8];
+  SpinorIO<P_DF64>::load_colour(base, Vh, h, col, d);
+  Spins4 v;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    v.re[i] = df2_pack(d[4 * i], d[4 * i + 2]);
+    v.im[i] = df2_pack(d[4 * i + 1], d[4 * i + 3]);
+  }
+  return v;
+}
+__device__ __forceinline__ void unpack_spins(const Spins4& v, df64 d[8]) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    df2_unpack(v.re[i], d[4 * i], d[4 * i + 2]);
+    df2_unpack(v.im[i], d[4 * i + 1], d[4 * i + 3]);
+  }
+}
+__device__ __forceinline__ void store_spins(void* base, int Vh, int h, int col, const Spins4& v) {
+  df64 d[8];
+  unpack_spins(v, d);
+  SpinorIO<P_DF64>::store_colour(base, Vh, h, col, d);
+}
+__device__ __forceinline__ void scale_spins(Spins4& v, df64 c) {
+  const df64x2 cc = df2_all(c);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    v.re[i] = df2_mul(v.re[i], cc);
+    v.im[i] = df2_mul(v.im[i], cc);
+  }
+}
+// v += c y
+__device__ __forceinline__ void axpy_spins(Spins4& v, df64 c, const Spins4& y) {
+  const df64x2 cc = df2_all(c);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    v.re[i] = df2_add(v.re[i], df2_mul(cc, y.re[i]));
+    v.im[i] = df2_add(v.im[i], df2_mul(cc, y.im[i]));
+  }
+}
+// v <- s (1 + i t g5) v
+__device__ __forceinline__ void twist_spins(Spins4& v, double sd, double td) {
+  if (td != 0.0) {
+    const df64 t = df_of_bits(td);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const df64x2 tt = df2_all(i == 0 ? t : -t), re = v.re[i], im = v.im[i];
+      v.re[i] = df2_add(re, df2_neg(df2_mul(tt, im)));
+      v.im[i] = df2_add(im, df2_mul(tt, re));
+    }
+  }
+  if (sd != 1.0) {
+    const df64x2 s = df2_all(df_of_bits(sd));
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      v.re[i] = df2_mul(s, v.re[i]);
+      v.im[i] = df2_mul(s, v.im[i]);
+    }
+  }
+}
+
 #ifndef LQCD_DSLASH3_MIN_BLOCKS
 #define LQCD_DSLASH3_MIN_BLOCKS 4
 #endif
@@ -430,62 +489,54 @@ __global__ void __launch_bounds__(3 * TILE, LQCD_DSLASH3_MIN_BLOCKS) k_dslash3(c
     double v0 = 0.0, v1 = 0.0, v2 = 0.0;
     // every thread runs the hops (they share projections through barriers); a thread
     // past the end of the lattice takes the last site and drops the result
-    R acc[8];
+    Spins4 acc;
     dslash_site3s_df<LP, DAG, TILE>(w.g, h < Vh ? h : Vh - 1, w.out_par, w.in, w.Uout, w.Uin, col, j, acc, sh);
     if (h < Vh) {
-      const R a = (R)w.a;
+      R v[8], u[8];
       if constexpr (EpiTraits<EPI>::lin) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] *= a;
-        if constexpr (EpiTraits<EPI>::tw) twist8(acc, w.tw_s, w.tw_t);
-        R y[8];
+        if (w.a != 1.0) scale_spins(acc, df_of_bits(w.a));
+        if constexpr (EpiTraits<EPI>::tw) twist_spins(acc, w.tw_s, w.tw_t);
+        Spins4 y;
         if (w.y1) {
-          SpinorIO<SP>::load_colour(w.y1, Vh, h, col, y);
-          const R c = (R)w.c1;
-#pragma unroll
-          for (int i = 0; i < 8; ++i) acc[i] += c * y[i];
+          y = load_spins(w.y1, Vh, h, col);
+          axpy_spins(acc, df_of_bits(w.c1), y);
         }
         if (w.y2) {
-          R y2[8];
-          SpinorIO<SP>::load_colour(w.y2, Vh, h, col, y2);
-          if constexpr (EpiTraits<EPI>::tw) twist8(y2, 1.0, w.ty_t);
-          const R c = (R)w.c2;
-#pragma unroll
-          for (int i = 0; i < 8; ++i) acc[i] += c * y2[i];
+          Spins4 y2 = load_spins(w.y2, Vh, h, col);
+          if constexpr (EpiTraits<EPI>::tw) twist_spins(y2, 1.0, w.ty_t);
+          axpy_spins(acc, df_of_bits(w.c2), y2);
         }
-        SpinorIO<SP>::store_colour(w.out, Vh, h, col, acc);
+        store_spins(w.out, Vh, h, col, acc);
         if (!EpiTraits<EPI>::red) {
         } else if (w.red == 1) {
-          v0 = colour_norm2(acc);
+          unpack_spins(acc, v);
+          v0 = colour_norm2(v);
         } else if (w.red == 2) {
-          R z[8];
-          SpinorIO<SP>::load_colour(w.zin, Vh, h, col, z);
-          colour_dot(z, acc, v0, v1);
+          unpack_spins(acc, v);
+          SpinorIO<SP>::load_colour(w.zin, Vh, h, col, u);
+          colour_dot(u, v, v0, v1);
         } else if (w.red == 3) {
-          colour_dot(acc, y, v0, v1);
-          v2 = colour_norm2(acc);
+          unpack_spins(acc, v);
+          unpack_spins(y, u);
+          colour_dot(v, u, v0, v1);
+          v2 = colour_norm2(v);
         }
       } else {
-        const R alpha = (R)w.sc->alpha;
-        R y[8], r[8];
-        SpinorIO<SP>::load_colour(w.y1, Vh, h, col, y);
-        SpinorIO<SP>::load_colour(w.out, Vh, h, col, r);
+        const df64 alpha = df_of_bits(w.sc->alpha);
+        Spins4 y = load_spins(w.y1, Vh, h, col), r = load_spins(w.out, Vh, h, col);
         if constexpr (EpiTraits<EPI>::tw) {
-          twist8(acc, w.tw_s, w.tw_t);
-          twist8(y, 1.0, w.ty_t);
+          twist_spins(acc, w.tw_s, w.tw_t);
+          twist_spins(y, 1.0, w.ty_t);
         }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) r[i] -= alpha * (y[i] + a * acc[i]);
-        SpinorIO<SP>::store_colour(w.out, Vh, h, col, r);
-        v0 = colour_norm2(r);
-        using XR = typename SpinorIO<XSloppy<SP>::P>::Real;
-        R p[8];
-        XR x[8];
-        SpinorIO<SP>::load_colour(w.zin, Vh, h, col, p);
-        SpinorIO<XSloppy<SP>::P>::load_colour(w.z, Vh, h, col, x);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] += cvt<XR>(alpha) * cvt<XR>(p[i]);
-        SpinorIO<XSloppy<SP>::P>::store_colour(w.z, Vh, h, col, x);
+        axpy_spins(y, df_of_bits(w.a), acc);
+        axpy_spins(r, -alpha, y);
+        store_spins(w.out, Vh, h, col, r);
+        unpack_spins(r, v);
+        v0 = colour_norm2(v);
+        static_assert(XSloppy<SP>::P == P_DF64, "the solution accumulator's type");
+        Spins4 x = load_spins(w.z, Vh, h, col);
+        axpy_spins(x, alpha, load_spins(w.zin, Vh, h, col));
+        store_spins(w.z, Vh, h, col, x);
       }
     }
     if constexpr (EpiTraits<EPI>::red) tile_partial<3 * TILE>(w, start / TILE, v0, v1, v2, L.partials);
