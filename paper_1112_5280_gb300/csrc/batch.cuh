@@ -24,9 +24,11 @@ namespace lqcd {
 constexpr int TILE = LQCD_TILE;   // sites per tile (one tile per CTA pass of a batched kernel)
 constexpr int MAX_SLOTS = 1024;   // slots in one launch
 
-// Dslash epilogues. EPI_PLAIN: EPI_LIN for launches in which no slot reduces or runs a
-// finisher (chosen by launch_dslash), compiled without the reduction code.
-enum Epi { EPI_LIN = 0, EPI_CG = 1, EPI_LIN_TW = 2, EPI_CG_TW = 3, EPI_PLAIN = 4 };
+// Dslash epilogues. EPI_PLAIN, EPI_PLAIN_TW: EPI_LIN and EPI_LIN_TW for launches in which no
+// slot reduces or runs a finisher (chosen by launch_dslash), compiled without the reduction
+// code, whose registers spill the hops' (twisted M-hat without it: double-float 24^3x48
+// 320.9 -> 300.1 us, FP64 16^3x32 298.6 -> 285.5, FP16-12 32^3x64 168.2 -> 155.1).
+enum Epi { EPI_LIN = 0, EPI_CG = 1, EPI_LIN_TW = 2, EPI_CG_TW = 3, EPI_PLAIN = 4, EPI_PLAIN_TW = 5 };
 
 // Slot state machine of the Krylov engine.
 enum SlotState { S_RUNNING = 0, S_UPDATE = 1, S_DONE = 2, S_FAILED = 3, S_IDLE = 4 };

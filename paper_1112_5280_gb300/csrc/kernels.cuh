@@ -12,11 +12,11 @@ namespace lqcd {
 // keep the Wilson kernels free of the twist code.
 template <int EPI>
 struct EpiTraits {
-  static constexpr bool lin = (EPI == EPI_LIN || EPI == EPI_LIN_TW || EPI == EPI_PLAIN);
-  static constexpr bool tw = (EPI == EPI_LIN_TW || EPI == EPI_CG_TW);
-  static constexpr bool red = (EPI != EPI_PLAIN);
+  static constexpr bool lin = (EPI != EPI_CG && EPI != EPI_CG_TW);
+  static constexpr bool tw = (EPI == EPI_LIN_TW || EPI == EPI_CG_TW || EPI == EPI_PLAIN_TW);
+  static constexpr bool red = (EPI != EPI_PLAIN && EPI != EPI_PLAIN_TW);
   // the launch may finish the one before it (K3 of the CG: no reduction of its own)
-  static constexpr bool finishes = (EPI == EPI_PLAIN || EPI == EPI_LIN_TW);
+  static constexpr bool finishes = !red;
 };
 
 // Occupancy target (CTAs of TILE threads per SM) of the Dslash: 6 leaves 168

@@ -88,6 +88,8 @@ cudaError_t dispatch_tw(bool dag, int epi, const Launch& L, int grid, cudaStream
   switch (epi) {
     case EPI_LIN_TW: return dag ? go_dslash<NR, true, EPI_LIN_TW>(L, grid, s, form)
                                 : go_dslash<NR, false, EPI_LIN_TW>(L, grid, s, form);
+    case EPI_PLAIN_TW: return dag ? go_dslash<NR, true, EPI_PLAIN_TW>(L, grid, s, form)
+                                  : go_dslash<NR, false, EPI_PLAIN_TW>(L, grid, s, form);
     case EPI_CG_TW: if (dag) return go_dslash<NR, true, EPI_CG_TW>(L, grid, s, form); break;
   }
   return cudaErrorInvalidValue;
@@ -130,6 +132,7 @@ cudaError_t dispatch_nr(bool dag, int epi, const Launch& L, int grid, cudaStream
                                : go_dslash<NR, false, EPI_PLAIN>(L, grid, s, form);
     case EPI_CG: if (dag) return go_dslash<NR, true, EPI_CG>(L, grid, s, form); break;
     case EPI_LIN_TW:
+    case EPI_PLAIN_TW:
     case EPI_CG_TW:
 #ifdef LQCD_TW_EXTERN
       return LQCD_CAT(launch_dslash_tw_, LQCD_SFX)(NR, dag, epi, L, grid, s, form);
@@ -169,7 +172,8 @@ cudaError_t LQCD_CAT(launch_dslash_, LQCD_SFX)(int nr, bool dag, int epi, const 
                                                 int grid, cudaStream_t s, int form) {
   // a twisted single-slot work needs the twisted epilogue (a batched launch's works live
   // on the device; their callers pick the epilogue from the slots they hold)
-  if (!L.works && L.inline_work.twist && epi != EPI_LIN_TW && epi != EPI_CG_TW) return cudaErrorInvalidValue;
+  if (!L.works && L.inline_work.twist && epi != EPI_LIN_TW && epi != EPI_PLAIN_TW && epi != EPI_CG_TW)
+    return cudaErrorInvalidValue;
 #ifdef LQCD_STREAM_EXTERN
   if (L.stream_links && (nr == 18 || nr == 12))
     return LQCD_CAT(launch_dslash_stream_, LQCD_SFX)(nr, dag, epi, L, grid, s, form);
