@@ -24,6 +24,8 @@ namespace lqcd {
 // with everything else unchanged: a 32^3x64 FP16 operator chain with its result to the host
 // layout 1379 -> 1295 us (the download 181 -> 98 us), a 24^3x48 double-float one 1670 ->
 // 1618 us, a 22x18x14x38 configuration and source in and the result out 777 -> 723 us.
+// They are programmatic dependents and let theirs start, as the operators between them do: a
+// download between two 8^4 M-hats 12.3 -> 9.65 us a call.
 
 // ------------------------------------------------------------------ words
 
@@ -117,6 +119,7 @@ constexpr int LAYOUT_THREADS = 256;
 // TO_AOS false: AoS U[site][mu][row][col] -> [parity][mu][word][V/2] of double2; true: back
 template <bool TO_AOS>
 __global__ void __launch_bounds__(LAYOUT_THREADS) k_gauge_aos(const double* in, Geom g, double* out) {
+  pdl_entry();
   __shared__ double sm[2][TILE_H][73];
   const int h0 = blockIdx.x * TILE_H, nh = min(TILE_H, g.Vh - h0);
   const size_t first = (size_t)h0 * 2 * 72;
@@ -155,18 +158,18 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_gauge_aos(const double* in, 
 static unsigned aos_grid(const Geom& g) { return (unsigned)((g.Vh + TILE_H - 1) / TILE_H); }
 
 cudaError_t links_from_aos(const double* aos, const Geom& g, double2* U, cudaStream_t s) {
-  k_gauge_aos<false><<<aos_grid(g), LAYOUT_THREADS, 0, s>>>(aos, g, reinterpret_cast<double*>(U));
-  return cudaGetLastError();
+  return launch_k(k_gauge_aos<false>, dim3(aos_grid(g)), dim3(LAYOUT_THREADS), 0, s, aos, g,
+                  reinterpret_cast<double*>(U));
 }
 cudaError_t links_to_aos(const double2* U, const Geom& g, double2* aos, cudaStream_t s) {
-  k_gauge_aos<true><<<aos_grid(g), LAYOUT_THREADS, 0, s>>>(reinterpret_cast<const double*>(U), g,
-                                                          reinterpret_cast<double*>(aos));
-  return cudaGetLastError();
+  return launch_k(k_gauge_aos<true>, dim3(aos_grid(g)), dim3(LAYOUT_THREADS), 0, s,
+                  reinterpret_cast<const double*>(U), g, reinterpret_cast<double*>(aos));
 }
 
 // One link of the FP64 18-real layout to precision P with NR reals; word sizes as in LinkIO.
 template <int P, int NR>
 __global__ void __launch_bounds__(LAYOUT_THREADS) k_gauge_convert(const double2* __restrict__ in64, Geom g, void* out) {
+  pdl_entry();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (par, mu, h)
   if (i >= 8LL * g.Vh) return;
   const size_t pm = (size_t)(i / g.Vh);  // 4 par + mu
@@ -200,9 +203,8 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_gauge_convert(const double2*
 template <int P, int NR>
 static cudaError_t go_gauge_convert(const void* a, const Geom& g, void* o, cudaStream_t s) {
   const long long n = 8LL * g.Vh;
-  k_gauge_convert<P, NR><<<(unsigned)((n + LAYOUT_THREADS - 1) / LAYOUT_THREADS), LAYOUT_THREADS, 0, s>>>(
-      static_cast<const double2*>(a), g, o);
-  return cudaGetLastError();
+  return launch_k(k_gauge_convert<P, NR>, dim3((unsigned)((n + LAYOUT_THREADS - 1) / LAYOUT_THREADS)),
+                  dim3(LAYOUT_THREADS), 0, s, static_cast<const double2*>(a), g, o);
 }
 
 cudaError_t gauge_convert(const void* d64, const Geom& g, int prec, int nr, void* d_out,
@@ -219,6 +221,7 @@ cudaError_t gauge_convert(const void* d64, const Geom& g, int prec, int nr, void
 
 // FP64 master words from the double-float copy (hi + lo, exact in FP64)
 __global__ void __launch_bounds__(LAYOUT_THREADS) k_master_from_df(double2* U, const float4* Ud, long long n) {
+  pdl_entry();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float4 d = Ud[i];
@@ -226,8 +229,8 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_master_from_df(double2* U, c
 }
 cudaError_t master_from_df(double2* U, const float4* Ud, const Geom& g, cudaStream_t s) {
   const long long n = 72LL * g.Vh;
-  k_master_from_df<<<(unsigned)((n + LAYOUT_THREADS - 1) / LAYOUT_THREADS), LAYOUT_THREADS, 0, s>>>(U, Ud, n);
-  return cudaGetLastError();
+  return launch_k(k_master_from_df, dim3((unsigned)((n + LAYOUT_THREADS - 1) / LAYOUT_THREADS)),
+                  dim3(LAYOUT_THREADS), 0, s, U, Ud, n);
 }
 
 // ------------------------------------------------------------------ spinors
@@ -235,6 +238,7 @@ cudaError_t master_from_df(double2* U, const float4* Ud, const Geom& g, cudaStre
 template <int P>
 __global__ void __launch_bounds__(LAYOUT_THREADS) k_spinor_from_aos(const double* __restrict__ aos, Geom g, void* ev,
                                                                     void* od) {
+  pdl_entry();
   using Wd = Words<P>;
   __shared__ double sm[2][TILE_H][25];
   const int h0 = blockIdx.x * TILE_H, nh = min(TILE_H, g.Vh - h0);
@@ -258,6 +262,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_spinor_from_aos(const double
 template <int P>
 __global__ void __launch_bounds__(LAYOUT_THREADS) k_spinor_to_aos(const void* ev, const void* od, Geom g,
                                                                   double* __restrict__ aos) {
+  pdl_entry();
   using Wd = Words<P>;
   __shared__ double sm[2][TILE_H][25];
   __shared__ int rps[TILE_H];
@@ -290,6 +295,8 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_spinor_to_aos(const void* ev
 // One thread per site and eight reals (one FP16 word, two FP32, four FP64 or double-float).
 template <int PI, int PO>
 __global__ void __launch_bounds__(LAYOUT_THREADS) k_spinor_convert(const void* in, void* out, int Vh, double scale) {
+  pdl_wait();
+  if (in != out) pdl_trigger();  // in place: the next grid starts when this one is done
   using Wi = Words<PI>;
   using Wo = Words<PO>;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (group, h)
@@ -311,13 +318,11 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_spinor_convert(const void* i
 
 template <int P>
 static cudaError_t go_from_aos(const double* a, const Geom& g, void* e, void* o, cudaStream_t s) {
-  k_spinor_from_aos<P><<<aos_grid(g), LAYOUT_THREADS, 0, s>>>(a, g, e, o);
-  return cudaGetLastError();
+  return launch_k(k_spinor_from_aos<P>, dim3(aos_grid(g)), dim3(LAYOUT_THREADS), 0, s, a, g, e, o);
 }
 template <int P>
 static cudaError_t go_to_aos(const void* e, const void* o, const Geom& g, double* a, cudaStream_t s) {
-  k_spinor_to_aos<P><<<aos_grid(g), LAYOUT_THREADS, 0, s>>>(e, o, g, a);
-  return cudaGetLastError();
+  return launch_k(k_spinor_to_aos<P>, dim3(aos_grid(g)), dim3(LAYOUT_THREADS), 0, s, e, o, g, a);
 }
 
 cudaError_t spinor_from_aos(const double* d_aos, const Geom& g, int prec, void* d_even,
@@ -350,14 +355,13 @@ static cudaError_t go_convert_in(const void* in, void* out, int pout, int Vh, do
   const long long n = 3LL * Vh;
   const unsigned nb = (unsigned)((n + LAYOUT_THREADS - 1) / LAYOUT_THREADS);
   switch (pout) {
-    case P_F64: k_spinor_convert<PI, P_F64><<<nb, LAYOUT_THREADS, 0, s>>>(in, out, Vh, sc); break;
-    case P_F32: k_spinor_convert<PI, P_F32><<<nb, LAYOUT_THREADS, 0, s>>>(in, out, Vh, sc); break;
-    case P_F16: k_spinor_convert<PI, P_F16><<<nb, LAYOUT_THREADS, 0, s>>>(in, out, Vh, sc); break;
-    case P_BF16: k_spinor_convert<PI, P_BF16><<<nb, LAYOUT_THREADS, 0, s>>>(in, out, Vh, sc); break;
-    case P_DF64: k_spinor_convert<PI, P_DF64><<<nb, LAYOUT_THREADS, 0, s>>>(in, out, Vh, sc); break;
-    default: return cudaErrorInvalidValue;
+    case P_F64: return launch_k(k_spinor_convert<PI, P_F64>, dim3(nb), dim3(LAYOUT_THREADS), 0, s, in, out, Vh, sc);
+    case P_F32: return launch_k(k_spinor_convert<PI, P_F32>, dim3(nb), dim3(LAYOUT_THREADS), 0, s, in, out, Vh, sc);
+    case P_F16: return launch_k(k_spinor_convert<PI, P_F16>, dim3(nb), dim3(LAYOUT_THREADS), 0, s, in, out, Vh, sc);
+    case P_BF16: return launch_k(k_spinor_convert<PI, P_BF16>, dim3(nb), dim3(LAYOUT_THREADS), 0, s, in, out, Vh, sc);
+    case P_DF64: return launch_k(k_spinor_convert<PI, P_DF64>, dim3(nb), dim3(LAYOUT_THREADS), 0, s, in, out, Vh, sc);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t spinor_convert(const void* in, int pin, void* out, int pout, int Vh, double scale,

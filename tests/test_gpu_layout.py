@@ -117,3 +117,53 @@ def test_conversion_range(ctx, scale):
         back = ctx.field(dims, "f64")
         back.copy_from(f)
         assert np.array_equal(back.download().view(np.float64), want.view(np.float64))
+
+
+def test_layout_under_capture():
+    """Uploads, conversions and downloads of device arrays in a captured graph, beside the
+    operators, a memset and a copy on a side stream, on a borrowed stream: each replay follows
+    the source tensor."""
+    import torch
+
+    dims = (6, 2, 4, 6)
+    st = torch.cuda.Stream()
+    ctx = lqcd.Context(0, stream=st)
+    g = ctx.gauge(dims, synth.random_links(dims, 0.6, seed=9), "f32")
+    src = torch.zeros((int(np.prod(dims)), 4, 3), dtype=torch.complex128, device="cuda")
+    out = torch.full_like(src, -7.0)
+    stage = torch.zeros_like(src)
+    side = torch.cuda.Stream()
+    f, a, b = ctx.field(dims, "f64"), ctx.field(dims, "f32"), ctx.field(dims, "f32")
+
+    def chain():
+        f.zero()
+        side.wait_stream(st)
+        with torch.cuda.stream(side):
+            src.copy_(stage)
+        st.wait_stream(side)
+        f.upload(src)
+        a.zero()
+        a.copy_from(f, 0.5)
+        lqcd.apply_M(g, 0.14, a, b)
+        b.copy_from(b, 2.0)
+        b.download(out)
+
+    torch.cuda.synchronize()
+    chain()
+    ctx.sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        chain()
+    for seed in (3, 4):
+        stage.copy_(torch.from_numpy(synth.gaussian_spinor(dims, seed=seed)))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        got = out.cpu().numpy()
+        out.fill_(-7.0)
+        torch.cuda.synchronize()
+        chain()
+        ctx.sync()
+        assert np.array_equal(got, out.cpu().numpy()) and np.abs(got).max() > 1
+    del graph
+    ctx.close()
