@@ -103,8 +103,11 @@ LQCD_API long long lqcd_ctx_launch_count(const lqcd_ctx* ctx);
 /* The one-shot solves keep their device buffers on the context between calls
  * (the Krylov engine of lqcd_solve*, lqcd_solve_normal and the HMC driver; the
  * BiCGStab vectors; operator and upload temporaries), so repeated solves
- * allocate nothing. This waits for the context's stream and frees them; the
- * next call allocates again. Objects the caller created are untouched. */
+ * allocate nothing, and up to 1 GiB of the buffers of destroyed fields, gauge
+ * fields and momenta, for the next ones of the same size (given back also when
+ * an allocation for the context fails). This waits for the context's stream and
+ * frees them; the next call allocates again. Objects the caller created are
+ * untouched. */
 LQCD_API int lqcd_ctx_release_cache(lqcd_ctx* ctx);
 
 /* ---------------------------------------------------------------- gauge field (A1) */

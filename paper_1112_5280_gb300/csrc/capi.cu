@@ -60,7 +60,7 @@ int ctx_partials(lqcd_ctx* c, size_t n) {
   if (c->partials) cudaFree(c->partials);
   c->partials = nullptr;
   c->partials_cap = 0;
-  LQCD_CK(cudaMalloc(&c->partials, n * sizeof(double)));
+  LQCD_CK(ctx_malloc(c, (void**)&c->partials, n * sizeof(double)));
   c->partials_cap = n;
   return LQCD_OK;
 }
@@ -71,7 +71,7 @@ int ctx_tmp(lqcd_ctx* c, size_t bytes) {
   if (c->tmp) cudaFree(c->tmp);
   c->tmp = nullptr;
   c->tmp_bytes = 0;
-  LQCD_CK(cudaMalloc(&c->tmp, bytes));
+  LQCD_CK(ctx_malloc(c, (void**)&c->tmp, bytes));
   c->tmp_bytes = bytes;
   return LQCD_OK;
 }
@@ -82,7 +82,7 @@ int ctx_work(lqcd_ctx* c, size_t bytes) {
   if (c->work) cudaFree(c->work);
   c->work = nullptr;
   c->work_bytes = 0;
-  LQCD_CK(cudaMalloc(&c->work, bytes));
+  LQCD_CK(ctx_malloc(c, (void**)&c->work, bytes));
   c->work_bytes = bytes;
   return LQCD_OK;
 }
@@ -93,9 +93,63 @@ int ctx_staging(lqcd_ctx* c, size_t bytes) {
   if (c->staging) cudaFree(c->staging);
   c->staging = nullptr;
   c->staging_bytes = 0;
-  LQCD_CK(cudaMalloc(&c->staging, bytes));
+  LQCD_CK(ctx_malloc(c, (void**)&c->staging, bytes));
   c->staging_bytes = bytes;
   return LQCD_OK;
+}
+
+static bool capturing(const lqcd_ctx* c) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
+cudaError_t ctx_malloc(lqcd_ctx* c, void** out, size_t bytes) {
+  cudaError_t e = cudaMalloc(out, bytes);
+  if (e == cudaErrorMemoryAllocation && ctx_pool_release(c)) {
+    cudaGetLastError();
+    e = cudaMalloc(out, bytes);
+  }
+  return e;
+}
+
+cudaError_t ctx_alloc(lqcd_ctx* c, void** out, size_t bytes) {
+  if (!capturing(c)) {
+    std::lock_guard<std::mutex> lk(c->pool_mu);
+    auto it = c->pool.find(bytes);
+    if (it != c->pool.end()) {
+      *out = it->second;
+      c->pool.erase(it);
+      c->pool_bytes -= bytes;
+      return cudaSuccess;
+    }
+  }
+  return ctx_malloc(c, out, bytes);
+}
+
+void ctx_free(lqcd_ctx* c, void* p, size_t bytes) {
+  if (!p) return;
+  if (!capturing(c)) {
+    std::lock_guard<std::mutex> lk(c->pool_mu);
+    if (c->pool_bytes + bytes <= POOL_BYTES) {
+      c->pool.insert({bytes, p});
+      c->pool_bytes += bytes;
+      return;
+    }
+  }
+  cudaFree(p);
+}
+
+bool ctx_pool_release(lqcd_ctx* c) {
+  std::lock_guard<std::mutex> lk(c->pool_mu);
+  const bool any = !c->pool.empty();
+  for (auto& kv : c->pool) cudaFree(kv.second);
+  c->pool.clear();
+  c->pool_bytes = 0;
+  return any;
 }
 
 int gauge_links(const lqcd_gauge* gc, int field_prec, const void** base, int* nr) {
@@ -106,7 +160,7 @@ int gauge_links(const lqcd_gauge* gc, int field_prec, const void** base, int* nr
   void*& slot = g->copy[lp][n == 12];
   if (!slot) {
     size_t b = gauge_copy_bytes(lp, n, g->g.Vh);
-    LQCD_CK(cudaMalloc(&slot, b));
+    LQCD_CK(ctx_alloc(g->ctx, &slot, b));
     g->bytes += b;
     LQCD_CK(gauge_convert(g->copy[P_F64][0], g->g, lp, n, slot, g->ctx->stream));
   }
@@ -212,6 +266,7 @@ void ctx_release(lqcd_ctx* c) {
   cudaSetDevice(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
   ctx_drop_engine(c);
+  ctx_pool_release(c);
   if (c->partials) cudaFree(c->partials);
   if (c->scratch_sc) cudaFree(c->scratch_sc);
   if (c->host_sc) cudaFreeHost(c->host_sc);
@@ -271,6 +326,7 @@ int lqcd_ctx_release_cache(lqcd_ctx* c) {
   LQCD_CK(cudaSetDevice(c->device));
   LQCD_CK(cudaStreamSynchronize(c->stream));
   ctx_drop_engine(c);
+  ctx_pool_release(c);
   void** bufs[] = {&c->tmp, &c->work, reinterpret_cast<void**>(&c->staging)};
   size_t* caps[] = {&c->tmp_bytes, &c->work_bytes, &c->staging_bytes};
   for (int i = 0; i < 3; ++i) {
@@ -319,7 +375,7 @@ static int gauge_upload_impl(lqcd_ctx* c, const int dims[4], const double* U, bo
   gg->prec = prec;
   gg->compress = compress;
   const size_t b64 = gauge_copy_bytes(P_F64, 18, g.Vh);
-  cudaError_t e = cudaMalloc(&gg->copy[P_F64][0], b64);
+  cudaError_t e = ctx_alloc(c, &gg->copy[P_F64][0], b64);
   if (e != cudaSuccess) {
     delete gg;
     return set_error(LQCD_ENOMEM, "gauge field: %s", cudaGetErrorString(e));
@@ -368,7 +424,7 @@ int lqcd_gauge_add_copy(lqcd_gauge* g, int prec, int compress) {
   void*& slot = g->copy[lp][compress == 12];
   if (slot) return LQCD_OK;
   const size_t b = gauge_copy_bytes(lp, compress, g->g.Vh);
-  cudaError_t e = cudaMalloc(&slot, b);
+  cudaError_t e = ctx_alloc(g->ctx, &slot, b);
   if (e != cudaSuccess) {
     slot = nullptr;
     return set_error(LQCD_ENOMEM, "gauge copy: %s", cudaGetErrorString(e));
@@ -384,9 +440,8 @@ void lqcd_gauge_destroy(lqcd_gauge* g) {
   if (!g) return;
   cudaSetDevice(g->ctx->device);
   cudaStreamSynchronize(g->ctx->stream);
-  for (auto& row : g->copy)
-    for (auto& p : row)
-      if (p) cudaFree(p);
+  for (int p = 0; p < NPREC; ++p)
+    for (int k = 0; k < 2; ++k) ctx_free(g->ctx, g->copy[p][k], gauge_copy_bytes(p, k ? 12 : 18, g->g.Vh));
   lqcd_ctx* c = g->ctx;
   delete g;
   ctx_release(c);
@@ -412,7 +467,7 @@ int lqcd_field_create(lqcd_ctx* c, const int dims[4], int prec, int subset, lqcd
   f->half_bytes = half_spinor_bytes(prec, g.Vh);
   for (int p = 0; p < 2; ++p) {
     if (subset != LQCD_FULL && subset != p) continue;
-    cudaError_t e = cudaMalloc(&f->half[p], f->half_bytes);
+    cudaError_t e = ctx_alloc(c, &f->half[p], f->half_bytes);
     if (e == cudaSuccess) e = cudaMemsetAsync(f->half[p], 0, f->half_bytes, c->stream);
     if (e != cudaSuccess) {
       lqcd_field_destroy(f);
@@ -431,8 +486,7 @@ void lqcd_field_destroy(lqcd_field* f) {
   if (!f) return;
   cudaSetDevice(f->ctx->device);
   cudaStreamSynchronize(f->ctx->stream);
-  for (auto& p : f->half)
-    if (p) cudaFree(p);
+  for (auto& p : f->half) ctx_free(f->ctx, p, f->half_bytes);
   lqcd_ctx* c = f->ctx;
   delete f;
   ctx_release(c);
@@ -676,8 +730,8 @@ int lqcd_dslash_batch_create(int n, const lqcd_gauge* const* g, const lqcd_field
   b->nr = nr;
   b->dagger = dagger != 0;
   b->n = n;
-  cudaError_t e = cudaMalloc(&b->d_works, sizeof(Work) * n);
-  if (e == cudaSuccess) e = cudaMalloc(&b->d_prefix, sizeof(int) * (n + 1));
+  cudaError_t e = ctx_malloc(c, (void**)&b->d_works, sizeof(Work) * n);
+  if (e == cudaSuccess) e = ctx_malloc(c, (void**)&b->d_prefix, sizeof(int) * (n + 1));
   if (e == cudaSuccess) e = cudaMemcpy(b->d_works, w.data(), sizeof(Work) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(b->d_prefix, prefix.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {

@@ -547,7 +547,7 @@ int ensure_partials(lqcd_engine* e, size_t n) {
   if (e->d_partials) cudaFree(e->d_partials);
   e->d_partials = nullptr;
   size_t cap = std::max(n, 2 * e->partials_cap);
-  LQCD_CK(cudaMalloc(&e->d_partials, cap * sizeof(double)));
+  LQCD_CK(ctx_malloc(e->ctx, (void**)&e->d_partials, cap * sizeof(double)));
   e->partials_cap = cap;
   e->dirty = true;
   return LQCD_OK;
@@ -584,7 +584,7 @@ int alloc_block(lqcd_engine* e, size_t bytes, void** out) {
     e->bytes_pooled -= p->first;
     e->pool.erase(p);
   }
-  cudaError_t err = cudaMalloc(out, bytes);
+  cudaError_t err = ctx_malloc(e->ctx, out, bytes);
   if (err != cudaSuccess) {
     cudaGetLastError();
     return set_error(LQCD_ENOMEM, "slot buffers (%zu bytes): %s", bytes, cudaGetErrorString(err));
@@ -700,11 +700,11 @@ int lqcd_engine_create(lqcd_ctx* c, const lqcd_solve_opts* opts, size_t budget, 
   e->ru_every = o.ru_interval > 0 ? std::min(o.ru_interval, o.chunk) : 0;  // 0: per batch
   e->budget = budget;
   e->max_slots = max_slots;
-  cudaError_t err = cudaMalloc(&e->d_sc, sizeof(Scalars) * max_slots);
+  cudaError_t err = ctx_malloc(c, (void**)&e->d_sc, sizeof(Scalars) * max_slots);
   if (err == cudaSuccess) err = cudaMemset(e->d_sc, 0, sizeof(Scalars) * max_slots);
   if (err == cudaSuccess) err = cudaMallocHost(&e->h_sc, sizeof(Scalars) * max_slots);
-  if (err == cudaSuccess) err = cudaMalloc(&e->d_works, sizeof(Work) * NSTEP * max_slots);
-  if (err == cudaSuccess) err = cudaMalloc(&e->d_prefix, sizeof(int) * (max_slots + 1));
+  if (err == cudaSuccess) err = ctx_malloc(c, (void**)&e->d_works, sizeof(Work) * NSTEP * max_slots);
+  if (err == cudaSuccess) err = ctx_malloc(c, (void**)&e->d_prefix, sizeof(int) * (max_slots + 1));
   if (err != cudaSuccess) {
     lqcd_engine_destroy(e);
     return set_error(LQCD_ENOMEM, "engine: %s", cudaGetErrorString(err));

@@ -496,7 +496,7 @@ int lqcd_mom_create(lqcd_ctx* c, const int dims[4], lqcd_mom** out) {
   m->ctx = c;
   m->g = g;
   m->bytes = gauge_copy_bytes(P_F64, 18, g.Vh);
-  if (cudaMalloc(&m->d, m->bytes) != cudaSuccess) {
+  if (ctx_alloc(c, reinterpret_cast<void**>(&m->d), m->bytes) != cudaSuccess) {
     cudaGetLastError();
     delete m;
     return set_error(LQCD_ENOMEM, "momentum field (%zu bytes)", gauge_copy_bytes(P_F64, 18, g.Vh));
@@ -504,7 +504,7 @@ int lqcd_mom_create(lqcd_ctx* c, const int dims[4], lqcd_mom** out) {
   cudaError_t e = cudaMemsetAsync(m->d, 0, m->bytes, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
-    cudaFree(m->d);
+    ctx_free(c, m->d, m->bytes);
     delete m;
     return set_error(LQCD_ECUDA, "momentum field: %s", cudaGetErrorString(e));
   }
@@ -517,7 +517,7 @@ void lqcd_mom_destroy(lqcd_mom* m) {
   if (!m) return;
   cudaSetDevice(m->ctx->device);
   cudaStreamSynchronize(m->ctx->stream);
-  cudaFree(m->d);
+  ctx_free(m->ctx, m->d, m->bytes);
   lqcd_ctx* c = m->ctx;
   delete m;
   ctx_release(c);
@@ -675,7 +675,7 @@ int lqcd_hmc_trajectory(lqcd_gauge* g, const lqcd_hmc_params* p, lqcd_mom* m, co
   if (rc == LQCD_OK && p->chrono == 2) rc = lqcd_field_create(c, dims, LQCD_F64, LQCD_FULL, &guess);
   if (rc == LQCD_OK) rc = ctx_engine(c, o, 1, &e);
   if (rc == LQCD_OK && p->accept_u > 0.0) {
-    if (cudaMalloc(&backup, ubytes) != cudaSuccess) {
+    if (ctx_alloc(c, &backup, ubytes) != cudaSuccess) {
       cudaGetLastError();
       rc = set_error(LQCD_ENOMEM, "link backup");
     } else if (cudaMemcpyAsync(backup, g->copy[P_F64][0], ubytes, cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess) {
@@ -785,7 +785,7 @@ int lqcd_hmc_trajectory(lqcd_gauge* g, const lqcd_hmc_params* p, lqcd_mom* m, co
   }
   if (backup) {
     cudaStreamSynchronize(c->stream);
-    cudaFree(backup);
+    ctx_free(c, backup, ubytes);
   }
   if (rc != LQCD_OK && e) ctx_drop_engine(c);  // a failure may leave a request in the engine
   for (lqcd_field* f : {x, y, xd, yd, xprev, guess}) lqcd_field_destroy(f);

@@ -6,6 +6,8 @@
 
 #include <atomic>
 #include <cstdarg>
+#include <map>
+#include <mutex>
 #include <string>
 
 #include "lqcd.h"
@@ -26,6 +28,10 @@ struct lqcd_ctx {
   void* work = nullptr;               // solver vectors of the one-shot BiCGStab
   size_t work_bytes = 0;
   long long launches = 0;
+  // freed field and link buffers by size, for the next object of that size (ctx_alloc)
+  std::mutex pool_mu;
+  std::multimap<size_t, void*> pool;
+  size_t pool_bytes = 0;
   // engine reused by the one-shot solves (lqcd_solve*, the HMC driver) while their options
   // match; it holds no reference to the context and is destroyed with it
   struct lqcd_engine* engine_cache = nullptr;
@@ -103,6 +109,21 @@ int ctx_partials(lqcd_ctx* c, size_t n);
 int ctx_tmp(lqcd_ctx* c, size_t bytes);
 int ctx_work(lqcd_ctx* c, size_t bytes);
 int ctx_staging(lqcd_ctx* c, size_t bytes);
+
+// Device buffers of fields, link copies and momenta. A cudaMalloc and cudaFree pair stops the
+// device, which a program pays for every configuration that it loads and the HMC driver for
+// each of its work fields (a 22x18x14x38 configuration and source loaded, applied and dropped:
+// 716 -> 495 us; a 16^3x32 trajectory 142.6 -> 139.8 ms). So up to POOL_BYTES of freed buffers stay
+// with the context for the next object of the same size. They are given back by
+// lqcd_ctx_release_cache, with the context, and when any allocation for the context fails
+// (ctx_malloc). Whoever frees has waited for the context's stream, and a change of stream
+// waits for the old one, so a buffer in the pool has no work pending. A stream in capture
+// allocates and frees past the pool, as refused or accepted by CUDA.
+constexpr size_t POOL_BYTES = (size_t)1 << 30;
+cudaError_t ctx_malloc(lqcd_ctx* c, void** out, size_t bytes);
+cudaError_t ctx_alloc(lqcd_ctx* c, void** out, size_t bytes);
+void ctx_free(lqcd_ctx* c, void* p, size_t bytes);
+bool ctx_pool_release(lqcd_ctx* c);  // whether it held anything
 
 // link copy for fields of precision field_prec (created on first use)
 int gauge_links(const lqcd_gauge* g, int field_prec, const void** base, int* nr);

@@ -282,15 +282,15 @@ int lqcd_autotune_dslash(int n, const lqcd_gauge* const* g, int prec, int compre
   char* buf = nullptr;
   Work* d_works = nullptr;
   int* d_prefix = nullptr;
-  cudaError_t err = cudaMalloc(&buf, off[n]);
+  cudaError_t err = ctx_malloc(c, (void**)&buf, off[n]);
   if (err == cudaSuccess) err = cudaMemsetAsync(buf, 0, off[n], st);
   for (int i = 0; i < n; ++i) {
     const size_t hb = (off[i + 1] - off[i]) / 2;
     w[i].in = buf + off[i];
     w[i].out = buf + off[i] + hb;
   }
-  if (err == cudaSuccess && n > 1) err = cudaMalloc(&d_works, sizeof(Work) * n);
-  if (err == cudaSuccess && n > 1) err = cudaMalloc(&d_prefix, sizeof(int) * (n + 1));
+  if (err == cudaSuccess && n > 1) err = ctx_malloc(c, (void**)&d_works, sizeof(Work) * n);
+  if (err == cudaSuccess && n > 1) err = ctx_malloc(c, (void**)&d_prefix, sizeof(int) * (n + 1));
   if (err == cudaSuccess && n > 1)
     err = cudaMemcpyAsync(d_works, w.data(), sizeof(Work) * n, cudaMemcpyHostToDevice, st);
   if (err == cudaSuccess && n > 1)
