@@ -13,7 +13,6 @@ struct C2 {
   double re, im;
 };
 __device__ __forceinline__ C2 cmul(C2 a, C2 b) { return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
-__device__ __forceinline__ C2 cadd(C2 a, C2 b) { return {a.re + b.re, a.im + b.im}; }
 
 struct M3 {
   C2 e[9];
@@ -59,18 +58,9 @@ __device__ __forceinline__ M3 load_link(const double2* U, const Geom& g, const S
   }
   return m;
 }
-__device__ __forceinline__ M3 mul_nn(const M3& a, const M3& b) {
-  M3 c;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      C2 s = cmul(a.e[i * 3], b.e[j]);
-      s = cadd(s, cmul(a.e[i * 3 + 1], b.e[3 + j]));
-      s = cadd(s, cmul(a.e[i * 3 + 2], b.e[6 + j]));
-      c.e[i * 3 + j] = s;
-    }
-  return c;
+// a + b c, four multiply-adds
+__device__ __forceinline__ C2 cmac(C2 a, C2 b, C2 c) {
+  return {fma(-b.im, c.im, fma(b.re, c.re, a.re)), fma(b.im, c.re, fma(b.re, c.im, a.im))};
 }
 // ---------------------------------------------------------------- double-float matrices
 // The FP64 pipes of this part run at 1/64 of the FP32 rate, so the SU(3) products of the

