@@ -182,10 +182,75 @@ struct FirstSets {
   static constexpr bool value = SP == P_F64 || SP == P_DF64;
 };
 
+// How a hop adds to the sums: HOP_SETS: acc = instead of acc +=; HOP_PACKED: acc += in packed
+// FP32 pairs
+enum HopForm { HOP_ADDS, HOP_SETS, HOP_PACKED };
+
+// acc(s0), acc(s1) += S w
+template <int S>
+__device__ __forceinline__ void acc_add2(float* acc, int s0, int s1, int col, int im, f32x2 w) {
+  float &x = acc[sidx(s0, col) + im], &y = acc[sidx(s1, col) + im];
+  const f32x2 t = p_pack(x, y);
+  p_unpack(S > 0 ? p_add(t, w) : p_sub(t, w), x, y);
+}
+// (S a, -S b) of the lanes (a, b)
+template <int S>
+__device__ __forceinline__ f32x2 p_alt(f32x2 v) {
+  float a, b;
+  p_unpack(v, a, b);
+  return S > 0 ? p_pack(a, -b) : p_pack(-a, b);
+}
+// The rest of a hop in FP32, packed (field.cuh): the lanes are the two spin rows of h, which
+// meet the same link entry, and each lane rounds as hop_half_scalar does. It
+// halves the issue slots of the 96 multiply-adds and adds of a hop, at the cost of a second
+// copy of each link real. Measured per application: BF16-12 32^3x64 73.5 -> 69.1 us, FP16-18
+// 77.2 -> 75.3, FP32-12 95.9 -> 94.5, FP32-18 122.4 -> 121.6; FP32-12 16^3x32 7.0 -> 6.8, its
+// CG 57.1 -> 55.3 us an iteration. The plain FP16-12 operator (71.2 -> 71.4) stays scalar.
+template <int MU, int S, bool ADJ>
+__device__ __forceinline__ void hop_half_packed(const Cx<float> h0[3], const Cx<float> h1[3], const float u[18],
+                                                float acc[24]) {
+  f32x2 hr[3], hi[3], nr[3], ni[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    hr[b] = p_pack(h0[b].re, h1[b].re);
+    hi[b] = p_pack(h0[b].im, h1[b].im);
+    nr[b] = p_neg(hr[b]);
+    ni[b] = p_neg(hi[b]);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    f32x2 wr, wi;  // lanes (w0, w1)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int k = (ADJ ? b * 3 + a : a * 3 + b) * 2;
+      const f32x2 rr = p_pack(u[k], u[k]), ii = p_pack(u[k + 1], u[k + 1]);
+      wr = b == 0 ? p_mul(rr, hr[b]) : p_fma(rr, hr[b], wr);
+      wi = b == 0 ? p_mul(rr, hi[b]) : p_fma(rr, hi[b], wi);
+      wr = p_fma(ii, ADJ ? hi[b] : ni[b], wr);
+      wi = p_fma(ii, ADJ ? nr[b] : hr[b], wi);
+    }
+    acc_add2<1>(acc, 0, 1, a, 0, wr);
+    acc_add2<1>(acc, 0, 1, a, 1, wi);
+    if (MU == 0) {  // (l3, l2) = S i (w0, w1)
+      acc_add2<-S>(acc, 3, 2, a, 0, wi);
+      acc_add2<S>(acc, 3, 2, a, 1, wr);
+    } else if (MU == 1) {  // (l3, l2) = (-S w0, S w1)
+      acc_add2<1>(acc, 3, 2, a, 0, p_alt<-S>(wr));
+      acc_add2<1>(acc, 3, 2, a, 1, p_alt<-S>(wi));
+    } else if (MU == 2) {  // (l2, l3) = S i (w0, -w1)
+      acc_add2<1>(acc, 2, 3, a, 0, p_alt<-S>(wi));
+      acc_add2<1>(acc, 2, 3, a, 1, p_alt<S>(wr));
+    } else {  // (l2, l3) = S (w0, w1)
+      acc_add2<S>(acc, 2, 3, a, 0, wr);
+      acc_add2<S>(acc, 2, 3, a, 1, wi);
+    }
+  }
+}
+
 // The rest of a hop: acc += (U or U^dag) h, lifted back to four spins by (1 + S g_MU); FIRST:
 // acc = that.
 template <int MU, int S, bool ADJ, bool FIRST, typename R>
-__device__ __forceinline__ void hop_half(const Cx<R> h0[3], const Cx<R> h1[3], const R u[18], R acc[24]) {
+__device__ __forceinline__ void hop_half_scalar(const Cx<R> h0[3], const Cx<R> h1[3], const R u[18], R acc[24]) {
   // w = U h (or U^dag h) per spin row: for each product u h, re += u.re h.re - u.im h.im and
   // im += u.re h.im + u.im h.re, as four multiply-adds in this order
   Cx<R> w0[3], w1[3];
@@ -229,29 +294,35 @@ __device__ __forceinline__ void hop_half(const Cx<R> h0[3], const Cx<R> h1[3], c
   }
 }
 
+template <int MU, int S, bool ADJ, int FORM, typename R>
+__device__ __forceinline__ void hop_half(const Cx<R> h0[3], const Cx<R> h1[3], const R u[18], R acc[24]) {
+  if constexpr (FORM == HOP_PACKED) hop_half_packed<MU, S, ADJ>(h0, h1, u, acc);
+  else hop_half_scalar<MU, S, ADJ, FORM == HOP_SETS>(h0, h1, u, acc);
+}
+
 // One hop: acc += eta * (1 + S g_MU) (U or U^dag) psi, eta = +-1.
-template <int MU, int S, bool ADJ, bool FIRST, typename R>
+template <int MU, int S, bool ADJ, int FORM, typename R>
 __device__ __forceinline__ void hop(const R psi[24], const R u[18], int eta, R acc[24]) {
   Cx<R> h0[3], h1[3];
   project<MU, S>(psi, eta, h0, h1);
-  hop_half<MU, S, ADJ, FIRST>(h0, h1, u, acc);
+  hop_half<MU, S, ADJ, FORM>(h0, h1, u, acc);
 }
 
 // One hop from the raw storage words of the neighbour spinor: FP16 spinors are projected in
 // half2 before conversion, every other precision is unpacked and projected in its arithmetic
 // type. Every Dslash form calls this, so a site's arithmetic is the same in all of them.
-template <int MU, int S, bool ADJ, bool FIRST, int SP>
+template <int MU, int S, bool ADJ, int FORM, int SP>
 __device__ __forceinline__ void hop_words(const typename SpinorIO<SP>::Word w[SpinorIO<SP>::NW],
                                           const typename SpinorIO<SP>::Real u[18], int eta,
                                           typename SpinorIO<SP>::Real acc[24]) {
   if constexpr (SP == P_F16) {
     Cx<float> h0[3], h1[3];
     project_h2<MU, S>(w, eta, h0, h1);
-    hop_half<MU, S, ADJ, FIRST>(h0, h1, u, acc);
+    hop_half<MU, S, ADJ, FORM>(h0, h1, u, acc);
   } else {
     typename SpinorIO<SP>::Real psi[24];
     SpinorIO<SP>::unpack(w, psi);
-    hop<MU, S, ADJ, FIRST>(psi, u, eta, acc);
+    hop<MU, S, ADJ, FORM>(psi, u, eta, acc);
   }
 }
 
@@ -298,7 +369,7 @@ __device__ __forceinline__ void issue_hop(const Geom& g, int h, const int nf[4],
   LinkIO<LP, NR>::load_raw(link_dir<LP, NR>(FWD ? Uout : Uin, g.Vh, MU), g.Vh, FWD ? h : n, b.u);
 }
 
-template <int K, int SP, int LP, int NR, bool DAG>
+template <int K, int SP, int LP, int NR, bool DAG, bool PACKED>
 __device__ __forceinline__ void compute_hop(const Geom& g, int t, const HopBuf<SP, LP, NR>& b,
                                             typename SpinorIO<SP>::Real acc[24]) {
   using R = typename SpinorIO<SP>::Real;
@@ -311,22 +382,23 @@ __device__ __forceinline__ void compute_hop(const Geom& g, int t, const HopBuf<S
   // backward: U_mu(x - mu)^dag psi(x - mu), projector (1 + g) for D, (1 - g) for D^dag
   const int eta = (MU == 3 && t == (FWD ? g.L[3] - 1 : 0)) ? g.t_bc : 1;
   constexpr int S = FWD ? (DAG ? 1 : -1) : (DAG ? -1 : 1);
-  hop_words<MU, S, !FWD, K == 0 && FirstSets<SP>::value, SP>(b.s, u, eta, acc);
+  constexpr int FORM = (K == 0 && FirstSets<SP>::value) ? HOP_SETS : (PACKED ? HOP_PACKED : HOP_ADDS);
+  hop_words<MU, S, !FWD, FORM, SP>(b.s, u, eta, acc);
 }
 
-template <int K, int D, int SP, int LP, int NR, bool DAG>
+template <int K, int D, int SP, int LP, int NR, bool DAG, bool PACKED>
 struct HopPipe {
   __device__ __forceinline__ static void run(const Geom& g, int h, int t, const int nf[4],
                                              const int nb[4], const void* in, const void* Uout,
                                              const void* Uin, HopBuf<SP, LP, NR> (&b)[D],
                                              typename SpinorIO<SP>::Real acc[24]) {
-    compute_hop<K, SP, LP, NR, DAG>(g, t, b[K % D], acc);
+    compute_hop<K, SP, LP, NR, DAG, PACKED>(g, t, b[K % D], acc);
     if (K + D < 8) issue_hop<(K + D < 8 ? K + D : 0), SP, LP, NR>(g, h, nf, nb, in, Uout, Uin, b[K % D]);
-    HopPipe<K + 1, D, SP, LP, NR, DAG>::run(g, h, t, nf, nb, in, Uout, Uin, b, acc);
+    HopPipe<K + 1, D, SP, LP, NR, DAG, PACKED>::run(g, h, t, nf, nb, in, Uout, Uin, b, acc);
   }
 };
-template <int D, int SP, int LP, int NR, bool DAG>
-struct HopPipe<8, D, SP, LP, NR, DAG> {
+template <int D, int SP, int LP, int NR, bool DAG, bool PACKED>
+struct HopPipe<8, D, SP, LP, NR, DAG, PACKED> {
   __device__ __forceinline__ static void run(const Geom&, int, int, const int*, const int*,
                                              const void*, const void*, const void*,
                                              HopBuf<SP, LP, NR> (&)[D],
@@ -349,7 +421,7 @@ struct HopPrologue<D, D, SP, LP, NR> {
 };
 
 // acc = (D_{p,1-p} in)(h) for output parity p. Uout: links of parity p, Uin: links of 1-p.
-template <int SP, int LP, int NR, bool DAG>
+template <int SP, int LP, int NR, bool DAG, bool PACKED>
 __device__ __forceinline__ void dslash_site(const Geom& g, int h, int out_par, const void* in,
                                             const void* Uout, const void* Uin,
                                             typename SpinorIO<SP>::Real acc[24]) {
@@ -362,7 +434,7 @@ __device__ __forceinline__ void dslash_site(const Geom& g, int h, int out_par, c
 #pragma unroll
     for (int i = 0; i < 24; ++i) acc[i] = 0;
   }
-  HopPipe<0, D, SP, LP, NR, DAG>::run(g, h, t, nf, nb, in, Uout, Uin, b, acc);
+  HopPipe<0, D, SP, LP, NR, DAG, PACKED>::run(g, h, t, nf, nb, in, Uout, Uin, b, acc);
 }
 
 // ---------------------------------------------------------------- colour-split form
@@ -401,13 +473,6 @@ struct ProjShare {
 // S a on both lanes
 template <int S>
 __device__ __forceinline__ df64x2 df2_sgn(df64x2 a) { return S > 0 ? a : df2_neg(a); }
-// (S a, -S b) of the lanes (a, b)
-template <int S>
-__device__ __forceinline__ f32x2 p_alt(f32x2 v) {
-  float a, b;
-  p_unpack(v, a, b);
-  return S > 0 ? p_pack(a, -b) : p_pack(-a, b);
-}
 template <int S>
 __device__ __forceinline__ df64x2 df2_alt(df64x2 a) { return {p_alt<S>(a.hi), p_alt<S>(a.lo)}; }
 __device__ __forceinline__ f32x2 p_swap(f32x2 v) {

@@ -188,7 +188,8 @@ __device__ __forceinline__ void dslash_tile(const Launch& L, int slot, int start
   double v0 = 0.0, v1 = 0.0, v2 = 0.0;
   if (h < w.g.Vh) {
     R acc[24];
-    dslash_site<SP, LP, NR, DAG>(w.g, h, w.out_par, w.in, w.Uout, w.Uin, acc);
+    constexpr bool packed = std::is_same<R, float>::value && !(SP == P_F16 && NR == 12 && EPI == EPI_PLAIN);
+    dslash_site<SP, LP, NR, DAG, packed>(w.g, h, w.out_par, w.in, w.Uout, w.Uin, acc);
     dslash_epilogue<SP, EPI>(w, h, acc, v0, v1, v2);
   }
   if constexpr (EpiTraits<EPI>::red)
@@ -292,7 +293,7 @@ struct MrhsPipe {
     mrhs_load_link<NR>(s, K, u);
     const int eta = (MU == 3 && t == (FWD ? g.L[3] - 1 : 0)) ? g.t_bc : 1;
     constexpr int S = FWD ? (DAG ? 1 : -1) : (DAG ? -1 : 1);
-    hop_words<MU, S, !FWD, false, SP>(b[K % D], u, eta, acc);
+    hop_words<MU, S, !FWD, HOP_ADDS, SP>(b[K % D], u, eta, acc);
     if (K + D < 8) {
       constexpr int KN = (K + D < 8) ? K + D : 0;
       IO::load_raw(in, g.Vh, (KN % 2 == 0) ? nf[KN / 2] : nb[KN / 2], b[K % D]);
