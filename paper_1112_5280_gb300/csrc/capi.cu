@@ -119,8 +119,8 @@ cudaError_t ctx_malloc(lqcd_ctx* c, void** out, size_t bytes) {
 cudaError_t ctx_alloc(lqcd_ctx* c, void** out, size_t bytes) {
   if (!capturing(c)) {
     std::lock_guard<std::mutex> lk(c->pool_mu);
-    auto it = c->pool.find(bytes);
-    if (it != c->pool.end()) {
+    for (auto it = c->pool.end(); it != c->pool.begin();) {
+      if ((--it)->first != bytes) continue;
       *out = it->second;
       c->pool.erase(it);
       c->pool_bytes -= bytes;
@@ -132,15 +132,18 @@ cudaError_t ctx_alloc(lqcd_ctx* c, void** out, size_t bytes) {
 
 void ctx_free(lqcd_ctx* c, void* p, size_t bytes) {
   if (!p) return;
-  if (!capturing(c)) {
-    std::lock_guard<std::mutex> lk(c->pool_mu);
-    if (c->pool_bytes + bytes <= POOL_BYTES) {
-      c->pool.insert({bytes, p});
-      c->pool_bytes += bytes;
-      return;
-    }
+  if (bytes > POOL_BYTES || capturing(c)) {
+    cudaFree(p);
+    return;
   }
-  cudaFree(p);
+  std::lock_guard<std::mutex> lk(c->pool_mu);
+  while (c->pool_bytes + bytes > POOL_BYTES) {  // the oldest make room
+    cudaFree(c->pool.front().second);
+    c->pool_bytes -= c->pool.front().first;
+    c->pool.pop_front();
+  }
+  c->pool.push_back({bytes, p});
+  c->pool_bytes += bytes;
 }
 
 bool ctx_pool_release(lqcd_ctx* c) {

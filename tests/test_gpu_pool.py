@@ -55,3 +55,21 @@ def test_pool_is_bounded_and_given_back():
     ctx.release_cache()
     assert empty - _free() <= 32 << 20
     ctx.close()
+
+
+def test_newest_buffers_stay():
+    """A full pool makes room for the buffers freed last."""
+    ctx = lqcd.Context(0)
+    large, small = (16, 16, 16, 32), (8, 8, 8, 16)
+    old = [ctx.field(large, "f64") for _ in range(50)]  # 1.26 GB
+    for f in old:
+        f.close()
+    keep = [ctx.field(small, "f64") for _ in range(8)]
+    for f in keep:
+        f.close()
+    before = _free()
+    again = [ctx.field(small, "f64") for _ in range(8)]
+    assert _free() == before  # from the pool
+    for f in again:
+        f.close()
+    ctx.close()
