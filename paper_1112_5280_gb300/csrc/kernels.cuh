@@ -26,18 +26,30 @@ struct EpiTraits {
 #define LQCD_DSLASH_MIN_BLOCKS 6
 #endif
 // FP16 / BF16 spinors: the same bytes in flight come from half the words, so the half
-// precisions take a higher occupancy target: 10 CTAs per SM (96 registers). Measured on
-// GB300 against 6: the plain operator at 32^3x64 unchanged (70.3 against 70.2 us), the
-// solvers' linear epilogue 71.0 against 87.2 us despite a 148-byte spill, the 32^3x64 mixed
-// CG 1.6% (FP16) and 2.0% (BF16) faster, twisted FP16 CG 4.6%.
+// precisions take a higher occupancy target: 10 CTAs per SM (96 registers) for BF16 and for the
+// plain FP16-12 operator, 8 (128 registers) for the other FP16 kernels, whose hops are packed
+// (dslash.cuh) and spill at 96. Measured for FP16 at 8 against 10: the 32^3x64 FP16-12 CG 47.2
+// against 48.2 ms, the 16^3x32 twisted one 58.7 against 61.5 us an iteration, 12 sources at
+// 24^3x48 184.2 against 189.2 ms, FP16-18 32^3x64 73.8 against 75.3 us; the plain FP16-12 M-hat
+// there 151.3 against 149.5 (its small launches: go_dslash). BF16-12 at 8: 70.1 against 69.0. At 12 (80 registers) all lose.
 #ifndef LQCD_DSLASH_MIN_BLOCKS_HALF
 #define LQCD_DSLASH_MIN_BLOCKS_HALF 10
 #endif
+#ifndef LQCD_DSLASH_MIN_BLOCKS_F16
+#define LQCD_DSLASH_MIN_BLOCKS_F16 8
+#endif
+// the plain FP16-12 operator, which keeps the scalar hops
+template <int SP, int NR, int EPI>
+struct ScalarF16 {
+  static constexpr bool value = SP == P_F16 && NR == 12 && EPI == EPI_PLAIN;
+};
 // Double-float needs the full 255 registers per thread (4 CTAs of 64 threads).
-template <int SP>
+template <int SP, int NR, int EPI>
 struct DslashMinBlocks {
-  static constexpr int value =
-      (SP == P_DF64) ? 4 : ((SP == P_F16 || SP == P_BF16) ? LQCD_DSLASH_MIN_BLOCKS_HALF : LQCD_DSLASH_MIN_BLOCKS);
+  static constexpr int value = SP == P_DF64 ? 4
+                               : SP == P_BF16 || ScalarF16<SP, NR, EPI>::value ? LQCD_DSLASH_MIN_BLOCKS_HALF
+                               : SP == P_F16 ? LQCD_DSLASH_MIN_BLOCKS_F16
+                                             : LQCD_DSLASH_MIN_BLOCKS;
 };
 // The second register budget of the FP32 Dslash (launch form 3): 8 CTAs per SM, 128
 // registers per thread. More warps with fewer hops in flight each; it pays where the
@@ -188,7 +200,7 @@ __device__ __forceinline__ void dslash_tile(const Launch& L, int slot, int start
   double v0 = 0.0, v1 = 0.0, v2 = 0.0;
   if (h < w.g.Vh) {
     R acc[24];
-    constexpr bool packed = std::is_same<R, float>::value && !(SP == P_F16 && NR == 12 && EPI == EPI_PLAIN);
+    constexpr bool packed = std::is_same<R, float>::value && !ScalarF16<SP, NR, EPI>::value;
     dslash_site<SP, LP, NR, DAG, packed>(w.g, h, w.out_par, w.in, w.Uout, w.Uin, acc);
     dslash_epilogue<SP, EPI>(w, h, acc, v0, v1, v2);
   }
@@ -200,7 +212,7 @@ __device__ __forceinline__ void dslash_tile(const Launch& L, int slot, int start
 // view), and over all tiles otherwise, so that operator launches run the plain loop without
 // the view's branches and without shared memory (measured: one loop with a static view cost
 // 1.3% more instructions and 2-3% of the headline launch).
-template <int SP, int LP, int NR, bool DAG, int EPI, int MB = DslashMinBlocks<SP>::value>
+template <int SP, int LP, int NR, bool DAG, int EPI, int MB = DslashMinBlocks<SP, NR, EPI>::value>
 __global__ void __launch_bounds__(TILE, MB) k_dslash(const Launch L) {
   pdl_wait();
   int block, stride;

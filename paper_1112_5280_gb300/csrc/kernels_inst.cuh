@@ -74,6 +74,15 @@ cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
       return launch_k(fh, dim3(grid + fin_ctas(L)), dim3(TILE), view_smem(L), s, L);
     }
   }
+  // up to one wave at 8 CTAs per SM the plain FP16-12 operator gains by the larger register
+  // budget too (16^3x32 7.4 -> 6.5 us), beyond it loses (32^3x64 M-hat 149.5 -> 151.3)
+  if constexpr (ScalarF16<SPX, NR, EPI>::value) {
+    if (L.ntiles <= LQCD_DSLASH_MIN_BLOCKS_F16 * device_sm_count()) {
+      auto fs = k_dslash<SPX, LPX, NR, DAG, EPI, LQCD_DSLASH_MIN_BLOCKS_F16>;
+      if (grid <= 0) grid = grid_for((const void*)fs, L.ntiles, 0, TILE, cps);
+      return launch_k(fs, dim3(grid + fin_ctas(L)), dim3(TILE), view_smem(L), s, L);
+    }
+  }
   if constexpr (!split_only) {
     auto fn = k_dslash<SPX, LPX, NR, DAG, EPI>;
     if (grid <= 0) grid = grid_for((const void*)fn, L.ntiles, 0, TILE, cps);
@@ -197,7 +206,7 @@ int site_occupancy_12() {
   if constexpr (P == P_DF64) {
     return 0;
   } else {
-    return kernel_occupancy((const void*)k_dslash<P, LPX, 12, false, EPI_LIN>, TILE);
+    return kernel_occupancy((const void*)k_dslash<P, LPX, 12, false, P == P_F16 ? EPI_PLAIN : EPI_LIN>, TILE);
   }
 }
 }  // namespace

@@ -27,3 +27,22 @@ def test_packed_hops_equal_scalar_hops(dims, t_bc, prec, compress):
     for a, b in zip(got[0][1], got[1][1]):
         assert np.array_equal(a, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("dagger", [False, True])
+def test_plain_f16_12_either_side_of_one_wave(dagger):
+    """Operators of up to 8 CTAs per SM and larger launches use two register budgets: one
+    16^3x32 application (1024 tiles) against two in a batch (2048), bit for bit."""
+    dims = (16, 16, 16, 32)
+    ctx = lqcd.Context(0)
+    g = ctx.gauge(dims, synth.random_links(dims, 0.5, seed=71), "f16", 12)
+    ins = [ctx.field(dims, "f16", lqcd.EVEN, synth.gaussian_spinor(dims, seed=72 + k)) for k in range(2)]
+    outs = [ctx.field(dims, "f16", lqcd.ODD) for _ in range(4)]
+    batch = lqcd.DslashBatch([g, g], ins, outs[:2], 1, dagger)
+    batch.apply()
+    for k in range(2):
+        lqcd.dslash_eo(g, ins[k], outs[2 + k], 1, dagger)
+        a, b = outs[k].download(), outs[2 + k].download()
+        assert np.array_equal(a, b) and np.abs(a).max() > 1
+    batch.close()
+    ctx.close()
