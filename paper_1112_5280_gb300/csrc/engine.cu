@@ -426,10 +426,47 @@ cudaError_t issue_iteration_block(lqcd_engine* e, int iters, bool capturing) {
   return cudaSuccess;
 }
 
+// Captures one chunk of iterations and makes it the engine's graph. After a failure the
+// engine has no key, so that the next rebuild captures again.
+int capture_chunk(lqcd_engine* e) {
+  cudaStream_t st = e->ctx->stream;
+  e->exec_key.clear();
+  cudaGraph_t graph = nullptr;
+  cudaError_t err = cudaSuccess;
+  if (!e->body_stream) err = cudaStreamCreateWithFlags(&e->body_stream, cudaStreamNonBlocking);
+  if (err == cudaSuccess) err = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+  if (err == cudaSuccess) {
+    err = issue_iteration_block(e, e->opts.chunk, true);
+    pdl_skip_next(false);
+    const cudaError_t end = cudaStreamEndCapture(st, &graph);
+    if (err == cudaSuccess) err = end;
+  }
+  if (err == cudaSuccess && e->exec) {
+    cudaGraphExecUpdateResultInfo info;
+    if (cudaGraphExecUpdate(e->exec, graph, &info) != cudaSuccess) {
+      cudaGetLastError();
+      cudaGraphExecDestroy(e->exec);
+      e->exec = nullptr;
+    }
+  }
+  if (err == cudaSuccess && !e->exec) {
+    err = cudaGraphInstantiate(&e->exec, graph, 0);
+    if (err != cudaSuccess) e->exec = nullptr;
+  }
+  if (graph) cudaGraphDestroy(graph);
+  if (err == cudaSuccess) return LQCD_OK;
+  cudaGetLastError();  // reported here; not the next launch's error
+  return set_error(LQCD_ECUDA, "iteration graph: %s", cudaGetErrorString(err));
+}
+
+// The tables and the graph of the active slots. The engine stays dirty until both stand: the
+// graph of another slot list must not run over these tables.
 int rebuild(lqcd_engine* e) {
   const int n = (int)e->active.size();
-  e->dirty = false;
-  if (n == 0) return LQCD_OK;
+  if (n == 0) {
+    e->dirty = false;
+    return LQCD_OK;
+  }
   // interleave tiles when every slot solves on the same gauge field (multi-RHS):
   // consecutive tiles then share links, which stream from HBM once per site block
   const lqcd_gauge* g0 = e->reqs[e->active[0]].gauge;
@@ -506,38 +543,14 @@ int rebuild(lqcd_engine* e) {
     for (int s = 0; s < NSTEP; ++s) key.push_back(batch_launch(e, s));
     const std::vector<unsigned> opts = {(unsigned)e->ru_every, e->any_twist, e->any_normal, e->any_plain,
                                         launch_config_epoch(), pdl_enabled()};
-    if (e->exec && opts == e->exec_opts && key.size() == e->exec_key.size() &&
-        !memcmp(key.data(), e->exec_key.data(), key.size() * sizeof(Launch)))
-      return LQCD_OK;
-    e->exec_key.clear();
-    if (!e->body_stream) LQCD_CK(cudaStreamCreateWithFlags(&e->body_stream, cudaStreamNonBlocking));
-    cudaGraph_t graph = nullptr;
-    LQCD_CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    cudaError_t err = issue_iteration_block(e, e->opts.chunk, true);
-    pdl_skip_next(false);
-    cudaError_t err2 = cudaStreamEndCapture(st, &graph);
-    if (err != cudaSuccess) return set_error(LQCD_ECUDA, "capture: %s", cudaGetErrorString(err));
-    if (err2 != cudaSuccess) return set_error(LQCD_ECUDA, "end capture: %s", cudaGetErrorString(err2));
-    if (e->exec) {
-      cudaGraphExecUpdateResultInfo info;
-      if (cudaGraphExecUpdate(e->exec, graph, &info) != cudaSuccess) {
-        cudaGetLastError();
-        cudaGraphExecDestroy(e->exec);
-        e->exec = nullptr;
-      }
+    if (!e->exec || opts != e->exec_opts || key.size() != e->exec_key.size() ||
+        memcmp(key.data(), e->exec_key.data(), key.size() * sizeof(Launch))) {
+      LQCD_TRY(capture_chunk(e));
+      e->exec_key = key;
+      e->exec_opts = opts;
     }
-    if (!e->exec) {
-      cudaError_t ie = cudaGraphInstantiate(&e->exec, graph, 0);
-      if (ie != cudaSuccess) {
-        cudaGraphDestroy(graph);
-        e->exec = nullptr;
-        return set_error(LQCD_ECUDA, "graph instantiate: %s", cudaGetErrorString(ie));
-      }
-    }
-    cudaGraphDestroy(graph);
-    e->exec_key = key;
-    e->exec_opts = opts;
   }
+  e->dirty = false;
   return LQCD_OK;
 }
 
