@@ -105,9 +105,11 @@ LQCD_API long long lqcd_ctx_launch_count(const lqcd_ctx* ctx);
  * BiCGStab vectors; operator and upload temporaries), so repeated solves
  * allocate nothing, and up to 1 GiB of the buffers of destroyed fields, gauge
  * fields and momenta, for the next ones of the same size (given back also when
- * an allocation for the context fails). This waits for the context's stream and
- * frees them; the next call allocates again. Objects the caller created are
- * untouched. */
+ * an allocation for the context fails). Once a call of the context was captured
+ * into a graph, or another context copied from a field of this one, destroyed
+ * objects are freed at once, after all work on the device. This waits for the
+ * context's stream and frees them; the next call allocates again. Objects the
+ * caller created are untouched. */
 LQCD_API int lqcd_ctx_release_cache(lqcd_ctx* ctx);
 
 /* ---------------------------------------------------------------- gauge field (A1) */

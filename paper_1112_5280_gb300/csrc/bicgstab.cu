@@ -75,7 +75,7 @@ int lqcd::bicgstab_solve(const lqcd_gauge* g, const lqcd_field* src, double kapp
   auto tw_inv = [&](Work& w) { if (ta != 0.0) set_twist(w, ts, -ta, 0.0); };
   auto tw_a = [&](Work& w) { if (ta != 0.0) set_twist(w, 1.0, 0.0, ta); };
   lqcd_ctx* c = g->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   cudaStream_t st = c->stream;
   const Geom gm = g->g;
   const int Vh = gm.Vh;

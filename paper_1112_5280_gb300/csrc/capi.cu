@@ -107,6 +107,12 @@ static bool capturing(const lqcd_ctx* c) {
   return st != cudaStreamCaptureStatusNone;
 }
 
+int ctx_enter(lqcd_ctx* c) {
+  LQCD_CK(cudaSetDevice(c->device));
+  if (!c->used_elsewhere && capturing(c)) c->used_elsewhere = true;
+  return LQCD_OK;
+}
+
 cudaError_t ctx_malloc(lqcd_ctx* c, void** out, size_t bytes) {
   cudaError_t e = cudaMalloc(out, bytes);
   if (e == cudaErrorMemoryAllocation && ctx_pool_release(c)) {
@@ -132,7 +138,7 @@ cudaError_t ctx_alloc(lqcd_ctx* c, void** out, size_t bytes) {
 
 void ctx_free(lqcd_ctx* c, void* p, size_t bytes) {
   if (!p) return;
-  if (bytes > POOL_BYTES || capturing(c)) {
+  if (bytes > POOL_BYTES || c->used_elsewhere || capturing(c)) {
     cudaFree(p);
     return;
   }
@@ -199,11 +205,6 @@ Launch single_launch(const Work& w, double* partials) {
 
 using namespace lqcd;
 
-static int ctx_set_device(lqcd_ctx* c) {
-  LQCD_CK(cudaSetDevice(c->device));
-  return LQCD_OK;
-}
-
 extern "C" {
 
 const char* lqcd_status_string(int s) {
@@ -233,7 +234,8 @@ int lqcd_ctx_create(lqcd_ctx** out, int device, void* stream) {
   if (device < 0 || device >= n) return set_error(LQCD_EINVAL, "device %d of %d", device, n);
   lqcd_ctx* c = new lqcd_ctx();
   c->device = device;
-  int rc = ctx_set_device(c);
+  cudaError_t dev = cudaSetDevice(device);
+  int rc = dev == cudaSuccess ? LQCD_OK : set_error(LQCD_ECUDA, "device %d: %s", device, cudaGetErrorString(dev));
   if (rc == LQCD_OK) {
     cudaError_t e = cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) rc = set_error(LQCD_ECUDA, "stream: %s", cudaGetErrorString(e));
@@ -287,7 +289,7 @@ extern "C" {
 int lqcd_ctx_set_stream(lqcd_ctx* c, void* stream) {
   clear_error();
   if (!c) return set_error(LQCD_EINVAL, "ctx is NULL");
-  LQCD_TRY(ctx_set_device(c));
+  LQCD_TRY(ctx_enter(c));
   LQCD_CK(cudaStreamSynchronize(c->stream));
   c->stream = stream ? (cudaStream_t)stream : c->own_stream;
   return LQCD_OK;
@@ -298,7 +300,7 @@ void* lqcd_ctx_stream(const lqcd_ctx* c) { return c ? (void*)c->stream : nullptr
 int lqcd_ctx_sync(lqcd_ctx* c) {
   clear_error();
   if (!c) return set_error(LQCD_EINVAL, "ctx is NULL");
-  LQCD_TRY(ctx_set_device(c));
+  LQCD_TRY(ctx_enter(c));
   LQCD_CK(cudaStreamSynchronize(c->stream));
   return LQCD_OK;
 }
@@ -310,7 +312,7 @@ int lqcd_debug_bounds(lqcd_ctx* c, unsigned long long* word) {
   if (!c || !word) return set_error(LQCD_EINVAL, "NULL argument");
   *word = 0;
 #ifdef LQCD_DEBUG_BOUNDS
-  LQCD_TRY(ctx_set_device(c));
+  LQCD_TRY(ctx_enter(c));
   LQCD_CK(cudaStreamSynchronize(c->stream));
   for (auto read : bounds_word_readers()) {
     unsigned long long v = 0;
@@ -326,7 +328,7 @@ int lqcd_debug_bounds(lqcd_ctx* c, unsigned long long* word) {
 int lqcd_ctx_release_cache(lqcd_ctx* c) {
   clear_error();
   if (!c) return set_error(LQCD_EINVAL, "NULL context");
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   LQCD_CK(cudaStreamSynchronize(c->stream));
   ctx_drop_engine(c);
   ctx_pool_release(c);
@@ -363,7 +365,7 @@ static int gauge_upload_impl(lqcd_ctx* c, const int dims[4], const double* U, bo
   if (compress != 18 && compress != 12) return set_error(LQCD_EINVAL, "compress must be 18 or 12");
   Geom g;
   LQCD_TRY(make_geom(dims, t_bc, g));
-  LQCD_TRY(ctx_set_device(c));
+  LQCD_TRY(ctx_enter(c));
   const size_t aos_bytes = (size_t)2 * g.Vh * 4 * 18 * sizeof(double);
   const double* src = U;
   if (!dev) {
@@ -420,7 +422,7 @@ int lqcd_gauge_add_copy(lqcd_gauge* g, int prec, int compress) {
   if (!g) return set_error(LQCD_EINVAL, "gauge is NULL");
   if (prec < LQCD_F64 || prec > LQCD_DF64) return set_error(LQCD_EINVAL, "precision %d", prec);
   if (compress != 18 && compress != 12) return set_error(LQCD_EINVAL, "compress must be 18 or 12");
-  LQCD_TRY(ctx_set_device(g->ctx));
+  LQCD_TRY(ctx_enter(g->ctx));
   const int lp = link_prec_for(prec);
   if (lp < 0 || lp >= NPREC) return set_error(LQCD_EINVAL, "link precision %d", lp);
   if (lp == P_DF64) compress = 18;  // double-float links keep 18 reals
@@ -460,7 +462,7 @@ int lqcd_field_create(lqcd_ctx* c, const int dims[4], int prec, int subset, lqcd
   if (subset < LQCD_EVEN || subset > LQCD_FULL) return set_error(LQCD_EINVAL, "subset %d", subset);
   Geom g;
   LQCD_TRY(make_geom(dims, -1, g));
-  LQCD_TRY(ctx_set_device(c));
+  LQCD_TRY(ctx_enter(c));
   lqcd_field* f = new lqcd_field();
   f->ctx = c;
   ctx_retain(c);
@@ -499,7 +501,7 @@ static int field_upload_impl(lqcd_field* f, const double* psi, bool dev) {
   clear_error();
   if (!f || !psi) return set_error(LQCD_EINVAL, "NULL argument");
   lqcd_ctx* c = f->ctx;
-  LQCD_TRY(ctx_set_device(c));
+  LQCD_TRY(ctx_enter(c));
   const size_t bytes = (size_t)2 * f->g.Vh * 24 * sizeof(double);
   const double* src = psi;
   if (!dev) {
@@ -521,7 +523,7 @@ int lqcd_field_download_dev(const lqcd_field* f, double* psi) {
   LQCD_TRACE("lqcd_field_download_dev");
   clear_error();
   if (!f || !psi) return set_error(LQCD_EINVAL, "NULL argument");
-  LQCD_TRY(ctx_set_device(f->ctx));
+  LQCD_TRY(ctx_enter(f->ctx));
   LQCD_CK(spinor_to_aos(f->half[0], f->half[1], f->g, f->prec, psi, f->ctx->stream));
   return LQCD_OK;
 }
@@ -531,7 +533,7 @@ int lqcd_field_download(const lqcd_field* f, double* psi) {
   clear_error();
   if (!f || !psi) return set_error(LQCD_EINVAL, "NULL argument");
   lqcd_ctx* c = f->ctx;
-  LQCD_TRY(ctx_set_device(c));
+  LQCD_TRY(ctx_enter(c));
   const size_t V = (size_t)2 * f->g.Vh;
   const size_t bytes = V * 24 * sizeof(double);
   LQCD_TRY(ctx_staging(c, bytes));
@@ -563,7 +565,8 @@ int lqcd_field_copy(lqcd_field* dst, const lqcd_field* src, double scale) {
   if (!dst || !src) return set_error(LQCD_EINVAL, "NULL argument");
   if (dst->g.Vh != src->g.Vh || memcmp(dst->g.L, src->g.L, sizeof dst->g.L))
     return set_error(LQCD_EINVAL, "lattice mismatch");
-  LQCD_TRY(ctx_set_device(dst->ctx));
+  LQCD_TRY(ctx_enter(dst->ctx));
+  if (src->ctx != dst->ctx) src->ctx->used_elsewhere = true;
   int n = 0;
   for (int p = 0; p < 2; ++p) {
     if (!dst->half[p] || !src->half[p]) continue;
@@ -578,7 +581,7 @@ int lqcd_field_copy(lqcd_field* dst, const lqcd_field* src, double scale) {
 int lqcd_field_zero(lqcd_field* f) {
   clear_error();
   if (!f) return set_error(LQCD_EINVAL, "field is NULL");
-  LQCD_TRY(ctx_set_device(f->ctx));
+  LQCD_TRY(ctx_enter(f->ctx));
   for (auto p : f->half)
     if (p) LQCD_CK(cudaMemsetAsync(p, 0, f->half_bytes, f->ctx->stream));
   return LQCD_OK;
@@ -588,7 +591,7 @@ int lqcd_field_norm2(const lqcd_field* f, double* out) {
   clear_error();
   if (!f || !out) return set_error(LQCD_EINVAL, "NULL argument");
   lqcd_ctx* c = f->ctx;
-  LQCD_TRY(ctx_set_device(c));
+  LQCD_TRY(ctx_enter(c));
   Work w = blank_work(f->g);
   LQCD_TRY(ctx_partials(c, 3 * (size_t)w.ntiles));
   double total = 0;
@@ -670,7 +673,7 @@ int lqcd_dslash_eo(const lqcd_gauge* g, const lqcd_field* in, lqcd_field* out, i
   if (in == out && in->subset == LQCD_FULL) {
     // in and out use different halves of the same field: allowed
   }
-  LQCD_TRY(ctx_set_device(g->ctx));
+  LQCD_TRY(ctx_enter(g->ctx));
   return dslash_lin(g, in->prec, in->half[1 - out_parity], out->half[out_parity], nullptr, 1.0, 0.0,
                     out_parity, dagger != 0);
 }
@@ -702,7 +705,7 @@ int lqcd_dslash_batch_create(int n, const lqcd_gauge* const* g, const lqcd_field
   std::vector<Work> w(n);
   std::vector<int> prefix(n + 1, 0);
   bool same_vh = true;
-  LQCD_TRY(ctx_set_device(c));
+  LQCD_TRY(ctx_enter(c));
   for (int i = 0; i < n; ++i) {
     LQCD_TRY(check_pair(g[i], in[i], out[i]));
     if (g[i]->ctx != c || in[i]->prec != prec) return set_error(LQCD_EINVAL, "batch mixes contexts or precisions");
@@ -768,7 +771,7 @@ int lqcd_dslash_batch_apply(lqcd_dslash_batch* b) {
   LQCD_TRACE("lqcd_dslash_batch_apply");
   clear_error();
   if (!b) return set_error(LQCD_EINVAL, "batch is NULL");
-  LQCD_TRY(ctx_set_device(b->ctx));
+  LQCD_TRY(ctx_enter(b->ctx));
   LQCD_CK(launch_dslash(b->prec, b->nr, b->dagger != 0, EPI_LIN, b->L, 0, b->ctx->stream));
   b->ctx->launches++;
   return LQCD_OK;
@@ -804,7 +807,7 @@ int lqcd_apply_Mhat_tm(const lqcd_gauge* g, double kappa, double mu, const lqcd_
   if (!in->half[0] || !out->half[0]) return set_error(LQCD_EINVAL, "fields must hold the even parity");
   if (in->half[0] == out->half[0]) return set_error(LQCD_EINVAL, "in and out must differ");
   lqcd_ctx* c = g->ctx;
-  LQCD_TRY(ctx_set_device(c));
+  LQCD_TRY(ctx_enter(c));
   LQCD_TRY(ctx_tmp(c, half_spinor_bytes(in->prec, g->g.Vh)));
   if (mu == 0.0) {
     LQCD_TRY(dslash_lin(g, in->prec, in->half[0], c->tmp, nullptr, 1.0, 0.0, 1, dagger != 0));
@@ -828,7 +831,7 @@ int lqcd_apply_M_tm(const lqcd_gauge* g, double kappa, double mu, const lqcd_fie
   if (in->subset != LQCD_FULL || out->subset != LQCD_FULL)
     return set_error(LQCD_EINVAL, "apply_M needs FULL fields");
   if (in == out) return set_error(LQCD_EINVAL, "in and out must differ");
-  LQCD_TRY(ctx_set_device(g->ctx));
+  LQCD_TRY(ctx_enter(g->ctx));
   const double a = (dagger ? -2.0 : 2.0) * kappa * mu;  // A (A^dag)
   for (int p = 0; p < 2; ++p) {
     if (mu == 0.0)

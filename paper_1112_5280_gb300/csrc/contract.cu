@@ -259,7 +259,7 @@ extern "C" int lqcd_meson_correlator(const lqcd_field* const* props, int ngamma,
     tab.use |= 1 << x;
   }
   lqcd_ctx* c = f0->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   const Geom& g = f0->g;
   Props props_arg;
   for (int i = 0; i < 12; ++i)

@@ -692,7 +692,7 @@ int lqcd_engine_create(lqcd_ctx* c, const lqcd_solve_opts* opts, size_t budget, 
   if (o.sloppy_compress != 12 && o.sloppy_compress != 18) return set_error(LQCD_EINVAL, "sloppy compress");
   if (o.maxiter < 1) o.maxiter = 50000;
   if (o.chunk < 1) o.chunk = 8;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   lqcd_engine* e = new lqcd_engine();
   e->ctx = c;
   ctx_retain(c);
@@ -795,7 +795,7 @@ static int submit_impl(lqcd_engine* e, const lqcd_gauge* gauge, const lqcd_field
   if (!(tol > 0) || !(kappa >= 0)) return set_error(LQCD_EINVAL, "tol must be > 0 and kappa >= 0");
   if (gauge->ctx != e->ctx || src->ctx != e->ctx) return set_error(LQCD_EINVAL, "context mismatch");
   lqcd_ctx* c = e->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   const size_t need = slot_bytes(e, gauge->g.Vh);
   if (e->budget && need > e->budget) return set_error(LQCD_ENOMEM, "request needs %zu bytes > budget %zu", need, e->budget);
   if (e->free_slots.empty()) return set_error(LQCD_EBUSY, "no free slot");
@@ -942,7 +942,7 @@ int lqcd_engine_step(lqcd_engine* e, int* n_active) {
   clear_error();
   if (!e) return set_error(LQCD_EINVAL, "engine is NULL");
   lqcd_ctx* c = e->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   cudaStream_t st = c->stream;
   if (!e->active.empty()) {
     if (e->dirty) {
@@ -1021,7 +1021,7 @@ int lqcd_engine_result(lqcd_engine* e, long long id, lqcd_field* x, lqcd_solve_i
   Request& q = it->second;
   PdlSolverScope pdl_scope(pdl_solver_off(q.ntiles));  // large launches: no PDL
   if (!q.finished) return set_error(LQCD_EBUSY, "request %lld still running", id);
-  LQCD_CK(cudaSetDevice(e->ctx->device));
+  LQCD_TRY(ctx_enter(e->ctx));
   if (x) {
     if (x->subset != LQCD_FULL || memcmp(x->g.L, q.g.L, sizeof q.g.L))
       return set_error(LQCD_EINVAL, "x must be a FULL field of the request's lattice");
@@ -1047,7 +1047,7 @@ int lqcd_engine_cancel(lqcd_engine* e, long long id, int status) {
   if (it == e->reqs.end()) return set_error(LQCD_EINVAL, "unknown request %lld", id);
   if (status >= 0) return set_error(LQCD_EINVAL, "cancel status must be a negative LQCD_E* code");
   if (it->second.finished) return LQCD_OK;
-  LQCD_CK(cudaSetDevice(e->ctx->device));
+  LQCD_TRY(ctx_enter(e->ctx));
   k_slot_cancel<<<1, 1, 0, e->ctx->stream>>>(e->d_sc + it->second.slot, status);
   LQCD_CK(cudaGetLastError());
   return LQCD_OK;

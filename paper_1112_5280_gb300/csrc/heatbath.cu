@@ -372,7 +372,7 @@ int lqcd_heatbath(lqcd_gauge* g, double beta, int nsweeps, unsigned long long se
   if (!(beta >= 0.0) || !std::isfinite(beta)) return set_error(LQCD_EINVAL, "beta must be finite and >= 0");
   if (nsweeps < 0) return set_error(LQCD_EINVAL, "nsweeps %d", nsweeps);
   lqcd_ctx* c = g->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   cudaStream_t st = c->stream;
   LQCD_TRY(ctx_partials(c, 1));
   unsigned long long* d_fails = reinterpret_cast<unsigned long long*>(c->partials);
@@ -416,7 +416,7 @@ int lqcd_plaquette(const lqcd_gauge* g, double* plaq) {
   clear_error();
   if (!g || !plaq) return set_error(LQCD_EINVAL, "NULL argument");
   lqcd_ctx* c = g->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   cudaStream_t st = c->stream;
   const int nb = (int)((2LL * g->g.Vh + PLAQ_THREADS - 1) / PLAQ_THREADS);
   const int n = 6 * nb;
@@ -437,7 +437,7 @@ int lqcd_gauge_download(const lqcd_gauge* g, double* host_U) {
   clear_error();
   if (!g || !host_U) return set_error(LQCD_EINVAL, "NULL argument");
   lqcd_ctx* c = g->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   const size_t bytes = (size_t)2 * g->g.Vh * 4 * 18 * sizeof(double);
   LQCD_TRY(ctx_staging(c, bytes));
   LQCD_CK(links_to_aos(static_cast<const double2*>(g->copy[P_F64][0]), g->g,

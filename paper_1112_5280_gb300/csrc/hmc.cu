@@ -491,7 +491,7 @@ int lqcd_mom_create(lqcd_ctx* c, const int dims[4], lqcd_mom** out) {
   *out = nullptr;
   Geom g;
   LQCD_TRY(make_geom(dims, -1, g));
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   lqcd_mom* m = new lqcd_mom();
   m->ctx = c;
   m->g = g;
@@ -527,7 +527,7 @@ int lqcd_mom_upload(lqcd_mom* m, const double* host) {
   clear_error();
   if (!m || !host) return set_error(LQCD_EINVAL, "NULL argument");
   lqcd_ctx* c = m->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   LQCD_TRY(ctx_staging(c, m->bytes));
   LQCD_CK(cudaMemcpyAsync(c->staging, host, m->bytes, cudaMemcpyHostToDevice, c->stream));
   LQCD_CK(links_from_aos(c->staging, m->g, m->d, c->stream));
@@ -540,7 +540,7 @@ int lqcd_mom_download(const lqcd_mom* m, double* host) {
   clear_error();
   if (!m || !host) return set_error(LQCD_EINVAL, "NULL argument");
   lqcd_ctx* c = m->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   LQCD_TRY(ctx_staging(c, m->bytes));
   LQCD_CK(links_to_aos(m->d, m->g, reinterpret_cast<double2*>(c->staging), c->stream));
   c->launches++;
@@ -552,7 +552,7 @@ int lqcd_mom_download(const lqcd_mom* m, double* host) {
 int lqcd_mom_zero(lqcd_mom* m) {
   clear_error();
   if (!m) return set_error(LQCD_EINVAL, "NULL argument");
-  LQCD_CK(cudaSetDevice(m->ctx->device));
+  LQCD_TRY(ctx_enter(m->ctx));
   LQCD_CK(cudaMemsetAsync(m->d, 0, m->bytes, m->ctx->stream));
   return LQCD_OK;
 }
@@ -561,7 +561,7 @@ int lqcd_mom_kinetic(const lqcd_mom* m, double* energy) {
   LQCD_TRACE("lqcd_mom_kinetic");
   clear_error();
   if (!m || !energy) return set_error(LQCD_EINVAL, "NULL argument");
-  LQCD_CK(cudaSetDevice(m->ctx->device));
+  LQCD_TRY(ctx_enter(m->ctx));
   return kinetic_impl(m, energy);
 }
 
@@ -570,7 +570,7 @@ int lqcd_gauge_force(const lqcd_gauge* g, double beta, double coeff, lqcd_mom* m
   clear_error();
   LQCD_TRY(check_mom(g, m));
   if (!std::isfinite(beta) || !std::isfinite(coeff)) return set_error(LQCD_EINVAL, "beta and coeff must be finite");
-  LQCD_CK(cudaSetDevice(g->ctx->device));
+  LQCD_TRY(ctx_enter(g->ctx));
   return gauge_force_impl(g, beta, coeff, m);
 }
 
@@ -585,7 +585,7 @@ int lqcd_fermion_force(const lqcd_gauge* g, double kappa, double mu, const lqcd_
   if (!std::isfinite(kappa) || !std::isfinite(mu) || !std::isfinite(coeff))
     return set_error(LQCD_EINVAL, "kappa, mu and coeff must be finite");
   lqcd_ctx* c = g->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   int dims[4] = {g->g.L[0], g->g.L[1], g->g.L[2], g->g.L[3]};
   lqcd_field *xx = nullptr, *y = nullptr, *xd = nullptr, *yd = nullptr;
   int rc = lqcd_field_create(c, dims, LQCD_F64, LQCD_FULL, &xx);
@@ -603,7 +603,7 @@ int lqcd_gauge_update(lqcd_gauge* g, const lqcd_mom* m, double eps) {
   clear_error();
   LQCD_TRY(check_mom(g, m));
   if (!std::isfinite(eps)) return set_error(LQCD_EINVAL, "eps must be finite");
-  LQCD_CK(cudaSetDevice(g->ctx->device));
+  LQCD_TRY(ctx_enter(g->ctx));
   return update_links(g, m, eps, true);
 }
 
@@ -655,7 +655,7 @@ int lqcd_hmc_trajectory(lqcd_gauge* g, const lqcd_hmc_params* p, lqcd_mom* m, co
       !std::isfinite(p->kappa) || !std::isfinite(p->mu) || p->chrono < 0 || p->chrono > 2)
     return set_error(LQCD_EINVAL, "bad HMC parameters");
   lqcd_ctx* c = g->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   lqcd_solve_opts o;
   lqcd_solve_opts_default(&o);
   if (opts) o = *opts;

@@ -129,7 +129,7 @@ extern "C" int lqcd_apply_Mhat_noalloc(const lqcd_gauge* g, double kappa, const 
                      "lqcd_apply_Mhat_noalloc: no resident %d-real link copy for this precision; "
                      "create it first with lqcd_gauge_add_copy(g, prec, %d)",
                      nr, nr);
-  LQCD_CK(cudaSetDevice(g->ctx->device));
+  LQCD_TRY(ctx_enter(g->ctx));
   void* tmp = nullptr;
   int rc = scratch_address(g->ctx->device, &tmp);
   if (rc != LQCD_OK) return rc;

@@ -96,7 +96,7 @@ extern "C" int lqcd_alu_peak(lqcd_ctx* ctx, int kind, double* tflops) {
   using namespace lqcd;
   clear_error();
   if (!ctx || !tflops) return set_error(LQCD_EINVAL, "NULL argument");
-  LQCD_CK(cudaSetDevice(ctx->device));
+  LQCD_TRY(ctx_enter(ctx));
   // about 15 ms per run at the nominal rates
   if (kind == 0) return measure<double>(ctx, 4000, tflops);
   if (kind == 1) return measure<float>(ctx, 240000, tflops);

@@ -31,6 +31,8 @@ struct lqcd_ctx {
   long long launches = 0;
   // freed field and link buffers (bytes, pointer), oldest first, for the next object of that
   // size (ctx_alloc)
+  // work on the context's objects may run outside its stream (ctx_enter, lqcd_field_copy)
+  std::atomic<bool> used_elsewhere{false};
   std::mutex pool_mu;
   std::deque<std::pair<size_t, void*>> pool;
   size_t pool_bytes = 0;
@@ -106,6 +108,9 @@ int make_geom(const int dims[4], int t_bc, Geom& g);
 size_t half_spinor_bytes(int prec, int Vh);
 size_t gauge_copy_bytes(int prec, int nr, int Vh);
 
+// Makes the context's device current at the start of a call, and notes a call that is captured.
+int ctx_enter(lqcd_ctx* c);
+
 // device buffers of the context, grown on demand (synchronises when growing)
 int ctx_partials(lqcd_ctx* c, size_t n);
 int ctx_tmp(lqcd_ctx* c, size_t bytes);
@@ -120,9 +125,11 @@ int ctx_staging(lqcd_ctx* c, size_t bytes);
 // more (so that a program that moves on to another lattice gains there too: the load and apply
 // after larger solves 719 -> 494 us). They are given back by lqcd_ctx_release_cache, with the
 // context, and when any allocation for the context fails (ctx_malloc). Whoever frees has
-// waited for the context's stream, and a change of stream waits for the old one, so a buffer
-// in the pool has no work pending. A stream in capture allocates and frees past the pool, as
-// refused or accepted by CUDA.
+// waited for the context's stream, and a change of stream waits for the old one. That is all
+// the work there is on a buffer unless a call was captured, whose graph may be in flight on any
+// stream, or another context copied from a field of this one. Such a context (used_elsewhere)
+// frees with cudaFree, which waits for the device, so a buffer in the pool has no work pending.
+// A stream in capture allocates and frees past the pool, as refused or accepted by CUDA.
 constexpr size_t POOL_BYTES = (size_t)1 << 30;
 cudaError_t ctx_malloc(lqcd_ctx* c, void** out, size_t bytes);
 cudaError_t ctx_alloc(lqcd_ctx* c, void** out, size_t bytes);

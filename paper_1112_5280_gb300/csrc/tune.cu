@@ -240,7 +240,7 @@ int lqcd_autotune_dslash(int n, const lqcd_gauge* const* g, int prec, int compre
   if (prec < LQCD_F64 || prec > LQCD_DF64) return set_error(LQCD_EINVAL, "precision %d", prec);
   if (compress != 0 && compress != 12 && compress != 18) return set_error(LQCD_EINVAL, "compress %d", compress);
   lqcd_ctx* c = g[0]->ctx;
-  LQCD_CK(cudaSetDevice(c->device));
+  LQCD_TRY(ctx_enter(c));
   cudaStream_t st = c->stream;
   int nr = -1;
   std::vector<Work> w(n);
