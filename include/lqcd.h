@@ -105,7 +105,9 @@ LQCD_API long long lqcd_ctx_launch_count(const lqcd_ctx* ctx);
  * BiCGStab vectors; operator and upload temporaries), so repeated solves
  * allocate nothing, and up to 1 GiB of the buffers of destroyed fields, gauge
  * fields and momenta, for the next ones of the same size (given back also when
- * an allocation for the context fails). Once a call of the context was captured
+ * an allocation of any context on the device fails; other allocators in the
+ * process, such as PyTorch's, cannot ask for them: call this before they need
+ * the device's last GiB). Once a call of the context was captured
  * into a graph, or another context copied from a field of this one, destroyed
  * objects are freed at once, after all work on the device. This waits for the
  * context's stream and frees them; the next call allocates again. Objects the

@@ -113,9 +113,27 @@ int ctx_enter(lqcd_ctx* c) {
   return LQCD_OK;
 }
 
+// every context of the process, for ctx_malloc
+static std::mutex& contexts_mu() {
+  static std::mutex* m = new std::mutex();
+  return *m;
+}
+static std::set<lqcd_ctx*>& contexts() {
+  static std::set<lqcd_ctx*>* s = new std::set<lqcd_ctx*>();
+  return *s;
+}
+
+static bool release_pools(int device) {
+  std::lock_guard<std::mutex> lk(contexts_mu());
+  bool any = false;
+  for (lqcd_ctx* c : contexts())
+    if (c->device == device) any = ctx_pool_release(c) || any;
+  return any;
+}
+
 cudaError_t ctx_malloc(lqcd_ctx* c, void** out, size_t bytes) {
   cudaError_t e = cudaMalloc(out, bytes);
-  if (e == cudaErrorMemoryAllocation && ctx_pool_release(c)) {
+  if (e == cudaErrorMemoryAllocation && release_pools(c->device)) {
     cudaGetLastError();
     e = cudaMalloc(out, bytes);
   }
@@ -242,7 +260,7 @@ int lqcd_ctx_create(lqcd_ctx** out, int device, void* stream) {
   }
   if (rc == LQCD_OK) {
     c->stream = stream ? (cudaStream_t)stream : c->own_stream;
-    cudaError_t e = cudaMalloc(&c->scratch_sc, 16 * sizeof(Scalars));
+    cudaError_t e = ctx_malloc(c, (void**)&c->scratch_sc, 16 * sizeof(Scalars));
     if (e == cudaSuccess) e = cudaMemset(c->scratch_sc, 0, 16 * sizeof(Scalars));
     if (e == cudaSuccess) e = cudaMallocHost(&c->host_sc, 16 * sizeof(Scalars));
     if (e != cudaSuccess) rc = set_error(LQCD_ECUDA, "scratch: %s", cudaGetErrorString(e));
@@ -250,6 +268,10 @@ int lqcd_ctx_create(lqcd_ctx** out, int device, void* stream) {
   if (rc != LQCD_OK) {
     lqcd_ctx_destroy(c);
     return rc;
+  }
+  {
+    std::lock_guard<std::mutex> lk(contexts_mu());
+    contexts().insert(c);
   }
   *out = c;
   return LQCD_OK;
@@ -271,6 +293,10 @@ void ctx_release(lqcd_ctx* c) {
   cudaSetDevice(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
   ctx_drop_engine(c);
+  {
+    std::lock_guard<std::mutex> lk(contexts_mu());
+    contexts().erase(c);
+  }
   ctx_pool_release(c);
   if (c->partials) cudaFree(c->partials);
   if (c->scratch_sc) cudaFree(c->scratch_sc);

@@ -124,7 +124,7 @@ int ctx_staging(lqcd_ctx* c, size_t bytes);
 // stay with the context for the next object of the same size, the newest ones when there are
 // more (so that a program that moves on to another lattice gains there too: the load and apply
 // after larger solves 719 -> 494 us). They are given back by lqcd_ctx_release_cache, with the
-// context, and when any allocation for the context fails (ctx_malloc). Whoever frees has
+// context, and when an allocation of any context on the device fails (ctx_malloc). Whoever frees has
 // waited for the context's stream, and a change of stream waits for the old one. That is all
 // the work there is on a buffer unless a call was captured, whose graph may be in flight on any
 // stream, or another context copied from a field of this one. Such a context (used_elsewhere)

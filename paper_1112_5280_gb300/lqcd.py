@@ -250,7 +250,9 @@ class Context:
         _check(self._lib.lqcd_ctx_sync(self.h))
 
     def release_cache(self):
-        """Frees the buffers the one-shot solves keep between calls (lqcd_ctx_release_cache)."""
+        """Frees the buffers the one-shot solves keep between calls and those of destroyed fields,
+        gauge fields and momenta, up to 1 GiB, that other allocators such as torch's cannot reach
+        (lqcd_ctx_release_cache)."""
         _check(self._lib.lqcd_ctx_release_cache(self.h))
 
     @property
