@@ -70,7 +70,8 @@ struct Scalars {
   int normal;       // 1: solve Mhat^dag Mhat x = phi; converged on |phi - Mhat^dag Mhat x|
   unsigned ticket;  // k_finish groups done (reset by the last)
   int bad;          // FIN_ALPHA found the step impossible (ST_*); FIN_BETA stops the slot
-  unsigned pad2[2];
+  unsigned updates_enabled;  // update blocks that request_update enabled (first slot of the launch)
+  unsigned pad2;
 };
 
 // One slot's operands for one batched kernel.

@@ -93,6 +93,7 @@ struct Request {
   SlotBuf buf;
   int tile0 = 0, ntiles = 0;
   bool finished = false;
+  unsigned updates_counted = 0;  // of Scalars::updates_enabled
   lqcd_solve_info info{};
   std::chrono::steady_clock::time_point t0;
 };
@@ -137,6 +138,8 @@ struct lqcd_engine {
   std::vector<Launch> exec_key;  // the launches in exec, with what else decided its shape
   std::vector<unsigned> exec_opts;
   cudaStream_t body_stream = nullptr;  // captures the graph's conditional bodies
+  // launches of the captured chunk outside its update blocks, and in one update block
+  long long chunk_launches = 0, update_launches = 0;
   std::vector<Work> h_works;
 };
 
@@ -297,17 +300,18 @@ StepKind kind_of(int s) {
 }
 
 // tw: some slot of the launch is twisted (its Dslash steps take the twisted epilogues;
-// untwisted slots carry the identity twist there and give the same bits)
-cudaError_t issue(lqcd_engine* e, int s, const Launch& L, bool tw) {
+// untwisted slots carry the identity twist there and give the same bits). st: the context's
+// stream, or the one that captures a part of the graph
+cudaError_t issue(lqcd_engine* e, int s, const Launch& L, bool tw, cudaStream_t st) {
   const StepKind k = kind_of(s);
   e->ctx->launches += L.finish == 1 ? 2 : 1;
   if (k.dslash) {
     const int epi = k.epi_or_op + (tw ? EPI_LIN_TW - EPI_LIN : 0);
-    if (k.f64) return launch_dslash(e->tp, 18, k.dag, epi, L, 0, e->ctx->stream);
-    return launch_dslash(e->sp, e->nr, k.dag, epi, L, 0, e->ctx->stream);
+    if (k.f64) return launch_dslash(e->tp, 18, k.dag, epi, L, 0, st);
+    return launch_dslash(e->sp, e->nr, k.dag, epi, L, 0, st);
   }
   const int prec = (k.epi_or_op == B_RU_FOLD) ? e->xp : e->sp;
-  return launch_blas(prec, k.epi_or_op, L, 0, e->ctx->stream, e->tp);
+  return launch_blas(prec, k.epi_or_op, L, 0, st, e->tp);
 }
 
 Launch batch_launch(const lqcd_engine* e, int s) {
@@ -353,9 +357,9 @@ std::vector<int> ru_steps(bool normal, bool plain) {
   return v;
 }
 
-cudaError_t issue_updates(lqcd_engine* e) {
+cudaError_t issue_updates(lqcd_engine* e, cudaStream_t st) {
   for (int s : ru_steps(e->any_normal, e->any_plain)) {
-    cudaError_t err = issue(e, s, batch_launch(e, s), e->any_twist);
+    cudaError_t err = issue(e, s, batch_launch(e, s), e->any_twist, st);
     if (err != cudaSuccess) return err;
   }
   return cudaSuccess;
@@ -386,10 +390,11 @@ cudaError_t capture_updates(lqcd_engine* e, cudaGraphConditionalHandle cond) {
   cudaGraph_t body = p.conditional.phGraph_out[0], done = nullptr;
   err = cudaStreamBeginCaptureToGraph(e->body_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
   if (err != cudaSuccess) return err;
-  e->ctx->stream = e->body_stream;
   pdl_skip_next(true);
-  err = issue_updates(e);
-  e->ctx->stream = st;
+  const long long before = e->ctx->launches;
+  err = issue_updates(e, e->body_stream);
+  e->update_launches = e->ctx->launches - before;
+  e->ctx->launches = before;  // counted when the block runs
   const cudaError_t end = cudaStreamEndCapture(e->body_stream, &done);
   pdl_skip_next(true);  // the iteration after the node
   return err != cudaSuccess ? err : end;
@@ -415,11 +420,11 @@ cudaError_t issue_iteration_block(lqcd_engine* e, int iters, bool capturing) {
     for (int s : {K1, K2, K3, K4, K6}) {
       Launch L = batch_launch(e, s);
       if (s == K6) L.cond = cond;
-      cudaError_t err = issue(e, s, L, e->any_twist);
+      cudaError_t err = issue(e, s, L, e->any_twist, e->ctx->stream);
       if (err != cudaSuccess) return err;
     }
     if (update) {
-      cudaError_t err = capturing ? capture_updates(e, cond) : issue_updates(e);
+      cudaError_t err = capturing ? capture_updates(e, cond) : issue_updates(e, e->ctx->stream);
       if (err != cudaSuccess) return err;
     }
   }
@@ -436,7 +441,10 @@ int capture_chunk(lqcd_engine* e) {
   if (!e->body_stream) err = cudaStreamCreateWithFlags(&e->body_stream, cudaStreamNonBlocking);
   if (err == cudaSuccess) err = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
   if (err == cudaSuccess) {
+    const long long before = e->ctx->launches;
     err = issue_iteration_block(e, e->opts.chunk, true);
+    e->chunk_launches = e->ctx->launches - before;
+    e->ctx->launches = before;  // counted when the graph runs
     pdl_skip_next(false);
     const cudaError_t end = cudaStreamEndCapture(st, &graph);
     if (err == cudaSuccess) err = end;
@@ -909,7 +917,7 @@ static int submit_impl(lqcd_engine* e, const lqcd_gauge* gauge, const lqcd_field
       for (int s : ru_steps(normal, !normal)) {
         if (err != cudaSuccess) break;
         if (!x0 && (s == RU_FOLD || s == RU_D1 || s == RU_RES)) continue;
-        err = issue(e, s, single_launch(w2[s], e->d_partials), mu != 0.0);
+        err = issue(e, s, single_launch(w2[s], e->d_partials), mu != 0.0, st);
       }
     }
     c->launches += 4;
@@ -951,9 +959,7 @@ int lqcd_engine_step(lqcd_engine* e, int* n_active) {
     }
     if (e->opts.use_graph) {
       LQCD_CK(cudaGraphLaunch(e->exec, st));
-      c->launches += (long long)e->opts.chunk * 5 +
-                     ((e->opts.chunk + e->ru_every - 1) / e->ru_every) *
-                         (long long)ru_steps(e->any_normal, e->any_plain).size();
+      c->launches += e->chunk_launches;
     } else {
       cudaError_t err = issue_iteration_block(e, e->opts.chunk, false);
       if (err != cudaSuccess) return set_error(LQCD_ECUDA, "iteration: %s", cudaGetErrorString(err));
@@ -962,6 +968,12 @@ int lqcd_engine_step(lqcd_engine* e, int* n_active) {
     for (long long id : e->active) maxslot = std::max(maxslot, e->reqs[id].slot + 1);
     LQCD_CK(cudaMemcpyAsync(e->h_sc, e->d_sc, sizeof(Scalars) * maxslot, cudaMemcpyDeviceToHost, st));
     LQCD_CK(cudaStreamSynchronize(st));
+    if (e->opts.use_graph) {  // the update blocks that ran in this chunk
+      Request& first = e->reqs[e->active[0]];
+      const unsigned n = e->h_sc[first.slot].updates_enabled;
+      c->launches += (long long)(n - first.updates_counted) * e->update_launches;
+      first.updates_counted = n;
+    }
     std::vector<long long> fin;
     for (long long id : e->active) {
       const Scalars& s = e->h_sc[e->reqs[id].slot];

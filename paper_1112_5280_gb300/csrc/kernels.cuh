@@ -579,8 +579,13 @@ enum Blas {
 // left for one (the default, set at each launch of the graph, is to skip it).
 __device__ __forceinline__ void request_update(const Launch& L) {
   if (!L.cond || blockIdx.x != 0) return;
+  int any = 0;
   for (int i = threadIdx.x; i < L.nslots; i += TILE)
-    if (*((volatile int*)&work_of(L, i).sc->state) == S_UPDATE) cudaGraphSetConditional(L.cond, 1);
+    any |= *((volatile int*)&work_of(L, i).sc->state) == S_UPDATE;
+  if (__syncthreads_or(any) && threadIdx.x == 0) {
+    cudaGraphSetConditional(L.cond, 1);
+    ++work_of(L, 0).sc->updates_enabled;
+  }
 }
 
 // out = x + c * y (complex c)
