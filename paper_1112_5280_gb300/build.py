@@ -98,8 +98,8 @@ if __name__ == "__main__":
 # Files that define the Dslash kernel and its launch (a change to any of them
 # invalidates profile counters taken on the old code).
 DSLASH_KERNEL_FILES = ("field.cuh", "dslash.cuh", "batch.cuh", "kernels.cuh", "kernels_inst.cuh",
-                       "kernels_f32.cu", "kernels_f32_stream.cu", "kernels_f16.cu", "kernels_f64.cu", "launch.h",
-                       "layout.cu")
+                       "kernels_f32.cu", "kernels_f32_stream.cu", "kernels_f16.cu", "kernels_f16_stream.cu", "kernels_f64.cu",
+                       "launch.h", "layout.cu")
 
 
 def source_hash(files=DSLASH_KERNEL_FILES) -> str:

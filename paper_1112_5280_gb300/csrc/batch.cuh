@@ -123,7 +123,7 @@ struct Launch {
   // (Dslash kernels; the step it belongs to needs alpha only two launches later)
   const Work* fin_works;
   int fin_groups;
-  int stream_links;        // 1: several gauge fields, more link bytes than L2 holds
+  int stream_links;        // works: 1: links read past L1 (the rule is in launch.h)
   // CUDA graph: the conditional node to enable when some slot waits for a reliable update
   unsigned long long cond;
 };

@@ -783,7 +783,7 @@ int lqcd_dslash_batch_create(int n, const lqcd_gauge* const* g, const lqcd_field
   std::set<const lqcd_gauge*> gauges;
   for (int i = 0; i < n; ++i)
     if (gauges.insert(g[i]).second) link_bytes += gauge_copy_bytes(link_prec_for(prec), nr, g[i]->g.Vh);
-  b->L.stream_links = stream_links((int)gauges.size(), link_bytes);
+  b->L.stream_links = stream_links(prec, n, (int)gauges.size(), link_bytes);
   if (n == 1) {
     b->L.works = nullptr;
     b->L.inline_work = w[0];

@@ -494,7 +494,7 @@ int rebuild(lqcd_engine* e) {
     const Request& q = e->reqs[id];
     if (gauges.insert(q.gauge).second) link_bytes += gauge_copy_bytes(link_prec_for(e->sp), e->nr, q.g.Vh);
   }
-  e->stream_links = stream_links((int)gauges.size(), link_bytes);
+  e->stream_links = stream_links(e->sp, n, (int)gauges.size(), link_bytes);
   // Slots on one gauge field may share each site block's link loads in the sloppy Dslash
   // steps (k_dslash_mrhs): a CTA applies the block's links to a group of slots. The group
   // size is the autotuner's measured choice for this key. Without one the slots load their

@@ -36,9 +36,9 @@ inline std::vector<int (*)(unsigned long long*)>& bounds_word_readers() {
 // (8 bytes, like FP64) and computes in double-float arithmetic (below).
 enum Prec { P_F64 = 0, P_F32 = 1, P_F16 = 2, P_BF16 = 3, P_DF64 = 4 };
 constexpr int NPREC = 5;  // number of storage precisions (size of per-precision tables)
-// FP32 links read past L1: the storage of P_F32 under another LinkIO (a template argument of
-// the kernels, never a field's precision)
-constexpr int P_F32_STREAM = NPREC;
+// FP32 and FP16 links read past L1: the storage of P_F32 and P_F16 under another LinkIO (template
+// arguments of the kernels, never a field's precision)
+constexpr int P_F32_STREAM = NPREC, P_F16_STREAM = NPREC + 1;
 
 __host__ __device__ constexpr int prec_bytes(int p) {
   return (p == P_F64 || p == P_DF64) ? 8 : ((p == P_F32 || p == P_F32_STREAM) ? 4 : 2);
@@ -301,10 +301,9 @@ struct BoundsWordRegistration {
 // against L1::no_allocate, per application: 16^3x32 FP32-18 8.6 -> 7.6 us, FP32-12 7.6 -> 7.1,
 // FP16-12 8.0 -> 7.3; 24^3x48, 12 sources, the whole FP32 solve 238 -> 217 ms; at 32^3x64,
 // where HBM bounds, FP32-12 96.4 -> 95.9, FP16-12 71.2 -> 71.3, FP32-18 121.4 -> 122.5.
-// L1::evict_first measured as no_allocate. Many different gauge fields in one launch, more
-// link bytes than L2 holds, are the exception: nothing is found again, and the links push
-// spinors out of L1 (18 mixed FP32 systems 57.7 -> 58.9 ms), so such FP32 launches keep
-// no_allocate (P_F32_STREAM, Launch::stream_links).
+// L1::evict_first measured as no_allocate. Launches whose links L2 cannot keep are the
+// exception: nothing is found again, and the links push spinors out of L1. They read past it
+// (P_F32_STREAM, P_F16_STREAM; the rule and its figures are at stream_links in launch.h).
 
 __device__ __forceinline__ double2 ld_ro(const double2* p) { return __ldg(p); }
 __device__ __forceinline__ float4 ld_ro(const float4* p) { return __ldg(p); }
@@ -329,6 +328,17 @@ __device__ __forceinline__ float4 ld_stream(const float4* p) {
                : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
   return v;
 }
+__device__ __forceinline__ uint2 ld_stream(const uint2* p) {
+  uint2 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ unsigned ld_stream(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+
 // half2 / bfloat162 packed in a 32-bit word
 __device__ __forceinline__ float2 unpack_h2(unsigned w) {
   __half2 h = *reinterpret_cast<__half2*>(&w);
@@ -695,18 +705,6 @@ struct LinkIO<P_F32, 12> {
   }
 };
 
-template <int NR>
-struct LinkIO<P_F32_STREAM, NR> : LinkIO<P_F32, NR> {
-  using Word = typename LinkIO<P_F32, NR>::Word;
-  static constexpr int NW = LinkIO<P_F32, NR>::NW;
-  __device__ static void load_raw(const void* base_mu, int Vh, int h, Word w[NW]) {
-    h = LQCD_SITE(h, Vh);
-    const Word* p = reinterpret_cast<const Word*>(base_mu) + h;
-#pragma unroll
-    for (int c = 0; c < NW; ++c) w[c] = ld_stream(p + (size_t)c * Vh);
-  }
-};
-
 template <>
 struct LinkIO<P_F16, 18> {
   using Real = float;
@@ -762,6 +760,23 @@ struct LinkIO<P_F16, 12> {
     unpack(w, u);
   }
 };
+
+// The same links read past L1
+template <int LP, int NR>
+struct LinkIOStream : LinkIO<LP, NR> {
+  using Word = typename LinkIO<LP, NR>::Word;
+  static constexpr int NW = LinkIO<LP, NR>::NW;
+  __device__ static void load_raw(const void* base_mu, int Vh, int h, Word w[NW]) {
+    h = LQCD_SITE(h, Vh);
+    const Word* p = reinterpret_cast<const Word*>(base_mu) + h;
+#pragma unroll
+    for (int c = 0; c < NW; ++c) w[c] = ld_stream(p + (size_t)c * Vh);
+  }
+};
+template <int NR>
+struct LinkIO<P_F32_STREAM, NR> : LinkIOStream<P_F32, NR> {};
+template <int NR>
+struct LinkIO<P_F16_STREAM, NR> : LinkIOStream<P_F16, NR> {};
 
 // a_i b_j - a_j b_i for complex a_i, b_j, a_j, b_i, in a fixed order of products and sums
 template <typename R>

@@ -1,0 +1,6 @@
+// Batched Dslash, spinor storage F16, links read past L1 (stream_links in launch.h). A
+// translation unit of its own, compiled in parallel with kernels_f16.cu.
+#define LQCD_SP lqcd::P_F16
+#define LQCD_SFX f16
+#define LQCD_STREAM_UNIT 1
+#include "kernels_inst.cuh"

@@ -1,6 +1,5 @@
-// Batched Dslash, spinor storage F32, links read past L1: launches over several gauge fields
-// with more link bytes than L2 holds. A translation unit of its own, compiled in parallel
-// with kernels_f32.cu.
+// Batched Dslash, spinor storage F32, links read past L1 (stream_links in launch.h). A
+// translation unit of its own, compiled in parallel with kernels_f32.cu.
 #define LQCD_SP lqcd::P_F32
 #define LQCD_SFX f32
 #define LQCD_STREAM_UNIT 1

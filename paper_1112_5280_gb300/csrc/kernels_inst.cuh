@@ -1,9 +1,9 @@
 // Instantiates the batched kernels for one spinor precision LQCD_SP with
 // launch-function suffix LQCD_SFX. Included by kernels_<prec>.cu.
 //
-// LQCD_STREAM_UNIT: this translation unit holds the FP32 Dslash with links read past L1
+// LQCD_STREAM_UNIT: this translation unit holds the Dslash with links read past L1
 // (launch_dslash_stream_<sfx>), to which the dispatcher of the LQCD_STREAM_EXTERN unit
-// forwards the launches with stream_links.
+// forwards the launches that stream_links (launch.h) names.
 //
 // LQCD_TW_UNIT: this translation unit holds only the twisted-mass Dslash epilogues
 // (launch_dslash_tw_<sfx>); LQCD_TW_EXTERN: the dispatcher of this unit forwards the
@@ -20,7 +20,7 @@ namespace lqcd {
 namespace {
 constexpr int SPX = LQCD_SP;
 #ifdef LQCD_STREAM_UNIT
-constexpr int LPX = P_F32_STREAM;
+constexpr int LPX = SPX == P_F32 ? P_F32_STREAM : P_F16_STREAM;
 #else
 constexpr int LPX = (SPX == P_F64 || SPX == P_DF64 || SPX == P_F32) ? SPX : P_F16;
 #endif
@@ -44,7 +44,7 @@ cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
   // shared-link multi-RHS launches (every slot on one gauge field): FP32-arithmetic
   // precisions, Wilson epilogues
   if (L.interleave == 2) {
-    if constexpr (LPX != P_F32_STREAM && (SPX == P_F32 || SPX == P_F16 || SPX == P_BF16) && !EpiTraits<EPI>::tw) {
+    if constexpr (LPX < NPREC && (SPX == P_F32 || SPX == P_F16 || SPX == P_BF16) && !EpiTraits<EPI>::tw) {
       auto fm = k_dslash_mrhs<SPX, LPX, NR, DAG, EPI>;
       if (grid <= 0) {
         int scps = 0;
@@ -184,7 +184,8 @@ cudaError_t LQCD_CAT(launch_dslash_, LQCD_SFX)(int nr, bool dag, int epi, const 
   if (!L.works && L.inline_work.twist && epi != EPI_LIN_TW && epi != EPI_PLAIN_TW && epi != EPI_CG_TW)
     return cudaErrorInvalidValue;
 #ifdef LQCD_STREAM_EXTERN
-  if (L.stream_links && (nr == 18 || nr == 12))
+  const bool stream = L.works ? L.stream_links : stream_links(SPX, 1, 1, link_copy_bytes(SPX, nr, L.inline_work.g.Vh));
+  if (stream && (nr == 18 || nr == 12))
     return LQCD_CAT(launch_dslash_stream_, LQCD_SFX)(nr, dag, epi, L, grid, s, form);
 #endif
   if (nr == 18) return dispatch_nr<18>(dag, epi, L, grid, s, form);

@@ -77,9 +77,30 @@ cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t dyn
 // between kernels, and what it follows in a captured graph is another kind of node.
 void pdl_skip_next(bool skip);
 
-// Launch::stream_links: the slots' link copies (bytes in all, over `gauges` different gauge
-// fields) are more than half of L2 (126 MB), which the launch's spinors share.
-inline int stream_links(int gauges, size_t link_bytes) { return gauges > 1 && link_bytes > ((size_t)64 << 20); }
+// Bytes of the link copy that fields of precision sp (FP32, FP16, BF16) read
+inline size_t link_copy_bytes(int sp, int nr, int Vh) { return (size_t)2 * 4 * nr * Vh * (sp == P_F32 ? 4 : 2); }
+
+// Launch::stream_links (single-slot launches: the rule itself): the links are read past L1, by
+// slots of `gauges` different gauge fields with link_bytes of links in all. Measured on GB300,
+// past L1 against through it, us a call:
+//  - Up to 58 MiB, which L2 still holds beside the spinors, L1 saves L2 traffic: M-hat FP32-18
+//    16^3x32 16.9 / 15.2, 18^3x36 (58 MiB) 30.2 / 27.2, FP16-12 16^3x64 28.0 / 23.4, 24^3x36
+//    (46 MiB) 42.1 / 41.1.
+//  - Above it L1 finds nothing again: FP32-12 20^3x40 (59 MiB) 35.0 / 36.6, 24^3x48 68.5 / 74.3
+//    (its CG 22.5 / 23.5 ms), FP16-12 24^3x48 (61 MiB) 51.2 / 53.9, FP16-18 there 50.8 / 56.0,
+//    BF16-18 64.9 / 70.5, five to ten 16^3x32 FP16 fields in a batch 1-7% less.
+//  - Above 256 MiB, twice L2, HBM bounds both, and rows that start off a sector boundary gain by
+//    L1: FP32-18 28^3x56 158.5 / 155.1, FP16-18 32^3x64 157.1 / 156.3.
+//  - Slots that share a gauge field find each other's links in L1 at every size: 24^3x48 with 12
+//    sources, FP16-12 258 / 247, FP32-12 280 / 245.
+//  - FP32 batches over several gauge fields take no upper bound (ten 16^3x32, 18 reals, 81.0 /
+//    81.8), and go past L1 also where some slots share one.
+inline bool stream_links(int sp, int slots, int gauges, size_t link_bytes) {
+  constexpr size_t MIB = (size_t)1 << 20;
+  if (sp != P_F32 && sp != P_F16 && sp != P_BF16) return false;
+  if (sp == P_F32 && gauges > 1) return link_bytes > 64 * MIB;
+  return gauges == slots && link_bytes > 58 * MIB && link_bytes <= 256 * MIB;
+}
 
 // Counts changes of what decides a launch's shape (tuner table, grid caps, kernel form): a
 // captured graph is good for as long as it stands.
