@@ -1,8 +1,5 @@
 // Layout kernels (gauge and spinor upload, even-odd split, precision
 // conversion, link compression) and the host dispatch of batched launches.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
 #include <atomic>
 #include <cstdlib>
 #include <mutex>
@@ -77,6 +74,9 @@ struct WordsHalf {
     const __half2 h(__double2half(a), __double2half(b));
     return *reinterpret_cast<const unsigned*>(&h);
   }
+  __device__ static unsigned pair_bits(double a, double b) {
+    return BF ? cv::to_bf16(a) | (cv::to_bf16(b) << 16) : cv::to_half(a) | (cv::to_half(b) << 16);
+  }
   __device__ static void get2(unsigned w, double* v) {
     const float2 f = BF ? unpack_b2(w) : unpack_h2(w);
     v[0] = cv::to_double(f.x);
@@ -87,6 +87,12 @@ struct WordsHalf {
   }
   __device__ static T put(const double* v) {
     return make_uint4(pair(v[0], v[1]), pair(v[2], v[3]), pair(v[4], v[5]), pair(v[6], v[7]));
+  }
+  // the same on integer bits, for k_spinor_convert: its threads convert in step, one word each,
+  // and the conversion instructions do not overlap with its loads (FP64 to FP16 at 16^3x32 20.6
+  // -> 13.0 us); the other kernels hide them (an FP16 upload at 32^3x64 99.5 us, by bits 105.8)
+  __device__ static T put_bits(const double* v) {
+    return make_uint4(pair_bits(v[0], v[1]), pair_bits(v[2], v[3]), pair_bits(v[4], v[5]), pair_bits(v[6], v[7]));
   }
 };
 template <>
@@ -313,7 +319,10 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_spinor_convert(const void* i
     for (int k = 0; k < 8; ++k) v[k] *= scale;
   }
 #pragma unroll
-  for (int w = 0; w < NO; ++w) dst[(size_t)w * Vh] = Wo::put(v + w * Wo::W);
+  for (int w = 0; w < NO; ++w) {
+    if constexpr (PO == P_F16 || PO == P_BF16) dst[(size_t)w * Vh] = Wo::put_bits(v + w * Wo::W);
+    else dst[(size_t)w * Vh] = Wo::put(v + w * Wo::W);
+  }
 }
 
 template <int P>
