@@ -496,7 +496,7 @@ typedef struct lqcd_tune_result {
   int form;         /* chosen kernel form: 0 one thread per site, 1 colour split (DF64),
                        2 shared-link multi-RHS, 3 one thread per site compiled for 8 CTAs
                        per SM (FP32: 128 registers, more warps with fewer loads each; the
-                       FP32 default, but for twisted launches of more tiles than that) */
+                       default where it fits a launch better) */
   int candidates;   /* configurations timed */
   double us_best;   /* per launch, chosen configuration */
   double us_default;/* per launch, untuned default (shared-link entries: the own-link launch) */

@@ -34,11 +34,7 @@ cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
   int cps = 0;
   if (form < 0 || grid <= 0) {
     const TuneChoice t = tune_choice(SPX, NR, L.ntiles);
-    if (form < 0) {
-      form = t.form;
-      // untuned FP32, twisted, more than one wave at the second register budget: the first
-      if (SPX == P_F32 && EpiTraits<EPI>::tw && !t.tuned && L.ntiles > DSLASH_MIN_BLOCKS_HI * device_sm_count()) form = 0;
-    }
+    if (form < 0) form = t.form;
     cps = t.ctas_per_sm;
   }
   // shared-link multi-RHS launches (every slot on one gauge field): FP32-arithmetic

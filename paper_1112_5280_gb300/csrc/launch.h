@@ -123,7 +123,6 @@ int dslash_occupancy(int sp, int nr, int form);
 struct TuneChoice {
   int ctas_per_sm;  // 0: occupancy limit
   int form;         // 0 site, 1 colour split, 3 site at the second register budget
-  bool tuned;       // from the table (else the defaults)
 };
 TuneChoice tune_choice(int sp, int nr, int ntiles);
 // Shared-link choice for nrhs slots on one gauge field of `blocks` site blocks: the tuned
@@ -136,14 +135,8 @@ int tune_shared_links(int sp, int nr, int nrhs, int blocks, int* ctas_per_sm);
 bool dslash_colour_split(int prec);
 void set_dslash_colour_split(int prec, bool on);
 
-// The Dslash form without a tuned choice. FP32 takes the second register budget (8 CTAs per
-// SM): measured on GB300 against 6 CTAs, 16^3x32 8.6 -> 7.4 us (12 link reals) and 10.0 -> 8.5
-// us (18; 1024 tiles are then one wave of resident CTAs instead of two), 32^3x64 101.3 -> 96.3
-// and 122.8 -> 121.7 us, M-hat there 219 -> 207 and 262 -> 258 us, the 16^3x32 CG 76.8 -> 65.9
-// us an iteration. The twisted epilogues keep more values alive: they gain while the launch
-// is one wave (16^3x32 M-hat 22.9 -> 18.4 us) and lose 5% beyond (go_dslash).
-inline int default_dslash_form(int prec) { return prec == P_F32 ? 3 : (dslash_colour_split(prec) ? 1 : 0); }
-
+// The Dslash form without a tuned choice (for FP32 a rule of waves: tune.cu)
+int default_dslash_form(int prec, int nr, int ntiles);
 
 // layout kernels (layout.cu)
 // (the AoS arrays need the alignment of their FP64 reals only)

@@ -194,14 +194,36 @@ bool get_num(const JVal& o, const char* k, double& out) {
 
 }  // namespace
 
+// FP32: the first register budget keeps three hops of loads in flight in 6 CTAs per SM, the
+// second (form 3) fewer in 8. Applications that follow one another overlap (programmatic launch)
+// while two of them fit the SMs, so what counts up to one wave is the budget that fits two, then
+// one; up to four waves, the one with fewer waves; beyond, the link reals. Measured on GB300,
+// form 0 / form 3, us a M-hat: 4^4 5.9 / 6.4, 12^3x24 (324 tiles) 8.8 / 9.2, 16^4 (512: two fit at
+// 8 CTAs only) 11.2 / 9.7, 14^3x32 (686: one fits) 12.2 / 13.8, 16^3x32 (1024: one fits at 8
+// only) 15.0 / 13.8 and, with 18 reals, 15.9 / 15.2, 16^3x48 (1536, two waves) 19.9 / 20.6, 16^3x64
+// (2048, three or two) 35.0 / 32.8 with 18 reals, 20^3x40 (2500) 34.9 / 36.3, its CG 11.4 / 12.3 ms,
+// 24^3x48 68.9 / 68.5 and 83.1 / 85.1 (CG 21.9 / 22.5 and 24.7 / 26.3 ms), 32^3x64 208 / 204 and
+// 254 / 259; 12 sources on one 24^3x48 field 269 / 245 us, ten 16^3x32 fields 65.5 / 63.5 and
+// 80.3 / 80.5. The twisted epilogues follow the same lines (14^3x32 12.1 / 14.0, 16^3x32
+// 15.7 / 14.2, 20^3x40 35.7 / 36.8, 32^3x64 211 / 205 and, with 18 reals, 257 / 263).
+int default_dslash_form(int prec, int nr, int ntiles) {
+  if (prec != P_F32) return dslash_colour_split(prec) ? 1 : 0;
+  const long long sms = device_sm_count(), first = LQCD_DSLASH_MIN_BLOCKS * sms, second = DSLASH_MIN_BLOCKS_HI * sms;
+  for (int launches : {2, 1}) {
+    if ((long long)launches * ntiles <= first) return 0;
+    if ((long long)launches * ntiles <= second) return 3;
+  }
+  const long long waves = (ntiles + first - 1) / first;
+  return (waves > 4 ? nr == 12 : (ntiles + second - 1) / second < waves) ? 3 : 0;
+}
+
 TuneChoice tune_choice(int sp, int nr, int ntiles) {
-  TuneChoice c{0, default_dslash_form(sp), false};
+  TuneChoice c{0, default_dslash_form(sp, nr, ntiles)};
   std::lock_guard<std::mutex> lk(g_mu);
   auto it = g_table.find({sp, nr, 0, bucket_of(ntiles)});
   if (it != g_table.end()) {
     c.ctas_per_sm = it->second.ctas_per_sm;
     c.form = it->second.form;
-    c.tuned = true;
   }
   return c;
 }
@@ -310,7 +332,7 @@ int lqcd_autotune_dslash(int n, const lqcd_gauge* const* g, int prec, int compre
   if (err == cudaSuccess) err = cudaEventCreate(&e0);
   if (err == cudaSuccess) err = cudaEventCreate(&e1);
   const int nsm = device_sm_count();
-  const int def_form = default_dslash_form(prec);
+  const int def_form = default_dslash_form(prec, nr, ntiles);
   // time `reps` launches of one configuration: best average of three trials (us)
   auto time_cfg = [&](const Launch& LL, int grid, int form, double* us) -> cudaError_t {
     cudaError_t e = cudaSuccess;
