@@ -26,12 +26,15 @@ struct EpiTraits {
 #define LQCD_DSLASH_MIN_BLOCKS 6
 #endif
 // FP16 / BF16 spinors: the same bytes in flight come from half the words, so the half
-// precisions take a higher occupancy target: 10 CTAs per SM (96 registers) for BF16 and for the
-// plain FP16-12 operator, 8 (128 registers) for the other FP16 kernels, whose hops are packed
+// precisions take a higher occupancy target: 10 CTAs per SM (96 registers) for BF16-12 and for the
+// plain FP16-12 operator, 8 (128 registers) for the other kernels, whose hops are packed
 // (dslash.cuh) and spill at 96. Measured for FP16 at 8 against 10: the 32^3x64 FP16-12 CG 47.2
 // against 48.2 ms, the 16^3x32 twisted one 58.7 against 61.5 us an iteration, 12 sources at
 // 24^3x48 184.2 against 189.2 ms, FP16-18 32^3x64 73.8 against 75.3 us; the plain FP16-12 M-hat
-// there 151.3 against 149.5 (its small launches: go_dslash). BF16-12 at 8: 70.1 against 69.0. At 12 (80 registers) all lose.
+// there 151.3 against 149.5 (its small launches: go_dslash). BF16-12 at 8: 70.1 against 69.0.
+// BF16-18 at 8 against 10, us a M-hat: 4^4 5.8 / 7.3, 16^3x32 12.9 / 16.1, 24^3x48 50.8 / 65.4, five
+// 16^3x32 fields in a batch 24.3 / 31.4; its 24^3x48 CG 26.1 / 27.4 ms (scalar hops at 10: 62.0 us and
+// 27.1 ms). At 12 (80 registers) all lose.
 #ifndef LQCD_DSLASH_MIN_BLOCKS_HALF
 #define LQCD_DSLASH_MIN_BLOCKS_HALF 10
 #endif
@@ -47,8 +50,8 @@ struct ScalarF16 {
 template <int SP, int NR, int EPI>
 struct DslashMinBlocks {
   static constexpr int value = SP == P_DF64 ? 4
-                               : SP == P_BF16 || ScalarF16<SP, NR, EPI>::value ? LQCD_DSLASH_MIN_BLOCKS_HALF
-                               : SP == P_F16 ? LQCD_DSLASH_MIN_BLOCKS_F16
+                               : (SP == P_BF16 && NR == 12) || ScalarF16<SP, NR, EPI>::value ? LQCD_DSLASH_MIN_BLOCKS_HALF
+                               : SP == P_F16 || SP == P_BF16 ? LQCD_DSLASH_MIN_BLOCKS_F16
                                              : LQCD_DSLASH_MIN_BLOCKS;
 };
 // The second register budget of the FP32 Dslash (launch form 3): 8 CTAs per SM, 128

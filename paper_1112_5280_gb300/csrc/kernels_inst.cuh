@@ -28,6 +28,14 @@ constexpr int LPX = (SPX == P_F64 || SPX == P_DF64 || SPX == P_F32) ? SPX : P_F1
 // CTAs before the launch's own that finish the launch before it
 int fin_ctas(const Launch& L) { return L.fin_works ? L.nslots * L.fin_groups : 0; }
 
+// the one-thread-per-site form at MB CTAs per SM
+template <int NR, bool DAG, int EPI, int MB>
+cudaError_t go_site(const Launch& L, int grid, int cps, cudaStream_t s) {
+  auto fn = k_dslash<SPX, LPX, NR, DAG, EPI, MB>;
+  if (grid <= 0) grid = grid_for((const void*)fn, L.ntiles, 0, TILE, cps);
+  return launch_k(fn, dim3(grid + fin_ctas(L)), dim3(TILE), view_smem(L), s, L);
+}
+
 template <int NR, bool DAG, int EPI>
 cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
   if (L.ntiles <= 0) return cudaSuccess;
@@ -63,29 +71,26 @@ cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
       return launch_k(fn3, dim3(grid + fin_ctas(L)), dim3(3 * TILE), 0, s, L);
     }
   }
-  if constexpr (SPX == P_F32) {
-    if (form == 3) {  // the FP32 Dslash at the second register budget
-      auto fh = k_dslash<SPX, LPX, NR, DAG, EPI, DSLASH_MIN_BLOCKS_HI>;
-      if (grid <= 0) grid = grid_for((const void*)fh, L.ntiles, 0, TILE, cps);
-      return launch_k(fh, dim3(grid + fin_ctas(L)), dim3(TILE), view_smem(L), s, L);
-    }
-  }
+  if constexpr (SPX == P_F32)
+    if (form == 3) return go_site<NR, DAG, EPI, DSLASH_MIN_BLOCKS_HI>(L, grid, cps, s);  // the second register budget
   // up to one wave at 8 CTAs per SM the plain FP16-12 operator gains by the larger register
   // budget too (16^3x32 7.4 -> 6.5 us), beyond it loses (32^3x64 M-hat 149.5 -> 151.3)
-  if constexpr (ScalarF16<SPX, NR, EPI>::value) {
-    if (L.ntiles <= LQCD_DSLASH_MIN_BLOCKS_F16 * device_sm_count()) {
-      auto fs = k_dslash<SPX, LPX, NR, DAG, EPI, LQCD_DSLASH_MIN_BLOCKS_F16>;
-      if (grid <= 0) grid = grid_for((const void*)fs, L.ntiles, 0, TILE, cps);
-      return launch_k(fs, dim3(grid + fin_ctas(L)), dim3(TILE), view_smem(L), s, L);
-    }
+  if constexpr (ScalarF16<SPX, NR, EPI>::value)
+    if (L.ntiles <= LQCD_DSLASH_MIN_BLOCKS_F16 * device_sm_count())
+      return go_site<NR, DAG, EPI, LQCD_DSLASH_MIN_BLOCKS_F16>(L, grid, cps, s);
+  // BF16-18 operators at 10 CTAs per SM where two launches that follow one another fit the SMs so and
+  // not at 8, and from one wave at 8 until its second is well filled, us a M-hat at 8 / 10: 14^3x32
+  // (686 tiles) 12.9 / 12.0, 18^3x30 (1367) 15.9 / 16.5, 16^3x46 (1472) 16.6 / 16.2, 16^3x48 (1536)
+  // 18.8 / 17.4 and twisted 19.7 / 17.5, 18^3x38 (1732) 19.2 / 20.5
+  if constexpr (SPX == P_BF16 && NR == 18 && (EPI == EPI_PLAIN || EPI == EPI_PLAIN_TW)) {
+    constexpr int LO = LQCD_DSLASH_MIN_BLOCKS_F16, HI = LQCD_DSLASH_MIN_BLOCKS_HALF;
+    const int sms = device_sm_count();
+    const bool two_fit = L.ntiles > LO / 2 * sms && L.ntiles <= HI / 2 * sms;
+    if (!L.gated && (two_fit || (L.ntiles > LO * sms && L.ntiles <= (HI + 1) * sms)))
+      return go_site<NR, DAG, EPI, HI>(L, grid, cps, s);
   }
-  if constexpr (!split_only) {
-    auto fn = k_dslash<SPX, LPX, NR, DAG, EPI>;
-    if (grid <= 0) grid = grid_for((const void*)fn, L.ntiles, 0, TILE, cps);
-    return launch_k(fn, dim3(grid + fin_ctas(L)), dim3(TILE), view_smem(L), s, L);
-  } else {
-    return cudaErrorInvalidValue;
-  }
+  if constexpr (!split_only) return go_site<NR, DAG, EPI, DslashMinBlocks<SPX, NR, EPI>::value>(L, grid, cps, s);
+  return cudaErrorInvalidValue;
 }
 
 template <int NR>
