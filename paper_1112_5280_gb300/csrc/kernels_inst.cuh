@@ -73,21 +73,22 @@ cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
   }
   if constexpr (SPX == P_F32)
     if (form == 3) return go_site<NR, DAG, EPI, DSLASH_MIN_BLOCKS_HI>(L, grid, cps, s);  // the second register budget
-  // up to one wave at 8 CTAs per SM the plain FP16-12 operator gains by the larger register
-  // budget too (16^3x32 7.4 -> 6.5 us), beyond it loses (32^3x64 M-hat 149.5 -> 151.3)
-  if constexpr (ScalarF16<SPX, NR, EPI>::value)
-    if (L.ntiles <= LQCD_DSLASH_MIN_BLOCKS_F16 * device_sm_count())
-      return go_site<NR, DAG, EPI, LQCD_DSLASH_MIN_BLOCKS_F16>(L, grid, cps, s);
-  // BF16-18 operators at 10 CTAs per SM where two launches that follow one another fit the SMs so and
-  // not at 8, and from one wave at 8 until its second is well filled, us a M-hat at 8 / 10: 14^3x32
-  // (686 tiles) 12.9 / 12.0, 18^3x30 (1367) 15.9 / 16.5, 16^3x46 (1472) 16.6 / 16.2, 16^3x48 (1536)
-  // 18.8 / 17.4 and twisted 19.7 / 17.5, 18^3x38 (1732) 19.2 / 20.5
-  if constexpr (SPX == P_BF16 && NR == 18 && (EPI == EPI_PLAIN || EPI == EPI_PLAIN_TW)) {
+  // Half-precision operators that come in both budgets, us a M-hat at 8 CTAs per SM / at 10. Up to
+  // one wave at 8 the plain FP16-12 operator gains by the larger register budget too (16^3x32
+  // 13.1 / 15.1), beyond it loses (32^3x64 151.3 / 149.5). Where two launches that follow one another
+  // fit the SMs at 10 and not at 8, 10 is faster: 14^3x32 (686 tiles) FP16-12 13.1 / 11.2, FP16-18
+  // 13.1 / 11.3, BF16-18 12.9 / 12.0 (601 tiles, FP16-12: 9.0 / 9.3, 768: 13.1 / 15.0). BF16-18 also
+  // takes 10 from one wave at 8 until its second is well filled: 18^3x30 (1367) 15.9 / 16.5, 16^3x46
+  // (1472) 16.6 / 16.2, 16^3x48 (1536) 18.8 / 17.4 and twisted 19.7 / 17.5, 18^3x38 (1732) 19.2 / 20.5.
+  // The solvers' launches, other kernels between them, stay at 8 there.
+  if constexpr ((SPX == P_F16 && EPI == EPI_PLAIN) || (SPX == P_BF16 && NR == 18 && (EPI == EPI_PLAIN || EPI == EPI_PLAIN_TW))) {
     constexpr int LO = LQCD_DSLASH_MIN_BLOCKS_F16, HI = LQCD_DSLASH_MIN_BLOCKS_HALF;
     const int sms = device_sm_count();
     const bool two_fit = L.ntiles > LO / 2 * sms && L.ntiles <= HI / 2 * sms;
-    if (!L.gated && (two_fit || (L.ntiles > LO * sms && L.ntiles <= (HI + 1) * sms)))
-      return go_site<NR, DAG, EPI, HI>(L, grid, cps, s);
+    bool ten = two_fit && !L.gated;
+    if (SPX == P_BF16) ten = ten || (!L.gated && L.ntiles > LO * sms && L.ntiles <= (HI + 1) * sms);
+    if (NR == 12) ten = ten || L.ntiles > LO * sms;
+    return ten ? go_site<NR, DAG, EPI, HI>(L, grid, cps, s) : go_site<NR, DAG, EPI, LO>(L, grid, cps, s);
   }
   if constexpr (!split_only) return go_site<NR, DAG, EPI, DslashMinBlocks<SPX, NR, EPI>::value>(L, grid, cps, s);
   return cudaErrorInvalidValue;
