@@ -90,6 +90,13 @@ cudaError_t go_dslash(const Launch& L, int grid, cudaStream_t s, int form) {
     if (NR == 12) ten = ten || L.ntiles > LO * sms;
     return ten ? go_site<NR, DAG, EPI, HI>(L, grid, cps, s) : go_site<NR, DAG, EPI, LO>(L, grid, cps, s);
   }
+  // the twisted FP64 operator at 8 CTAs per SM where that is one wave and 6 are two (16^3x32, 12
+  // reals, 345 -> 318 us a M-hat, 18 reals 286 -> 269; at 768 tiles, one wave either way, 239 -> 315)
+  if constexpr (SPX == P_F64 && EPI == EPI_PLAIN_TW) {
+    const int sms = device_sm_count();
+    if (L.ntiles > LQCD_DSLASH_MIN_BLOCKS * sms && L.ntiles <= DSLASH_MIN_BLOCKS_HI * sms)
+      return go_site<NR, DAG, EPI, DSLASH_MIN_BLOCKS_HI>(L, grid, cps, s);
+  }
   if constexpr (!split_only) return go_site<NR, DAG, EPI, DslashMinBlocks<SPX, NR, EPI>::value>(L, grid, cps, s);
   return cudaErrorInvalidValue;
 }
