@@ -18,6 +18,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <set>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -328,6 +329,11 @@ int lqcd_autotune_dslash(int n, const lqcd_gauge* const* g, int prec, int compre
   L.nslots = n;
   L.ntiles = ntiles;
   L.interleave = (same_vh && n > 1) ? 1 : 0;
+  // the kernel that launches over these gauge fields run (a single-slot launch finds out itself)
+  std::set<const lqcd_gauge*> gauges(g, g + n);
+  size_t link_bytes = 0;
+  for (const lqcd_gauge* q : gauges) link_bytes += gauge_copy_bytes(link_prec_for(prec), nr, q->g.Vh);
+  L.stream_links = stream_links(prec, n, (int)gauges.size(), link_bytes);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (err == cudaSuccess) err = cudaEventCreate(&e0);
   if (err == cudaSuccess) err = cudaEventCreate(&e1);
@@ -409,6 +415,7 @@ int lqcd_autotune_dslash(int n, const lqcd_gauge* const* g, int prec, int compre
       groups_tried.push_back(gsize);
       Launch LS = L;
       LS.interleave = 2;
+      LS.stream_links = 0;
       LS.mrhs_group = gsize;
       LS.mrhs_groups = (n + gsize - 1) / gsize;
       LS.ntiles = blocks * LS.mrhs_groups;
