@@ -42,7 +42,7 @@ enum Fin {
   FIN_NONE = 0,
   FIN_STORE0,    // res[0] = sum
   FIN_STORE1,    // res[1] = sum
-  FIN_ALPHA,     // CG: qq = |Mhat p|^2, alpha = rr / qq
+  FIN_ALPHA,     // CG: qq = |Mhat p|^2, alpha = rr / qq; run by the next launch (finish_before)
   FIN_BETA,      // CG: rr_new, beta, reliable-update / stop / maxiter decisions
   FIN_TRUERES,   // reliable update: |bhat - Mhat x|^2 -> converged?
   FIN_RHO,       // reliable update: |Mhat^dag u|^2 -> new sloppy scale and p coefficient
@@ -200,8 +200,8 @@ struct SlotView {
 };
 
 // Dynamic shared memory of a one-thread-per-site Dslash launch: the slot view for gated
-// launches, nothing otherwise (operator launches then keep the L1 carve-out of a kernel
-// without shared memory).
+// launches, nothing otherwise. (The epilogues that do not reduce hold 64 bytes of static shared
+// memory for finish_before; compiled without it the operators measured the same.)
 inline size_t view_smem(const Launch& L) {
   return (L.gated && L.nslots > 1 && L.nslots <= VIEW_SLOTS) ? sizeof(SlotView) : 0;
 }
@@ -307,9 +307,6 @@ __device__ __noinline__ static void run_fin(const Work& w, const double* v) {
       break;
     case FIN_STORE1:
       s->res[1] = sum;
-      break;
-    case FIN_ALPHA:
-      fin_alpha(w, sum);
       break;
     case FIN_BETA: {  // new |r|^2: beta, and whether to leave for a reliable update
       if (s->bad) {

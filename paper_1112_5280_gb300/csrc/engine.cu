@@ -532,10 +532,10 @@ int rebuild(lqcd_engine* e) {
   }
   e->ntiles_total = prefix[n];
   if (e->opts.ru_interval <= 0) {
-    // A slot waiting for a reliable update idles until the next update block, and a
-    // block costs six launches that skip when no slot needs them; measured on GB300
-    // (8^4 to 32^3x64, FP16/FP32 sloppy) the solve time is flat in the interval
-    // between 1 and 8 to within 3%, slightly lower at 4.
+    // A slot waiting for a reliable update idles until the next update block, and a block that
+    // no slot needs costs a graph's condition or, issued directly, ten launches that skip.
+    // Measured on GB300 when every block was ten launches (8^4 to 32^3x64, FP16/FP32 sloppy): the
+    // solve time is flat in the interval between 1 and 8 to within 3%, slightly lower at 4.
     e->ru_every = std::min(e->opts.chunk, 4);
   }
   cudaStream_t st = e->ctx->stream;

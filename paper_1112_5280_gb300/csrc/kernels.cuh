@@ -213,7 +213,7 @@ __device__ __forceinline__ void dslash_tile(const Launch& L, int slot, int start
 
 // The tile loop is written twice: over the running slots' tiles of a gated launch (slot
 // view), and over all tiles otherwise, so that operator launches run the plain loop without
-// the view's branches and without shared memory (measured: one loop with a static view cost
+// the view's branches and its shared memory (measured: one loop with a static view cost
 // 1.3% more instructions and 2-3% of the headline launch).
 template <int SP, int LP, int NR, bool DAG, int EPI, int MB = DslashMinBlocks<SP, NR, EPI>::value>
 __global__ void __launch_bounds__(TILE, MB) k_dslash(const Launch L) {
