@@ -20,6 +20,7 @@
 // phi). So a sweep's result depends on (seed, sweep) and the links only, not on the
 // launch shape. At most 1000 attempts per draw: a subgroup that never accepts is left
 // unchanged and counted (the count is returned).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -137,18 +138,20 @@ __device__ __noinline__ bool su2_draw(double alpha, uint64_t seed, uint64_t c0, 
 // double-float from the copy Ud on the FP32 pipes; the draw of b (Creutz) and |c| in FP64.
 // The updated link goes to Ud only: the caller rebuilds the FP64 master from it.
 //
-// k_heatbath_v: V = U W of every link of the class, three threads per link (row-split
-// products in gauge_field.cuh), FP32 bound like the gauge force. V [word][V/2] stays in L2.
+// k_heatbath_v: V = U W of the class's links h0 .. h0 + n - 1 (all of them, but where memory is
+// short: lqcd_heatbath), three threads per link (row-split products in gauge_field.cuh), FP32 bound
+// like the gauge force. V [word][n] stays in L2.
 // k_heatbath: the three subgroups, one thread per link, FP64 bound (about 200 FP64
 // instructions per draw). At 24^3x48, beta 6, a sweep takes 5.74 ms; as one kernel with one
 // thread per link (168 registers, staple code and draws sharing 12 warps per SM) 6.63 ms, and
 // as one kernel with three threads per link, where two thirds of the CTA wait at a barrier
 // during the draws, 6.27 ms.
-__global__ void __launch_bounds__(SPLIT_THREADS, 4) k_heatbath_v(const float4* Ud, Geom g, int mu, int par, float4* V) {
+__global__ void __launch_bounds__(SPLIT_THREADS, 4) k_heatbath_v(const float4* Ud, Geom g, int mu, int par, int h0,
+                                                                 int n, float4* V) {
   __shared__ SplitM sw;
   const int j = threadIdx.x % SPLIT_LINKS, i = threadIdx.x / SPLIT_LINKS;
   // threads past the last link repeat it (they share barriers and rows) and store nothing
-  const int at = blockIdx.x * SPLIT_LINKS + j, h = min(at, g.Vh - 1);
+  const int at = blockIdx.x * SPLIT_LINKS + j, h = h0 + min(at, n - 1);
   const Site x = site_of(g, par, h);
   const size_t base = link_base(g, x, mu), vh = (size_t)g.Vh;
   const RowD W = staple_row(Ud, g, x, mu, i);
@@ -156,31 +159,32 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4) k_heatbath_v(const float4* U
   for (int q = 0; q < 3; ++q) sw.put(i, q, j, W.e[q]);
   __syncthreads();
   const RowD r = split_row_times(Ud + base, vh, i, sw, j);
-  if (at >= g.Vh) return;
+  if (at >= n) return;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     const C2d e = c_unpack(r.e[q]);
-    V[(size_t)(3 * i + q) * vh + h] = make_float4(e.re.hi, e.re.lo, e.im.hi, e.im.lo);
+    V[(size_t)(3 * i + q) * n + at] = make_float4(e.re.hi, e.re.lo, e.im.hi, e.im.lo);
   }
 }
 
 constexpr int HB_THREADS = 128;
+constexpr int HB_MIN_PIECE = 1024;  // links whose V is in memory at a time, at least
 // 4 CTAs per SM (128 registers, a 108-byte spill): 3 and 5 measured the same.
 #ifndef LQCD_HB_MIN_BLOCKS
 #define LQCD_HB_MIN_BLOCKS 4
 #endif
 __global__ void __launch_bounds__(HB_THREADS, LQCD_HB_MIN_BLOCKS) k_heatbath(float4* Ud, const float4* Vd, Geom g, int mu,
-                                                                             int par, double beta, uint64_t seed,
+                                                                             int par, int h0, int n, double beta, uint64_t seed,
                                                                              uint64_t sweep,
                                                                              unsigned long long* fails) {
-  const int h = blockIdx.x * blockDim.x + threadIdx.x;
-  if (h >= g.Vh) return;
-  const Site x = site_of(g, par, h);
+  const int at = blockIdx.x * blockDim.x + threadIdx.x;
+  if (at >= n) return;
+  const Site x = site_of(g, par, h0 + at);
   M3d u = load_link_df(Ud, g, x, mu);
   M3d V;
 #pragma unroll
   for (int w = 0; w < 9; ++w) {
-    const float4 d = Vd[(size_t)w * g.Vh + h];
+    const float4 d = Vd[(size_t)w * n + at];
     V.e[w] = {df64(d.x, d.y), df64(d.z, d.w)};
   }
   const uint64_t s = (uint64_t)x.c[0] + (uint64_t)g.L[0] * ((uint64_t)x.c[1] + (uint64_t)g.L[1] *
@@ -384,18 +388,27 @@ int lqcd_heatbath(lqcd_gauge* g, double beta, int nsweeps, unsigned long long se
   LQCD_TRY(gauge_links(g, P_DF64, &dfbase, &dfnr));
   float4* Ud = static_cast<float4*>(const_cast<void*>(dfbase));
   LQCD_CK(gauge_convert(U, g->g, P_DF64, 18, Ud, st));
-  const unsigned vgrid = (unsigned)((g->g.Vh + SPLIT_LINKS - 1) / SPLIT_LINKS);
-  const unsigned grid = (unsigned)((g->g.Vh + HB_THREADS - 1) / HB_THREADS);
-  LQCD_TRY(ctx_staging(c, (size_t)9 * g->g.Vh * sizeof(float4)));
+  // V of a whole class, or of as many of its links at a time as there is memory for: no link's
+  // staples hold another of its class, so a class may be updated in pieces
+  int piece = g->g.Vh, rc;
+  while ((rc = ctx_staging(c, (size_t)9 * piece * sizeof(float4))) != LQCD_OK) {
+    if (cudaGetLastError() != cudaErrorMemoryAllocation || piece <= HB_MIN_PIECE) return rc;
+    piece = (piece + 1) / 2;
+    clear_error();
+  }
   float4* V = reinterpret_cast<float4*>(c->staging);
   const unsigned rgrid = (unsigned)((8LL * g->g.Vh + 255) / 256);
   for (int sw = 0; sw < nsweeps; ++sw) {
     const uint64_t sweep = (uint64_t)(sweep0 + (unsigned long long)sw);
     for (int mu = 0; mu < 4; ++mu)
       for (int par = 0; par < 2; ++par) {
-        k_heatbath_v<<<vgrid, SPLIT_THREADS, 0, st>>>(Ud, g->g, mu, par, V);
-        k_heatbath<<<grid, HB_THREADS, 0, st>>>(Ud, V, g->g, mu, par, beta, seed, sweep, d_fails);
-        c->launches += 2;
+        for (int h0 = 0; h0 < g->g.Vh; h0 += piece) {
+          const int n = std::min(piece, g->g.Vh - h0);
+          const unsigned vgrid = (unsigned)((n + SPLIT_LINKS - 1) / SPLIT_LINKS), grid = (unsigned)((n + HB_THREADS - 1) / HB_THREADS);
+          k_heatbath_v<<<vgrid, SPLIT_THREADS, 0, st>>>(Ud, g->g, mu, par, h0, n, V);
+          k_heatbath<<<grid, HB_THREADS, 0, st>>>(Ud, V, g->g, mu, par, h0, n, beta, seed, sweep, d_fails);
+          c->launches += 2;
+        }
       }
     if (reunit) {
       k_reunitarise<<<rgrid, 256, 0, st>>>(Ud, g->g);
