@@ -109,7 +109,7 @@ static bool capturing(const lqcd_ctx* c) {
 
 int ctx_enter(lqcd_ctx* c) {
   LQCD_CK(cudaSetDevice(c->device));
-  if (!c->used_elsewhere && capturing(c)) c->used_elsewhere = true;
+  if (c->stream_known && !c->used_elsewhere && capturing(c)) c->used_elsewhere = true;
   return LQCD_OK;
 }
 
@@ -260,6 +260,7 @@ int lqcd_ctx_create(lqcd_ctx** out, int device, void* stream) {
   }
   if (rc == LQCD_OK) {
     c->stream = stream ? (cudaStream_t)stream : c->own_stream;
+    c->stream_known = stream != nullptr;
     cudaError_t e = ctx_malloc(c, (void**)&c->scratch_sc, 16 * sizeof(Scalars));
     if (e == cudaSuccess) e = cudaMemset(c->scratch_sc, 0, 16 * sizeof(Scalars));
     if (e == cudaSuccess) e = cudaMallocHost(&c->host_sc, 16 * sizeof(Scalars));
@@ -318,10 +319,15 @@ int lqcd_ctx_set_stream(lqcd_ctx* c, void* stream) {
   LQCD_TRY(ctx_enter(c));
   LQCD_CK(cudaStreamSynchronize(c->stream));
   c->stream = stream ? (cudaStream_t)stream : c->own_stream;
+  if (stream) c->stream_known = true;
   return LQCD_OK;
 }
 
-void* lqcd_ctx_stream(const lqcd_ctx* c) { return c ? (void*)c->stream : nullptr; }
+void* lqcd_ctx_stream(const lqcd_ctx* c) {
+  if (!c) return nullptr;
+  c->stream_known = true;
+  return (void*)c->stream;
+}
 
 int lqcd_ctx_sync(lqcd_ctx* c) {
   clear_error();

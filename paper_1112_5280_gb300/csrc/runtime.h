@@ -33,6 +33,8 @@ struct lqcd_ctx {
   // size (ctx_alloc)
   // work on the context's objects may run outside its stream (ctx_enter, lqcd_field_copy)
   std::atomic<bool> used_elsewhere{false};
+  // the caller has the stream's handle (its own stream, or lqcd_ctx_stream) and may capture it
+  mutable std::atomic<bool> stream_known{false};
   std::mutex pool_mu;
   std::deque<std::pair<size_t, void*>> pool;
   size_t pool_bytes = 0;
@@ -108,7 +110,8 @@ int make_geom(const int dims[4], int t_bc, Geom& g);
 size_t half_spinor_bytes(int prec, int Vh);
 size_t gauge_copy_bytes(int prec, int nr, int Vh);
 
-// Makes the context's device current at the start of a call, and notes a call that is captured.
+// Makes the context's device current at the start of a call, and notes a call that is captured (which
+// only a caller with the stream's handle can do: the question costs 0.1 us of a 2.6 us upload).
 int ctx_enter(lqcd_ctx* c);
 
 // device buffers of the context, grown on demand (synchronises when growing)
