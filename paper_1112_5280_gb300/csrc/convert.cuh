@@ -65,7 +65,7 @@ __host__ __device__ inline int round_to_int(float x) {  // nearest, ties to even
 // their branch. Written as expressions the compiler ran them for every value beside the integer
 // path and chose afterwards, and the FP64 pipe was paid as before. Per call, so and now: an
 // upload at 16^3x32 in double-float 32.0 -> 8.8 us, in FP32 14.6 -> 7.5, a copy there from FP64 to
-// FP32 26.3 -> 13.0, at 32^3x64 247 -> 107.
+// FP32 26.3 -> 13.0, at 32^3x64 247 -> 107. Zeros are no call either: a point source is zeros.
 __host__ __device__ __noinline__ inline float to_float_any(double x) { return (float)x; }
 __host__ __device__ __noinline__ inline double to_double_any(float x) { return (double)x; }
 __host__ __device__ __noinline__ inline float2 to_df_any(double x) {
@@ -82,6 +82,7 @@ __host__ __device__ __noinline__ inline unsigned to_bf16_any(double x) {
 __host__ __device__ inline unsigned float_bits(unsigned hi, unsigned lo) {
   return (((hi & 0x7fffffffu) << 3) | (lo >> 29)) - (896u << 23);
 }
+__host__ __device__ inline bool zero_bits(unsigned hi, unsigned lo) { return !((hi & 0x7fffffffu) | lo); }
 // 1 where those round up (nearest, ties to even)
 __host__ __device__ inline unsigned rounds_up(unsigned f, unsigned rem) {
   return (rem + 0x0fffffffu + (f & 1u)) >> 29;
@@ -91,7 +92,7 @@ __host__ __device__ inline unsigned rounds_up(unsigned f, unsigned rem) {
 __host__ __device__ inline float to_float(double x) {
   const unsigned long long b = bits_of(x);
   const unsigned h = (unsigned)(b >> 32), l = (unsigned)b, e = (h >> 20) & 0x7ffu;
-  if (e - 897u > 252u) return to_float_any(x);
+  if (e - 897u > 252u) return zero_bits(h, l) ? float_of(h) : to_float_any(x);
   const unsigned f = float_bits(h, l);
   return float_of((h & 0x80000000u) | (f + rounds_up(f, l & 0x1fffffffu)));
 }
@@ -100,15 +101,21 @@ __host__ __device__ inline float to_float(double x) {
 __host__ __device__ inline unsigned to_half(double x) {
   const unsigned long long b = bits_of(x);
   const unsigned h = (unsigned)(b >> 32), e = (h >> 20) & 0x7ffu;
-  if (e - 1009u > 29u) return to_half_any(x);
+  if (e > 1038u) return to_half_any(x);
+  const unsigned sign = (h >> 16) & 0x8000u, sticky = (unsigned)b ? 1u : 0u;
+  if (e < 1009u) {  // below 2^-14: the multiple of 2^-24
+    const unsigned r = e < 995u ? 24u : 1019u - e, m = (h & 0xfffffu) | 0x100000u, q = m >> r;
+    const unsigned rem = ((m << 1) & ((2u << r) - 1u)) | sticky;
+    return sign | (q + ((rem + (1u << r) - 1u + (q & 1u)) >> (r + 1u)));
+  }
   const unsigned f = ((h & 0x7fffffffu) >> 10) - (1008u << 10);
-  const unsigned rem = ((h & 0x3ffu) << 1) | ((unsigned)b ? 1u : 0u);  // the lowest bit sticky
-  return ((h >> 16) & 0x8000u) | (f + ((rem + 0x3ffu + (f & 1u)) >> 11));
+  const unsigned rem = ((h & 0x3ffu) << 1) | sticky;
+  return sign | (f + ((rem + 0x3ffu + (f & 1u)) >> 11));
 }
 __host__ __device__ inline unsigned to_bf16(double x) {
   const unsigned long long b = bits_of(x);
   const unsigned h = (unsigned)(b >> 32), e = (h >> 20) & 0x7ffu;
-  if (e - 897u > 252u) return to_bf16_any(x);
+  if (e - 897u > 252u) return zero_bits(h, (unsigned)b) ? h >> 16 : to_bf16_any(x);
   const unsigned f = ((h & 0x7fffffffu) >> 13) - (896u << 7);
   const unsigned rem = ((h & 0x1fffu) << 1) | ((unsigned)b ? 1u : 0u);
   return ((h >> 16) & 0x8000u) | (f + ((rem + 0x1fffu + (f & 1u)) >> 14));
@@ -118,7 +125,7 @@ __host__ __device__ inline unsigned to_bf16(double x) {
 __host__ __device__ inline double to_double(float x) {
   const unsigned b = bits_of(x), u = b & 0x7fffffffu, e = u >> 23;
   const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
-  if (e - 1u >= 254u) return to_double_any(x);
+  if (e - 1u >= 254u) return u ? to_double_any(x) : double_of(sign);
   return double_of(sign | (((unsigned long long)u << 29) + (896ULL << 52)));
 }
 
@@ -127,7 +134,7 @@ __host__ __device__ inline void to_df(double x, float& hi, float& lo) {
   const unsigned long long b = bits_of(x);
   const unsigned h = (unsigned)(b >> 32), l = (unsigned)b, e = (h >> 20) & 0x7ffu;
   if (e - 949u > 200u) {
-    const float2 v = to_df_any(x);
+    const float2 v = zero_bits(h, l) ? make_float2(float_of(h), 0.0f) : to_df_any(x);
     hi = v.x;
     lo = v.y;
     return;
@@ -153,6 +160,8 @@ __host__ __device__ inline double from_df(float hi, float lo) {
       return double_of(((unsigned long long)(b & 0x80000000u) << 32) | (((unsigned long long)(e + 895u) << 52) + m));
     }
   }
+  const unsigned l = bits_of(lo);
+  if (!((b | l) & 0x7fffffffu)) return double_of((unsigned long long)(b & l & 0x80000000u) << 32);
   return (double)hi + (double)lo;
 }
 

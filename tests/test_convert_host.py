@@ -34,7 +34,7 @@ int main() {
     bad += !same(hi, (float)h) || !same(lo, (float)l);
     bad += !same(to_double(hi), (double)hi);
     bad += to_half(x) != __half_as_ushort(__double2half(x)) || to_bf16(x) != __bfloat16_as_ushort(__double2bfloat16(x));
-    for (float other : {lo, -lo, 0.5f * lo, 3.0f * lo}) bad += !same(from_df(hi, other), (double)hi + (double)other);
+    for (float other : {lo, -lo, 0.5f * lo, 3.0f * lo, 0.0f, -0.0f}) bad += !same(from_df(hi, other), (double)hi + (double)other);
   };
   const unsigned long long patterns[] = {0ull, 0x1fffffffull, 0x10000000ull, 0x10000001ull, 0x0fffffffull, 0x20000000ull,
                                          0x30000000ull, 0xfffffe0000000ull, 0xfffffffffffffull, 0xffffff0000000ull,
